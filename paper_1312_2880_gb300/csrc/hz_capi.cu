@@ -59,7 +59,7 @@ struct Plan {
   size_t total = 0;
   // offsets
   std::vector<size_t> off_kh, off_u, off_f, off_u2;
-  size_t off_kh64 = 0, off_vec = 0, vec_bytes = 0, off_ainv = 0, off_work = 0, off_state = 0, off_partials = 0,
+  size_t off_kh64 = 0, off_d = 0, off_vec = 0, vec_bytes = 0, off_ainv = 0, off_work = 0, off_state = 0, off_partials = 0,
          off_hist = 0, off_status = 0, off_sync = 0, sync_bytes = 0;
   int nvec = 11;
   int m_coarse = 0;
@@ -128,6 +128,8 @@ bool make_plan(int n, const hz_hierarchy_opts& o, Plan* P, std::string* err) {
   }
   size_t N = (size_t)(n + 1) * (n + 1);
   P->off_kh64 = off;
+  off = align256(off + N * 8);
+  P->off_d = off;
   off = align256(off + N * 8);
   P->vec_bytes = align256(N * 16 * B);  // one slot: B consecutive vectors
   P->rhat_bytes = P->vec_bytes;          // one shadow residual per instance (restarts renew it)
@@ -930,6 +932,8 @@ hz_status solve_end(hz_problem* P, double* history, int history_cap, hz_solve_in
                        P->stream));
   }
   CK(cudaStreamSynchronize(P->stream));
+  if (history && history_cap > 0)  // the device keeps squared norms
+    for (int q = 0; q < std::min(hl, history_cap); ++q) history[q] = std::sqrt(history[q] / P->kstate_host[0].bnorm2);
   hz_status worst = HZ_OK;
   for (int b = 0; b < B; ++b) {
     const KState& hs = P->kstate_host[b];
@@ -1355,6 +1359,8 @@ hz_status hz_setup_hierarchy(hz_problem* P, const hz_hierarchy_opts* opts, void*
     k.p32 = k.s32 = k.y32 = k.z32 = nullptr;
   }
   k.kh = P->kh64;
+  k.d = (double*)(A + pl.off_d);
+  CK(launch_k_diag((double*)(A + pl.off_d), P->kh64, Nn, s));
   k.n = n;
   k.N = (long long)(n + 1) * (n + 1);
   k.scale_b = 1.0 / ((double)n * n);
@@ -1522,7 +1528,7 @@ hz_status hz_apply(hz_problem* P, int op, const double* u, double* v) {
   if (!u || !v || (const double*)u == v || (op != HZ_OP_L && op != HZ_OP_M)) return fail(P, HZ_EINVAL, "bad apply arguments");
   StreamScope scope(P);
   double n2 = (double)P->n * P->n;
-  CK(launch_apply_fp64((double2*)v, (const double2*)u, P->kh64, P->n, op_beta(P, op), n2, P->stream));
+  CK(launch_apply_fp64((double2*)v, (const double2*)u, P->kh64, P->kv.d, P->n, op_beta(P, op), n2, P->stream));
   return HZ_OK;
 }
 
@@ -2126,17 +2132,17 @@ static hz_status cycle_run(hz_problem* P, hz_ray* R, const double2* b, double2* 
   int cycles = 0, hl = 0;
   while (st == HZ_EMAXIT && cycles < maxc) {
     ++cycles;
-    CK(launch_apply_fp64(v, x, P->kh64, P->n, 0.0, n2, s));
+    CK(launch_apply_fp64(v, x, P->kh64, P->kv.d, P->n, 0.0, n2, s));
     CK(launch_ray_residual_norm(r, b, v, N, partials, nrm, s));
     const hz_status vs = vcycle_dev(P, (const double*)r, (double*)z);
     if (vs != HZ_OK) return vs;
     CK(launch_ray_axpy(x, z, N, s));
     if (R) {
-      CK(launch_apply_fp64(v, x, P->kh64, P->n, 0.0, n2, s));
+      CK(launch_apply_fp64(v, x, P->kh64, P->kv.d, P->n, 0.0, n2, s));
       CK(launch_ray_residual_norm(r, b, v, N, partials, nrm, s));
       CK(ray_apply(R, x, r));
     }
-    CK(launch_apply_fp64(v, x, P->kh64, P->n, 0.0, n2, s));
+    CK(launch_apply_fp64(v, x, P->kh64, P->kv.d, P->n, 0.0, n2, s));
     CK(launch_ray_residual_norm(r, b, v, N, partials, nrm, s));
     double r2 = 0;
     CK(cudaMemcpyAsync(&r2, nrm, sizeof(double), cudaMemcpyDeviceToHost, s));

@@ -233,12 +233,13 @@ struct KrylovVecs {
   float2 *p32, *s32, *y32, *z32;
   const double2* b;
   const double* kh;  // k h on the finest grid, pitch n+1
+  const double* d;   // (k h)^2 - 4, the interior diagonal of L
   int n;
   long long N;
   double scale_b;  // h^2: the solver works on the h^2-scaled system
   KState* st;        // [batch]
   double* partials;  // [batch][part_stride]
-  double* hist;      // [batch][hist_stride]
+  double* hist;      // [batch][hist_stride] squared residual norms (the host divides and takes the root)
   int G;             // reduction grid size
   // Batches of right-hand sides: instance b (blockIdx.z) uses every vector (b, x, r, p, v, s, t,
   // y, z, tr and the FP32 copies) advanced by b * sv elements, its own state, partials and
@@ -264,9 +265,11 @@ cudaError_t launch_k_update_r(const KrylovVecs& k, cudaStream_t s);
 cudaError_t launch_k_update_x(const KrylovVecs& k, bool omega_half, cudaStream_t s);
 cudaError_t launch_k_true_residual(const KrylovVecs& k, cudaStream_t s);
 cudaError_t launch_k_restart(const KrylovVecs& k, cudaStream_t s);  // every instance of k (use instance_of for one)
+// d = (k h)^2 - 4 of N nodes.
+cudaError_t launch_k_diag(double* d, const double* kh, long long N, cudaStream_t s);
 // v = A u (scaled by out_scale) on the finest grid in FP64; beta = 0 for L, the shift for M.
-cudaError_t launch_apply_fp64(double2* v, const double2* u, const double* kh, int n, double beta, double out_scale,
-                              cudaStream_t s);
+cudaError_t launch_apply_fp64(double2* v, const double2* u, const double* kh, const double* d, int n, double beta,
+                              double out_scale, cudaStream_t s);
 
 // ---------------------------------------------------------------- ray correction (hz_ray.cu)
 

@@ -29,10 +29,12 @@ __device__ __forceinline__ double2 d2axpy(double2 a, double2 s, double2 b) {
 __device__ __forceinline__ double2 d2axmy(double2 a, double2 s, double2 b) {
   return make_double2(fma(-s.x, b.x, fma(s.y, b.y, a.x)), fma(-s.x, b.y, fma(-s.y, b.x, a.y)));
 }
-__device__ __forceinline__ double2 d2div(double2 a, double2 b) {
-  double inv = 1.0 / (b.x * b.x + b.y * b.y);
-  return make_double2((a.x * b.x + a.y * b.y) * inv, (a.y * b.x - a.x * b.y) * inv);
+__device__ __forceinline__ double d2norm(double2 a) { return a.x * a.x + a.y * a.y; }
+// a conj(b) c
+__device__ __forceinline__ double2 d2scale_conj(double2 a, double2 b, double c) {
+  return make_double2((a.x * b.x + a.y * b.y) * c, (a.y * b.x - a.x * b.y) * c);
 }
+__device__ __forceinline__ double2 d2div(double2 a, double2 b) { return d2scale_conj(a, b, 1.0 / d2norm(b)); }
 __device__ __forceinline__ double2 d2mul(double2 a, double2 b) {
   return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
@@ -50,51 +52,51 @@ __device__ __forceinline__ float2 narrow(double2 v) { return make_float2(f64_to_
 __device__ __forceinline__ bool fin(double v) { return isfinite(v); }
 __device__ __forceinline__ bool fin2(double2 v) { return isfinite(v.x) && isfinite(v.y); }
 
+// Sum over the block in a fixed order; the result is valid in every lane of warp k for value k. Every
+// thread stores its values, lane L of warp k adds column L of value k over the KB / 32 warps, then a
+// shuffle tree. GB300's FP64 pipe executes every lane of a warp instruction, so a shuffle tree in
+// each of the KB / 32 warps costs as much FP64 issue as the kernel's own arithmetic on small grids
+// (measured: the reduction of an update at n = 512 took 8.6 us of 31); summing through shared memory
+// first leaves one warp's adds per value, and one warp per value puts the values on different
+// sub-partitions (one warp for all three: k_update_r at n = 64 15.9 us, three warps: see grid_sum).
 template <int NV>
-__device__ __forceinline__ void warp_sum(double (&v)[NV]) {
-#pragma unroll
-  for (int k = 0; k < NV; ++k)
-#pragma unroll
-    for (int off = 16; off; off >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], off);
-}
-
-// Sum over the block in a fixed order; the result is valid in thread 0. Every thread stores its
-// values, lane L of warp 0 adds column L over the KB / 32 warps, then a shuffle tree. GB300's
-// FP64 pipe executes every lane of a warp instruction, so a shuffle tree in each of the KB / 32
-// warps costs as much FP64 issue as the kernel's own arithmetic on small grids (measured: the
-// reduction of an update at n = 512 took 8.6 us of 31); summing through shared memory first
-// leaves one warp's adds per block.
-template <int NV>
-__device__ __forceinline__ void block_sum(double (&v)[NV], double (*sm)[KB]) {
+__device__ __forceinline__ double block_sum(const double (&v)[NV], double (*sm)[KB]) {
+  static_assert(NV <= KB / 32, "one warp per value");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   __syncthreads();
 #pragma unroll
   for (int k = 0; k < NV; ++k) sm[k][threadIdx.x] = v[k];
   __syncthreads();
-  if (warp == 0) {
+  double s = 0.0;
+  if (warp < NV) {
+    s = sm[warp][lane];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double s = sm[k][lane];
+    for (int w = 1; w < KB / 32; ++w) s += sm[warp][w * 32 + lane];
 #pragma unroll
-      for (int w = 1; w < KB / 32; ++w) s += sm[k][w * 32 + lane];
-      v[k] = s;
-    }
-    warp_sum<NV>(v);
+    for (int off = 16; off; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
   }
+  return s;  // valid in lane 0 of warp k < NV
 }
 
-// Grid-wide sum. Every block stores its partial; the block that arrives last adds all partials
-// in block order and returns true with the totals in `tot` (in every thread of that block).
-template <int NV>
-__device__ bool grid_sum(double (&v)[NV], double* partials, unsigned int* ticket, double (&tot)[NV]) {
-  __shared__ double sm[NV][KB];
+// Grid-wide sum over G blocks of KB threads' sums. A launch of G / VB blocks carries VB of them each:
+// block b the sums of blocks b and b + gridDim.x (value k of the q-th one in v[q NV + k]; those past
+// G are zero), so the partials, and with them every bit of the result, do not depend on VB. Every
+// block stores its partials; the block that arrives last adds all partials in block order and
+// returns true with the totals in `tot` (in every thread of that block).
+template <int NV, int VB = 1>
+__device__ bool grid_sum(double (&v)[NV * VB], double* partials, int G, unsigned int* ticket, double (&tot)[NV]) {
+  __shared__ double sm[NV * VB][KB];
   __shared__ int is_last;
   __shared__ double res[NV];
-  block_sum<NV>(v, sm);
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) partials[k * gridDim.x + blockIdx.x] = v[k];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const double s = block_sum<NV * VB>(v, sm);
+  if (lane == 0 && warp < NV * VB) {
+    const int b = blockIdx.x + (warp / NV) * gridDim.x;
+    if (b < G) partials[(warp % NV) * G + b] = s;
     __threadfence();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
     unsigned int t = atomicAdd(ticket, 1u);
     is_last = (t == gridDim.x - 1);
   }
@@ -105,14 +107,11 @@ __device__ bool grid_sum(double (&v)[NV], double* partials, unsigned int* ticket
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
     w[k] = 0.0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += KB) w[k] += __ldcg(&partials[k * gridDim.x + b]);
+    for (int b = threadIdx.x; b < G; b += KB) w[k] += __ldcg(&partials[k * G + b]);
   }
-  block_sum<NV>(w, sm);
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) res[k] = w[k];
-    *ticket = 0;
-  }
+  const double r = block_sum<NV>(w, sm);
+  if (lane == 0 && warp < NV) res[warp] = r;
+  if (threadIdx.x == 0) *ticket = 0;
   __syncthreads();
 #pragma unroll
   for (int k = 0; k < NV; ++k) tot[k] = res[k];
@@ -120,8 +119,8 @@ __device__ bool grid_sum(double (&v)[NV], double* partials, unsigned int* ticket
 }
 
 // (h^2 A y) at node (i, j) = flat index e of the finest grid (pitch n+1), A = L (beta = 0) or M.
-// The FP64 pipe bounds these kernels, so interior nodes of L take the real-diagonal path:
-// d = (kh)^2 - 4 (one FMA) and v = nb + d y (two FMAs); boundary nodes and M use the complex row.
+// Interior nodes of L take the real-diagonal path v = nb + d y (two FMAs) with d = (kh)^2 - 4 stored
+// per node; boundary nodes and M use the complex row.
 // Boundary rows and the shifted operator M: the complex diagonal. Out of line, so that the
 // compiler never evaluates this branch's FP64 arithmetic for interior nodes (it is taken by 4n of
 // (n+1)^2 nodes; with the branch if-converted the apply kernels were measured 1.65x slower).
@@ -132,26 +131,145 @@ __device__ __noinline__ double2 apply_row(const Y2* __restrict__ y, double k, in
   return d2add(d2mul(d, ldy(y, e)), nb);
 }
 
-template <class Y2>
-__device__ __forceinline__ double2 apply_at(const Y2* __restrict__ y, const double* __restrict__ kh, int e, int i,
-                                            int j, int n, double beta) {
-  const int w = n + 1;
-  Nbr b = neighbours(i, j, n);
-  double2 nb = d2add(d2add(ldy(y, j * w + b.iw), ldy(y, j * w + b.ie)), d2add(ldy(y, b.js * w + i), ldy(y, b.jn * w + i)));
-  const double k = kh[e];
-  if (b.sides == 0 && beta == 0.0) {
-    const double2 ye = ldy(y, e);
-    const double dr = fma(k, k, -4.0);
-    return make_double2(fma(dr, ye.x, nb.x), fma(dr, ye.y, nb.y));
+// Packed FP32 pairs (two additions per instruction).
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack(float2 v) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(v.x), "f"(v.y));
+  return r;
+}
+__device__ __forceinline__ float2 unpack(f32x2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+// a - b as a + (-1) b: the product is exact, so one rounding as in a subtraction
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(b), "l"(0xbf800000bf800000ull), "l"(a));
+  return r;
+}
+// s + r = a + b exactly (Knuth's two-sum), both components.
+__device__ __forceinline__ void two_sum(f32x2 a, f32x2 b, f32x2& s, f32x2& r) {
+  s = add2(a, b);
+  const f32x2 z = sub2(s, a);
+  r = add2(sub2(a, sub2(s, z)), sub2(b, z));
+}
+
+// s + r in FP64, |r| <= ulp(s) / 2: r is added to the widened s on the integer pipe, aligned to s's
+// last FP64 place. `odd` is set where that would need rounding or care: a remainder reaching below
+// that place, a power of two losing its leading bit, a subnormal, an infinity or a NaN.
+__device__ __forceinline__ double join(float s, float r, unsigned& odd) {
+  const unsigned us = (unsigned)__float_as_int(s), ur = (unsigned)__float_as_int(r);
+  int hi = (((int)us >> 3) & 0x8fffffff) + 0x38000000;
+  unsigned lo = us << 29;
+  if (ur << 1) {
+    // r in units of s's last FP64 place: mantissa * 2^(sh), below 2^29
+    const int es = (int)(us >> 23) & 0xff, er = (int)(ur >> 23) & 0xff;
+    const int sh = er - es + 29;
+    const unsigned m = (ur << 8) | 0x80000000u;  // the mantissa, at the top of the word
+    const unsigned drop = (unsigned)min(max(8 - sh, 0), 31);
+    const unsigned q = m >> drop;  // m 2^(sh - 8)
+    const int sg = (int)(us ^ ur) >> 31;
+    odd |= (q << drop) ^ m;
+    if (er == 0 || es == 255 || er == 255 || sh < -23 || (sg && !(us & 0x7fffffu))) odd = 1;
+    const long long bits = (long long)((unsigned long long)(unsigned)hi << 32 | lo) + (((long long)q ^ sg) - sg);
+    hi = (int)(bits >> 32);
+    lo = (unsigned)bits;
+  } else if (((us + 0x00800000u) & 0x7f000000u) == 0) {  // zero, subnormal, infinity or NaN
+    odd |= us << 1;  // an exact zero stays
+    hi = (int)(us & 0x80000000u);
   }
-  return apply_row(y, k, e, b.sides, beta, nb);
+  return __hiloint2double(hi, (int)lo);
+}
+// Sum of four FP32 complex values in FP64 without the FP64 pipe, which bounds the operator kernels:
+// error-free additions on the FP32 pipe leave a leading part and a remainder, joined in integers
+// (six FP64 additions, 460 cycles of a sub-partition's pipe per node, and eight widenings become
+// about 100 ordinary instructions). The result is the exact sum, which is what adding in FP64 gives
+// unless one of its additions rounds; `odd` is set where the remainder has more than 24 bits or join
+// cannot place it, and the caller then adds in FP64.
+__device__ __forceinline__ double2 nb_sum(float2 a, float2 b, float2 c, float2 d, unsigned& odd) {
+  f32x2 s1, r1, s2, r2, s, r3, r, r4, r5;
+  two_sum(pack(a), pack(b), s1, r1);
+  two_sum(pack(c), pack(d), s2, r2);
+  two_sum(s1, s2, s, r3);
+  two_sum(r1, r2, r, r4);
+  two_sum(r, r3, r, r5);
+  two_sum(s, r, s, r);  // s1 + s2 may have cancelled: |r| <= ulp(s) / 2 again
+  const float2 sv = unpack(s), rv = unpack(r);
+  const f32x2 rest = (r4 | r5) << 1;
+  odd = ((unsigned)(rest >> 32) & ~1u) | (unsigned)rest;
+  double2 o;
+  o.x = join(sv.x, rv.x, odd);
+  o.y = join(sv.y, rv.y, odd);
+  return o;
+}
+// Neighbour sum (W + E) + (S + N) of FP64 values.
+__device__ __forceinline__ double2 nb_sum64(double2 w, double2 e, double2 s, double2 n) {
+  return d2add(d2add(w, e), d2add(s, n));
+}
+
+__device__ __forceinline__ double2 interior(double d, double2 y, double2 nb) {
+  return make_double2(fma(d, y.x, nb.x), fma(d, y.y, nb.y));
+}
+
+// The five values of y around node (i, j), out-of-domain neighbours mirrored, and the node's d; loading
+// and computing are apart so that a thread with several nodes in flight loads them all first.
+template <class Y2>
+struct Star {
+  Y2 c, w, e, s, n;
+  double d;
+  int sides;
+  __device__ __forceinline__ void load(const Y2* __restrict__ y, const double* __restrict__ dd, int q, int i, int j,
+                                       int nn) {
+    const int p = nn + 1;
+    const Y2* at = y + q;
+    c = at[0];
+    w = at[i > 0 ? -1 : 1];
+    e = at[i < nn ? 1 : -1];
+    s = at[j > 0 ? -p : p];
+    n = at[j < nn ? p : -p];
+    d = dd[q];
+    sides = (i == 0) + (i == nn) + (j == 0) + (j == nn);
+  }
+};
+__device__ __noinline__ double2 nb_sum_fp64(float2 w, float2 e, float2 s, float2 n) {
+  return nb_sum64(widen(w), widen(e), widen(s), widen(n));
+}
+__device__ __forceinline__ double2 nb_of(const Star<double2>& t) { return nb_sum64(t.w, t.e, t.s, t.n); }
+__device__ __forceinline__ double2 nb_of(const Star<float2>& t) {
+  unsigned odd;
+  double2 nb = nb_sum(t.w, t.e, t.s, t.n, odd);
+  if (odd) nb = nb_sum_fp64(t.w, t.e, t.s, t.n);
+  return nb;
+}
+template <class Y2>
+__device__ __forceinline__ double2 apply_star(const Star<Y2>& t, const Y2* __restrict__ y, const double* __restrict__ kh,
+                                              int q, double beta) {
+  const double2 nb = nb_of(t);
+  if (t.sides == 0 && beta == 0.0) return interior(t.d, widen(t.c), nb);
+  return apply_row(y, kh[q], q, t.sides, beta, nb);
+}
+template <class Y2>
+__device__ __forceinline__ double2 apply_at(const Y2* __restrict__ y, const double* __restrict__ kh,
+                                            const double* __restrict__ dd, int e, int i, int j, int n, double beta) {
+  Star<Y2> t;
+  t.load(y, dd, e, i, j, n);
+  return apply_star(t, y, kh, e, beta);
 }
 
 // Grid-stride walk over the (n+1)^2 nodes that keeps (i, j) up to date without dividing per node.
 struct NodeWalk {
-  int e, i, j, di, dj, w, stride;
-  __device__ __forceinline__ NodeWalk(int n, int stride_) : w(n + 1), stride(stride_) {
-    e = blockIdx.x * blockDim.x + threadIdx.x;
+  int e, i, j, di, dj, w, stride, block;
+  __device__ __forceinline__ NodeWalk() {}
+  __device__ __forceinline__ NodeWalk(int n, int stride_, int block_ = blockIdx.x)
+      : w(n + 1), stride(stride_), block(block_) {
+    e = block * KB + threadIdx.x;
     j = e / w;
     i = e - j * w;
     dj = stride / w;
@@ -166,6 +284,8 @@ struct NodeWalk {
       ++j;
     }
   }
+  // a node of a block below G: the blocks that a launch carries beyond G have none
+  __device__ __forceinline__ bool live(int N, int G) const { return e < N && block < G; }
 };
 
 __device__ __forceinline__ void hist_push(KState* st, double* hist, double v) {
@@ -227,7 +347,7 @@ __global__ void k_init_kernel(KrylovVecs k, double tol, int maxit, int hist_cap)
     acc[3] = fma(rh.x, rh.x, fma(rh.y, rh.y, acc[3]));
   }
   double tot[4];
-  if (!grid_sum<4>(acc, k.partials, &k.st->ticket[KT_INIT], tot)) return;
+  if (!grid_sum<4>(acc, k.partials, k.G, &k.st->ticket[KT_INIT], tot)) return;
   if (threadIdx.x == 0) {
     KState* st = k.st;
     st->bnorm2 = tot[0];
@@ -288,7 +408,7 @@ __global__ void k_update_p_kernel(KrylovVecs k) {
       acc[2] = fma(rh.x, rh.x, fma(rh.y, rh.y, acc[2]));
     }
     double tot[3];
-    if (!grid_sum<3>(acc, k.partials, &st->ticket[KT_SHADOW], tot)) return;
+    if (!grid_sum<3>(acc, k.partials, k.G, &st->ticket[KT_SHADOW], tot)) return;
     if (threadIdx.x == 0) {
       st->rho = make_double2(tot[0], tot[1]);
       st->rhat2 = tot[2];
@@ -322,25 +442,40 @@ __global__ void k_update_p_kernel(KrylovVecs k) {
 }
 
 // v = A y with <r^, v>; alpha = rho / <r^, v>.
-template <class Y2>
-__global__ void k_apply_rv_kernel(KrylovVecs k, const Y2* __restrict__ y) {
+template <class Y2, int VB>
+__global__ void __launch_bounds__(KB, 4) k_apply_rv_kernel(KrylovVecs k, const Y2* __restrict__ y) {
   pdl_enter();
   k = instance(k);
   y += blockIdx.z * k.sv;
   KState* st = k.st;
   if (st->done) return;
-  double acc[2] = {0.0, 0.0};
+  double acc[2 * VB] = {};
   const int N = (int)k.N;
-  for (NodeWalk it(k.n, gridDim.x * KB); it.e < N; it.next()) {
-    const int e = it.e;
-    double2 v = apply_at(y, k.kh, e, it.i, it.j, k.n, 0.0);
-    k.v[e] = v;
-    double2 rh = k.rhat[e];
-    acc[0] = fma(rh.x, v.x, fma(rh.y, v.y, acc[0]));
-    acc[1] = fma(rh.x, v.y, fma(-rh.y, v.x, acc[1]));
+  NodeWalk it[VB];
+#pragma unroll
+  for (int q = 0; q < VB; ++q) it[q] = NodeWalk(k.n, k.G * KB, blockIdx.x + q * gridDim.x);
+  while (it[0].e < N) {
+    Star<Y2> star[VB];
+    double2 rh[VB];
+#pragma unroll
+    for (int q = 0; q < VB; ++q)
+      if (it[q].live(N, k.G)) {
+        star[q].load(y, k.d, it[q].e, it[q].i, it[q].j, k.n);
+        rh[q] = k.rhat[it[q].e];
+      }
+#pragma unroll
+    for (int q = 0; q < VB; ++q) {
+      if (it[q].live(N, k.G)) {
+        const double2 v = apply_star(star[q], y, k.kh, it[q].e, 0.0);
+        k.v[it[q].e] = v;
+        acc[2 * q] = fma(rh[q].x, v.x, fma(rh[q].y, v.y, acc[2 * q]));
+        acc[2 * q + 1] = fma(rh[q].x, v.y, fma(-rh[q].y, v.x, acc[2 * q + 1]));
+      }
+      it[q].next();
+    }
   }
   double tot[2];
-  if (!grid_sum<2>(acc, k.partials, &st->ticket[KT_RV], tot)) return;
+  if (!grid_sum<2, VB>(acc, k.partials, k.G, &st->ticket[KT_RV], tot)) return;
   if (threadIdx.x == 0) {
     double2 rv = make_double2(tot[0], tot[1]);
     st->rv = rv;
@@ -373,10 +508,10 @@ __global__ void k_update_s_kernel(KrylovVecs k) {
     acc[0] = fma(s.x, s.x, fma(s.y, s.y, acc[0]));
   }
   double tot[1];
-  if (!grid_sum<1>(acc, k.partials, &st->ticket[KT_S], tot)) return;
+  if (!grid_sum<1>(acc, k.partials, k.G, &st->ticket[KT_S], tot)) return;
   if (threadIdx.x == 0) {
     st->ss = tot[0];
-    hist_push(st, k.hist, sqrt(tot[0] / st->bnorm2));
+    hist_push(st, k.hist, tot[0]);
     if (!fin(tot[0])) {
       st->done = 3;
     } else if (tot[0] <= st->tol2) {
@@ -388,26 +523,41 @@ __global__ void k_update_s_kernel(KrylovVecs k) {
 }
 
 // t = A z with <t, s> and <t, t>; omega = <t, s> / <t, t>.
-template <class Y2>
-__global__ void k_apply_ts_kernel(KrylovVecs k, const Y2* __restrict__ z) {
+template <class Y2, int VB>
+__global__ void __launch_bounds__(KB, 4) k_apply_ts_kernel(KrylovVecs k, const Y2* __restrict__ z) {
   pdl_enter();
   k = instance(k);
   z += blockIdx.z * k.sv;
   KState* st = k.st;
   if (st->done) return;
-  double acc[3] = {0.0, 0.0, 0.0};
+  double acc[3 * VB] = {};
   const int N = (int)k.N;
-  for (NodeWalk it(k.n, gridDim.x * KB); it.e < N; it.next()) {
-    const int e = it.e;
-    double2 t = apply_at(z, k.kh, e, it.i, it.j, k.n, 0.0);
-    k.t[e] = t;
-    double2 s = k.s[e];
-    acc[0] = fma(t.x, s.x, fma(t.y, s.y, acc[0]));
-    acc[1] = fma(t.x, s.y, fma(-t.y, s.x, acc[1]));
-    acc[2] = fma(t.x, t.x, fma(t.y, t.y, acc[2]));
+  NodeWalk it[VB];
+#pragma unroll
+  for (int q = 0; q < VB; ++q) it[q] = NodeWalk(k.n, k.G * KB, blockIdx.x + q * gridDim.x);
+  while (it[0].e < N) {
+    Star<Y2> star[VB];
+    double2 s[VB];
+#pragma unroll
+    for (int q = 0; q < VB; ++q)
+      if (it[q].live(N, k.G)) {
+        star[q].load(z, k.d, it[q].e, it[q].i, it[q].j, k.n);
+        s[q] = k.s[it[q].e];
+      }
+#pragma unroll
+    for (int q = 0; q < VB; ++q) {
+      if (it[q].live(N, k.G)) {
+        const double2 t = apply_star(star[q], z, k.kh, it[q].e, 0.0);
+        k.t[it[q].e] = t;
+        acc[3 * q] = fma(t.x, s[q].x, fma(t.y, s[q].y, acc[3 * q]));
+        acc[3 * q + 1] = fma(t.x, s[q].y, fma(-t.y, s[q].x, acc[3 * q + 1]));
+        acc[3 * q + 2] = fma(t.x, t.x, fma(t.y, t.y, acc[3 * q + 2]));
+      }
+      it[q].next();
+    }
   }
   double tot[3];
-  if (!grid_sum<3>(acc, k.partials, &st->ticket[KT_TS], tot)) return;
+  if (!grid_sum<3, VB>(acc, k.partials, k.G, &st->ticket[KT_TS], tot)) return;
   if (threadIdx.x == 0) {
     st->ts = make_double2(tot[0], tot[1]);
     st->tt = tot[2];
@@ -441,13 +591,23 @@ __global__ void k_update_r_kernel(KrylovVecs k) {
     acc[2] = fma(r.x, r.x, fma(r.y, r.y, acc[2]));
   }
   double tot[3];
-  if (!grid_sum<3>(acc, k.partials, &st->ticket[KT_XR], tot)) return;
-  if (threadIdx.x == 0) {
+  if (!grid_sum<3>(acc, k.partials, k.G, &st->ticket[KT_XR], tot)) return;
+  if (threadIdx.x >= 32) return;
+  // The divisions of the next beta and of the two stall ratios, one per lane: lane 0 rho_new / rho_old,
+  // lane 1 alpha / omega, lane 2 cos^2, lane 3 the squared step.
+  const int lane = threadIdx.x;
+  const double2 rho_new = make_double2(tot[0], tot[1]), rho_old = st->rho;
+  const double2 num = lane == 0 ? rho_new : alpha, den = lane == 0 ? rho_old : omega;
+  const double ratio = (lane < 2 ? 1.0 : lane == 2 ? d2norm(rho_new) : d2norm(omega) * st->tt) /
+                       (lane < 2 ? d2norm(den) : lane == 2 ? st->rhat2 * tot[2] : tot[2]);
+  const double2 quot = d2scale_conj(num, den, ratio);
+  const double cos2 = __shfl_sync(0xffffffffu, ratio, 2), step2 = __shfl_sync(0xffffffffu, ratio, 3);
+  const double2 q1 = make_double2(__shfl_sync(0xffffffffu, quot.x, 1), __shfl_sync(0xffffffffu, quot.y, 1));
+  if (lane == 0) {
     st->omega_x = omega;  // x += omega z is due (k_update_x, beside the next preconditioner application)
     st->xw = 1;
     st->rr = tot[2];
-    hist_push(st, k.hist, sqrt(tot[2] / st->bnorm2));
-    double2 rho_new = make_double2(tot[0], tot[1]);
+    hist_push(st, k.hist, tot[2]);
     if (!fin(tot[0]) || !fin(tot[1]) || !fin(tot[2])) {
       st->done = 3;
     } else if (omega.x == 0.0 && omega.y == 0.0) {
@@ -461,9 +621,7 @@ __global__ void k_update_r_kernel(KrylovVecs k) {
       st->iters_x2 = 2 * st->it;
     }
     if (!st->done) {  // here |r|^2 > tol2 > 0
-      const double cos2 = (rho_new.x * rho_new.x + rho_new.y * rho_new.y) / (st->rhat2 * tot[2]);
       st->min_cos2 = fmin(st->min_cos2, cos2);
-      const double step2 = (omega.x * omega.x + omega.y * omega.y) * st->tt / tot[2];
       if (cos2 < st->stall_cos2) st->min_step2 = fmin(st->min_step2, step2);
       if (cos2 < st->stall_cos2 && step2 < st->stall_step2 && st->shadow_restarts < st->max_shadow_restarts) {
         // <r^, r> has collapsed relative to |r^| |r| and the iteration no longer moves r: the
@@ -474,9 +632,9 @@ __global__ void k_update_r_kernel(KrylovVecs k) {
       }
     }
     if (!st->done) {
-      st->rho_old = st->rho;
+      st->rho_old = rho_old;
       st->rho = rho_new;
-      st->beta = d2mul(d2div(rho_new, st->rho_old), d2div(alpha, omega));
+      st->beta = d2mul(quot, q1);
       st->first = 0;
       st->it += 1;
     }
@@ -552,14 +710,14 @@ __global__ void k_true_residual_kernel(KrylovVecs k) {
   const int N = (int)k.N;
   for (NodeWalk it(k.n, gridDim.x * KB); it.e < N; it.next()) {
     const int e = it.e;
-    double2 ax = apply_at(k.x, k.kh, e, it.i, it.j, k.n, 0.0);
+    double2 ax = apply_at(k.x, k.kh, k.d, e, it.i, it.j, k.n, 0.0);
     double2 bv = k.b[e];
     double2 tr = make_double2(fma(bv.x, k.scale_b, -ax.x), fma(bv.y, k.scale_b, -ax.y));
     k.tr[e] = tr;
     acc[0] = fma(tr.x, tr.x, fma(tr.y, tr.y, acc[0]));
   }
   double tot[1];
-  if (!grid_sum<1>(acc, k.partials, &st->ticket[KT_TRUE], tot)) return;
+  if (!grid_sum<1>(acc, k.partials, k.G, &st->ticket[KT_TRUE], tot)) return;
   if (threadIdx.x == 0) st->trr = tot[0];
 }
 
@@ -579,7 +737,7 @@ __global__ void k_restart_kernel(KrylovVecs k) {
     acc[2] = fma(r.x, r.x, fma(r.y, r.y, acc[2]));
   }
   double tot[3];
-  if (!grid_sum<3>(acc, k.partials, &st->ticket[KT_RESTART], tot)) return;
+  if (!grid_sum<3>(acc, k.partials, k.G, &st->ticket[KT_RESTART], tot)) return;
   if (threadIdx.x == 0) {
     st->rho = make_double2(tot[0], tot[1]);
     st->rr = tot[2];
@@ -594,17 +752,34 @@ __global__ void k_restart_kernel(KrylovVecs k) {
   }
 }
 
-__global__ void apply_fp64_kernel(double2* v, const double2* u, const double* kh, int n, double beta,
+// d = (k h)^2 - 4, the interior diagonal of L.
+__global__ void diag_kernel(double* __restrict__ d, const double* __restrict__ kh, int N) {
+  pdl_enter();
+  GRID_STRIDE(e, N) d[e] = fma(kh[e], kh[e], -4.0);
+}
+
+__global__ void apply_fp64_kernel(double2* v, const double2* u, const double* kh, const double* d, int n, double beta,
                                   double out_scale) {
   pdl_enter();
   const int N = (n + 1) * (n + 1);
   for (NodeWalk it(n, gridDim.x * KB); it.e < N; it.next()) {
     const int e = it.e;
-    double2 a = apply_at(u, kh, e, it.i, it.j, n, beta);
+    double2 a = apply_at(u, kh, d, e, it.i, it.j, n, beta);
     v[e] = make_double2(a.x * out_scale, a.y * out_scale);
   }
 }
 
+}  // namespace
+
+namespace {
+int device_sms() {
+  static int sms = 0;
+  if (!sms) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) || sms < 1) sms = 1;
+  }
+  return sms;
+}
 }  // namespace
 
 #define KGRID dim3(k.G, 1, k.batch)
@@ -621,25 +796,35 @@ cudaError_t launch_k_init(const KrylovVecs& k, double tol, int maxit, int hist_c
   return cudaGetLastError();
 }
 cudaError_t launch_k_update_p(const KrylovVecs& k, cudaStream_t s) { KLAUNCH(k_update_p_kernel) }
-cudaError_t launch_k_apply_rv(const KrylovVecs& k, cudaStream_t s) {
-  if (k.y32) pdl_launch(k_apply_rv_kernel<float2>, KGRID, KB, 0, s, k, k.y32);
-  else pdl_launch(k_apply_rv_kernel<double2>, KGRID, KB, 0, s, k, k.y);
+// Blocks of a full grid carry two of the reduction's G blocks each (see grid_sum): a thread then has two
+// nodes in flight, and all blocks are resident at once (1216 blocks of 40 registers run in 1.3 waves).
+// Small grids keep one, where latency counts.
+template <class Y2>
+cudaError_t apply_rv(const KrylovVecs& k, const Y2* y, cudaStream_t s) {
+  if (sizeof(Y2) == 8 && k.G > 4 * device_sms())
+    pdl_launch(k_apply_rv_kernel<float2, 2>, dim3((k.G + 1) / 2, 1, k.batch), KB, 0, s, k, (const float2*)y);
+  else
+    pdl_launch(k_apply_rv_kernel<Y2, 1>, KGRID, KB, 0, s, k, y);
   return cudaGetLastError();
+}
+template <class Y2>
+cudaError_t apply_ts(const KrylovVecs& k, const Y2* z, cudaStream_t s) {
+  if (sizeof(Y2) == 8 && k.G > 4 * device_sms())
+    pdl_launch(k_apply_ts_kernel<float2, 2>, dim3((k.G + 1) / 2, 1, k.batch), KB, 0, s, k, (const float2*)z);
+  else
+    pdl_launch(k_apply_ts_kernel<Y2, 1>, KGRID, KB, 0, s, k, z);
+  return cudaGetLastError();
+}
+cudaError_t launch_k_apply_rv(const KrylovVecs& k, cudaStream_t s) {
+  return k.y32 ? apply_rv<float2>(k, k.y32, s) : apply_rv<double2>(k, k.y, s);
 }
 cudaError_t launch_k_update_s(const KrylovVecs& k, cudaStream_t s) { KLAUNCH(k_update_s_kernel) }
 cudaError_t launch_k_apply_ts(const KrylovVecs& k, cudaStream_t s) {
-  if (k.z32) pdl_launch(k_apply_ts_kernel<float2>, KGRID, KB, 0, s, k, k.z32);
-  else pdl_launch(k_apply_ts_kernel<double2>, KGRID, KB, 0, s, k, k.z);
-  return cudaGetLastError();
+  return k.z32 ? apply_ts<float2>(k, k.z32, s) : apply_ts<double2>(k, k.z, s);
 }
 cudaError_t launch_k_update_r(const KrylovVecs& k, cudaStream_t s) { KLAUNCH(k_update_r_kernel) }
 cudaError_t launch_k_update_x(const KrylovVecs& k, bool omega_half, cudaStream_t s) {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) || sms < 1) sms = 1;
-  }
-  const dim3 grid(sms, 1, k.batch);  // one block per SM: the V-cycle kernels beside it keep the rest
+  const dim3 grid(device_sms(), 1, k.batch);  // one block per SM: the V-cycle kernels beside it keep the rest
   if (k.y32) {
     if (omega_half) pdl_launch(k_update_x_kernel<float2, true>, grid, XB, 0, s, k, (const float2*)k.z32);
     else pdl_launch(k_update_x_kernel<float2, false>, grid, XB, 0, s, k, (const float2*)k.y32);
@@ -656,12 +841,18 @@ cudaError_t launch_loop_control(const LoopCtl& c, cudaStream_t s) {
 }
 cudaError_t launch_k_restart(const KrylovVecs& k, cudaStream_t s) { KLAUNCH(k_restart_kernel) }
 
-cudaError_t launch_apply_fp64(double2* v, const double2* u, const double* kh, int n, double beta, double out_scale,
-                              cudaStream_t s) {
+cudaError_t launch_k_diag(double* d, const double* kh, long long N, cudaStream_t s) {
+  const int G = (int)((N + KB - 1) / KB < 4096 ? (N + KB - 1) / KB : 4096);
+  pdl_launch(diag_kernel, G, KB, 0, s, d, kh, (int)N);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_apply_fp64(double2* v, const double2* u, const double* kh, const double* d, int n, double beta,
+                              double out_scale, cudaStream_t s) {
   long long N = (long long)(n + 1) * (n + 1);
   int G = (int)((N + KB - 1) / KB);
   if (G > 4096) G = 4096;
-  pdl_launch(apply_fp64_kernel, G, KB, 0, s, v, u, kh, n, beta, out_scale);
+  pdl_launch(apply_fp64_kernel, G, KB, 0, s, v, u, kh, d, n, beta, out_scale);
   return cudaGetLastError();
 }
 
