@@ -63,8 +63,8 @@ typedef enum { HZ_SMOOTH_GS = 0, HZ_SMOOTH_KACZMARZ = 1, HZ_SMOOTH_DIRECT = 2, H
                HZ_SMOOTH_SOR = 4 } hz_smoother;
 
 /* Kernel forms of a Kaczmarz level (Sec. 4): one launch per colour; the whole level (sweeps,
-   residual and full weighting, or correction and sweeps) in one block's shared memory; one launch
-   per sweep over halo tiles; the whole level in the shared memory of a thread-block cluster of up
+   residual and full weighting, or correction and sweeps) in one block's shared memory; halo tiles
+   (FP32: one or two launches per pass, transfers included; FP64: one launch per sweep); the whole level in the shared memory of a thread-block cluster of up
    to 16 blocks (row bands, neighbour rows through distributed shared memory); the whole level in
    global memory by one persistent cooperative launch per pass, with bounded grid-wide barriers
    between the colour phases (single right-hand side only; a barrier wait that runs out ends the
@@ -95,10 +95,9 @@ typedef struct {
                        operations, same results as the per-level kernels for one-sweep Gauss-Seidel
                        and FP32 Kaczmarz levels); 0: one or more launches per level */
   int kacz_form;    /* how Kaczmarz levels below the finest run (hz_kacz_form): -1 (default) = one
-                       block if the level fits its shared memory, else tiles with two sweeps per
-                       launch (n_l >= 256, sweep count a multiple of 4), else a thread-block
-                       cluster, else tiles (even sweep counts), else colour launches in the FP32 form; a cluster,
-                       else colour launches in the FP64 form. A form that does not apply to a level
+                       block if the level fits its shared memory, else tiles (even sweep counts), else a
+                       thread-block cluster, else colour launches in the FP32 form; a cluster, else
+                       tiles up to n_l = 512, else colour launches in the FP64 form. A form that does not apply to a level
                        falls back to that default. */
   int gs_smoother;  /* smoother of the levels the rules of Sec. 5 give Gauss-Seidel: HZ_SMOOTH_GS
                        (default, red-black), HZ_SMOOTH_JACOBI (damped) or HZ_SMOOTH_SOR (red-black,
@@ -279,7 +278,7 @@ typedef enum {
   HZ_K_SMOOTH_RESTRICT, /* fused: GS sweep from a zero guess, residual, full weighting */
   HZ_K_PROLONG_SMOOTH, /* fused: bilinear correction and GS post-sweep */
   HZ_K_KACZ_LEVEL,     /* whole Kaczmarz level in one block (pre: sweeps + residual + FW; post: correction + sweeps) */
-  HZ_K_KACZ_SWEEP,     /* one five-colour Kaczmarz sweep over halo tiles */
+  HZ_K_KACZ_SWEEP,     /* Kaczmarz sweeps over halo tiles (FP32: a whole pass) */
   HZ_K_TAIL,           /* coarse tail: every level from hz_level_info.in_tail down, in one block */
   HZ_K_KACZ_CLUSTER,   /* whole Kaczmarz level over a thread-block cluster (pre or post, as HZ_K_KACZ_LEVEL) */
   HZ_K_JACOBI,         /* one damped Jacobi sweep, out of place */

@@ -49,6 +49,7 @@ struct Level {
   void* u2 = nullptr; // result of the fused post-smoothing pass (levels >= 1)
   int var_down = 0, var_up = 0;  // fused-pass variants (picked by the tile autotuner)
   int kform = 0;                 // hz_kacz_form of a Kaczmarz level (set up by plan_kaczmarz)
+  int pass_cfg = 0;              // tile geometry of its whole passes (pass_config)
   double omega = 1.0;            // relaxation factor of a Jacobi or SOR level
 };
 
@@ -388,21 +389,16 @@ bool kform_ok(const hz_problem* P, int l, int form) {
   }
   return false;
 }
-// Default form: FP32 - one block if the level fits, else a cluster, else tiles; FP64 - a cluster
-// (the FP64 pipe of one SM bounds the one-block form), else tiles up to n_l = 512, else colour
-// launches (the tiles' halo recomputation is FP64 work, which outweighs the saved launches on the
-// largest levels). Measured per Bi-CGSTAB iteration (four level launches): FP32 n_l = 128 cluster
-// 118 us, tiles 247 us; n_l = 256 cluster 240 us, tiles 259 us; FP64 n_l = 64 cluster 206 us,
+// Default form: FP32 - one block if the level fits, else tiles, else (odd sweep counts) a cluster; FP64
+// - a cluster (the FP64 pipe of one SM bounds the one-block form), else tiles up to n_l = 512, else
+// colour launches (the tiles' halo recomputation is FP64 work, which outweighs the saved launches on
+// the largest levels). Measured per Bi-CGSTAB iteration (four passes): FP32 n_l = 128 cluster 114 us,
+// tiles 93 us; n_l = 256 215 and 105 us; FP64 n_l = 64 cluster 206 us,
 // colour launches 820 us; FP64 in the n = 4096 solve's graph: n_l = 1024 tiles 2.67 ms, colour
 // launches 2.39 ms; n_l = 512 0.94 and 1.21 ms; n_l = 256 0.58 and 0.92 ms. All forms give the
 // same bits.
 int default_kform(const hz_problem* P, int l) {
-  // FP32 levels of n_l >= 256 with a multiple of 4 sweeps: two sweeps per tiled launch beat the
-  // cluster (config 3, n_l = 256: 0.13 ms per iteration against 0.23)
-  if (P->plan.fp32 && kacz_tile_sweeps_per_launch(true, P->lv[l].n, P->lv[l].nu) == 2 &&
-      !kacz_level_fits(true, P->lv[l].n) && kform_ok(P, l, HZ_KACZ_TILE))
-    return HZ_KACZ_TILE;
-  const int order32[] = {HZ_KACZ_LEVEL, HZ_KACZ_CLUSTER, HZ_KACZ_TILE}, order64[] = {HZ_KACZ_CLUSTER, HZ_KACZ_TILE};
+  const int order32[] = {HZ_KACZ_LEVEL, HZ_KACZ_TILE, HZ_KACZ_CLUSTER}, order64[] = {HZ_KACZ_CLUSTER, HZ_KACZ_TILE};
   const int* o = P->plan.fp32 ? order32 : order64;
   const int cnt = P->plan.fp32 ? 3 : (P->lv[l].n <= 512 ? 2 : 1);
   for (int q = 0; q < cnt; ++q)
@@ -416,23 +412,24 @@ void plan_kaczmarz(hz_problem* P) {
     if (L.smoother != HZ_SMOOTH_KACZMARZ) continue;
     const int want = P->opts.kacz_form;
     L.kform = (want >= 0 && kform_ok(P, l, want)) ? want : default_kform(P, l);
+    L.pass_cfg = pass_config(L.n, L.nu, P->plan.batch, P->num_sms);
   }
 }
 
-// Tiled sweeps on level l: `first_in` is the input of the first sweep (null = zero guess). One or
-// two sweeps per launch, ping-pong between u and u2 ending in u.
+// Tiled FP64 sweeps on level l, one per launch, ping-pong between u and u2 ending in u: `first_in` is
+// the input of the first sweep (null = zero guess). FP32 levels run whole passes (run_kacz_pass).
 cudaError_t kacz_tile_sweeps(hz_problem* P, int l, Src f, const void* first_in, bool post, const int* stop,
                              const Inst& bi) {
   const Level& L = P->lv[l];
   int pk;
   const void* kh = kh_of(P, l, &pk);
   const void* in = first_in;
-  const int per = kacz_tile_sweeps_per_launch(P->plan.fp32, L.n, L.nu), launches = L.nu / per;
   cudaError_t e;
-  for (int k = 0; k < launches; ++k) {
-    void* out = ((launches - 1 - k) % 2 == 0) ? L.u : L.u2;
-    if ((e = mark(P, launch_kacz_sweep_tile(P->plan.fp32, out, L.pitch, in, L.pitch, f.f, f.pf, f.f64, kh, pk, L.n,
-                                            op_beta(P, L.relax_op), post, per, stop, P->stream, bi),
+  for (int k = 0; k < L.nu; ++k) {
+    void* out = ((L.nu - 1 - k) % 2 == 0) ? L.u : L.u2;
+    if ((e = mark(P, launch_kacz_sweep_tile64((double2*)out, L.pitch, (const double2*)in, L.pitch, (const double2*)f.f,
+                                              f.pf, (const double*)kh, pk, L.n, op_beta(P, L.relax_op), post, stop,
+                                              P->stream, bi),
                   HZ_K_KACZ_SWEEP, l)))
       return e;
     in = out;
@@ -468,9 +465,33 @@ cudaError_t jacobi_sweeps(hz_problem* P, int l, Src f, bool from_zero, int sweep
   return cudaSuccess;
 }
 
+// A tiled Kaczmarz level whose passes run whole (hz_kpass.cu).
+bool kacz_pass(const hz_problem* P, int l) {
+  return l > 0 && l < P->plan.levels - 1 && P->plan.fp32 && P->lv[l].smoother == HZ_SMOOTH_KACZMARZ &&
+         P->lv[l].kform == HZ_KACZ_TILE;
+}
+
 // Where level l's result after post-relaxation lives (what level l-1 interpolates).
 void* final_u(const hz_problem* P, int l) {
-  return (l > 0 && fused(P, l)) ? P->lv[l].u2 : P->lv[l].u;
+  const bool out_of_place = fused(P, l) || (kacz_pass(P, l) && !pass_in_place(P->lv[l].pass_cfg, P->lv[l].nu));
+  return (l > 0 && out_of_place) ? P->lv[l].u2 : P->lv[l].u;
+}
+cudaError_t run_kacz_pass(hz_problem* P, int l, Src f, bool post, const int* stop, const Inst& bi) {
+  const Level& L = P->lv[l];
+  const Level& C = P->lv[l + 1];
+  KaczPassArgs a;
+  a.pu = L.pitch;
+  a.fc = (float2*)C.f;
+  a.ec = (const float2*)final_u(P, l + 1);
+  a.pc = C.pitch;
+  a.f = (const float2*)f.f;
+  a.pf = f.pf;
+  a.kh = (const float*)kh_of(P, l, &a.pk);
+  a.n = L.n;
+  a.bA = (float)op_beta(P, L.relax_op);
+  a.bB = (float)op_beta(P, L.resid_op);
+  a.stop = stop;
+  return mark(P, launch_kacz_pass(post, L.pass_cfg, L.nu, a, (float2*)L.u, (float2*)L.u2, P->stream, bi), HZ_K_KACZ_SWEEP, l);
 }
 
 // Pre-relaxation from a zero guess on level l into lv[l].u and the restricted residual into
@@ -502,6 +523,7 @@ cudaError_t level_down(hz_problem* P, int l, Src f, const int* stop, bool all = 
     return mark(P, launch_kacz_grid_pre(fp32, u, pu, C.f, C.pitch, f.f, f.pf, kh, pk, L.n, bA, bB, L.nu, stop,
                                         band_sync_of(P, l), s),
                 HZ_K_KACZ_GRID, l);
+  if (kacz_pass(P, l)) return run_kacz_pass(P, l, f, false, stop, bi);
   if (kp == KACZ_TILE) {
     if ((e = kacz_tile_sweeps(P, l, f, nullptr, false, stop, bi))) return e;
     return mark(P, launch_restrict_residual(fp32, C.f, C.pitch, u, pu, f.f, f.pf, f.f64, kh, pk, L.n, bB, stop, s, bi),
@@ -596,6 +618,7 @@ cudaError_t level_up(hz_problem* P, int l, Src f, void* out, int po, const int* 
                                          op_beta(P, L.relax_op), L.nu, stop, band_sync_of(P, l), P->stream),
                 HZ_K_KACZ_GRID, l);
   }
+  if (kacz_pass(P, l)) return run_kacz_pass(P, l, f, true, stop, bi);
   if ((e = mark(P, launch_prolong_add(fp32, L.u, L.pitch, ec, C.pitch, L.n, stop, P->stream, bi), HZ_K_PROLONG, l))) return e;
   if (kp == KACZ_TILE) {
     if ((e = kacz_tile_sweeps(P, l, f, L.u, true, stop, bi))) return e;

@@ -123,11 +123,10 @@ cudaError_t launch_kacz_grid_pre(bool fp32, void* u, int pu, void* fc, int pc, c
 cudaError_t launch_kacz_grid_post(bool fp32, void* u, int pu, const void* ec, int pc, const void* f, int pf,
                                   const void* kh, int pk, int n, double bA, int nu, const int* stop, BandSync bs,
                                   cudaStream_t s);
-// `sweeps` (1 or 2, from kacz_tile_sweeps_per_launch) Kaczmarz sweeps per launch over halo tiles.
-int kacz_tile_sweeps_per_launch(bool fp32, int n, int nu);
-cudaError_t launch_kacz_sweep_tile(bool fp32, void* uout, int po, const void* uin, int pu, const void* f, int pf,
-                                   bool f64_src, const void* kh, int pk, int n, double bA, bool post, int sweeps,
-                                   const int* stop, cudaStream_t s, const Inst& bi = Inst());
+// One FP64 Kaczmarz sweep over halo tiles.
+cudaError_t launch_kacz_sweep_tile64(double2* uout, int po, const double2* uin, int pu, const double2* f, int pf,
+                                     const double* kh, int pk, int n, double bA, bool post, const int* stop,
+                                     cudaStream_t s, const Inst& bi = Inst());
 // Coarse tail (hz_tail.cu): levels lt .. L-1 of the V-cycle in one block's shared memory.
 constexpr int TAIL_MAX_LEVELS = 12;
 constexpr int TAIL_MAX_SMEM = 200 * 1024;
@@ -169,6 +168,29 @@ cudaError_t launch_inject_kh(bool fp32, void* kh, int pk, const double* k0, int 
 // work: 2 * m * m double2 scratch, m = (nc+1)^2. status: device int, 0 on success, 1 if singular.
 cudaError_t launch_coarse_setup(bool fp32, void* ainvT, double2* work, const void* kh, int pk, int nc, double beta,
                                 int* status, cudaStream_t s);
+
+// A whole pre- or post-relaxation pass (nu sweeps, nu even) of an FP32 Kaczmarz level below the finest,
+// with its transfer, in launches of independent tiles (hz_kpass.cu) of the geometry that pass_config
+// picks. Pre: zero guess into u, restricted residual into fc. Post: sweeps of u + P ec, ending in u
+// (pass_in_place) or in u2.
+struct KaczPassArgs {
+  const float2* uin = nullptr;  // set per launch
+  float2* uout = nullptr;
+  int pu = 0;
+  float2* fc = nullptr;
+  const float2* ec = nullptr;
+  int pc = 0;
+  const float2* f = nullptr;
+  int pf = 0;
+  const float* kh = nullptr;
+  int pk = 0, n = 0;
+  float bA = 0, bB = 0;
+  const int* stop = nullptr;
+};
+int pass_config(int n, int nu, int batch, int sms);
+bool pass_in_place(int cfg, int nu);
+cudaError_t launch_kacz_pass(bool post, int cfg, int nu, const KaczPassArgs& a, float2* u, float2* u2, cudaStream_t s,
+                             const Inst& bi);
 
 // ---------------------------------------------------------------- Krylov (FP64)
 

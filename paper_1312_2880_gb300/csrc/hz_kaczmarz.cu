@@ -9,10 +9,10 @@
 //   diagonal and 1/|a_p|^2 computed once per launch (operations in hz_level.cuh). Pre mode: zero guess, nu sweeps (colours
 //   0..4), then the residual with the (B) operator and full weighting onto the coarse level. Post
 //   mode: u_pre + P e_c, then nu sweeps (colours 4..0).
-// kacz_sweep_tile: one or two full sweeps (all five colours each) per launch over tiles with a halo
-//   that holds the dependency cone of the sweeps (6 columns each side, 6 and 10 rows per sweep), so
-//   the tile interior holds exactly the sequential sweeps' values; each phase acts only on the
-//   part of the region that can still reach the tile. Out of place.
+// kacz_sweep_tile64: one full FP64 sweep (all five colours) per launch over tiles with a halo that holds
+//   the dependency cone of the sweep (6 columns each side, 6 and 10 rows), so the tile interior holds
+//   exactly the sequential sweep's values; each phase acts only on the part of the region that can
+//   still reach the tile. Out of place. (FP32 levels run whole passes in tiles: hz_kpass.cu.)
 // kacz_cluster_*: the kacz_level_* operations with the level split into row bands over a
 //   thread-block cluster of up to 16 blocks (distributed shared memory, one cluster barrier per
 //   colour), for levels too large for one block or, in FP64, too slow on one SM's FP64 pipe.
@@ -32,7 +32,7 @@ namespace hz {
 namespace {
 
 constexpr int LB = 1024;  // threads of the whole-level kernel
-// Tiles of the tiled form: KT x KT outputs per block after S sweeps per launch. The halo is the
+// Tiles of the tiled forms (FP64 here, FP32 in hz_kpass.cu): KT x KT outputs per block after S sweeps per launch. The halo is the
 // dependency cone of S five-colour sweeps (found by propagating dependencies through the colour
 // phases on an unbounded grid, every residue of the colour pattern): after one sweep in the order
 // 0..4 an output depends on starting values at most 6 columns to either side, 6 rows below and 10
@@ -44,19 +44,15 @@ struct TileGeo {
   static constexpr int HN = 6 * S_, HF = 10 * S_;  // halo rows on the near and the far side
   static constexpr int RX = KT_ + 2 * HX, RY = KT_ + HN + HF, REG = RX * RY;
 };
-using TileOne = TileGeo<32, 1, 256>;   // one sweep per launch: 44 x 48 regions
-using TileTwo = TileGeo<64, 2, 1024>;  // two sweeps per launch: 88 x 96 regions (FP32, n_l >= 1024)
-using TileTwoS = TileGeo<32, 2, 512>;  // two sweeps per launch: 56 x 64 regions (FP32, n_l = 256 .. 1023)
-template <class T, class G>
-constexpr size_t tile_smem() { return (size_t)G::REG * (2 * sizeof(c2<T>) + sizeof(T)); }
+using TileOne = TileGeo<32, 1, 256>;  // one sweep per launch: 44 x 48 regions
+constexpr size_t tile_smem() { return (size_t)TileOne::REG * (2 * sizeof(double2) + sizeof(double)); }
 
 // Actions of phase ph (of P = 5S; R = P - 1 - ph phases follow it) that can still reach the
 // tile's outputs. Propagating dependencies back from the outputs through the colour phases on an
 // unbounded grid (every residue of the colour pattern gives the same bounds) leaves, in tile
 // coordinates (output origin 0), the phase's colour in columns -1-R .. KT+R and rows -1-R .. KT+2R
 // (order 0..4) or -1-2R .. KT+R (order 4..0). An action outside that rectangle changes only values
-// no output depends on, so leaving it out keeps the outputs' bits, and it cuts the actions of a
-// two-sweep launch on 64-node tiles by a third against sweeping the whole region every phase.
+// no output depends on, so leaving it out keeps the outputs' bits.
 // Slot q of a phase is the (q mod per)-th node of the colour from column xlo in row ylo + q / per.
 template <class G, bool POST>
 struct PhaseRect {
@@ -285,10 +281,15 @@ __global__ void __launch_bounds__(LB) kacz_level_post_kernel(c2<T>* __restrict__
   lvl::for_nodes_blocked(n, [&](int, int i, int j, int p) { u[(long long)j * pu + i] = S.su[p]; });
 }
 
-template <class T, class F2, class G, bool POST>
-__device__ __forceinline__ void tile_sweeps(c2<T>* __restrict__ uout, int po, const c2<T>* __restrict__ uin, int pu,
-                                            const F2* __restrict__ f, int pf, const T* __restrict__ kh, int pk, int n,
-                                            T bA, const int* __restrict__ stop, Inst bi) {
+template <bool POST>
+__global__ void __launch_bounds__(TileOne::TBK) kacz_sweep_tile64_kernel(double2* __restrict__ uout, int po,
+                                                                         const double2* __restrict__ uin, int pu,
+                                                                         const double2* __restrict__ f, int pf,
+                                                                         const double* __restrict__ kh, int pk, int n,
+                                                                         double bA, const int* __restrict__ stop,
+                                                                         Inst bi) {
+  using T = double;
+  using G = TileOne;
   using PR = PhaseRect<G, POST>;
   static_assert(PR::fits(), "phase rectangles must keep their supports inside the tile region");
   constexpr int TBK = G::TBK, RX = G::RX, RY = G::RY, REG = G::REG, KT = G::KT;
@@ -309,7 +310,6 @@ __device__ __forceinline__ void tile_sweeps(c2<T>* __restrict__ uout, int po, co
   // the tile region's u, f~ and k H in flight at once (cp.async, one wait): a plain load per node
   // would put one L2 latency per node a thread copies on the launch's critical path. A warp
   // takes whole region rows, a lane every 32nd column: no division per node.
-  constexpr bool async_f = sizeof(F2) == sizeof(c2<T>);  // f~ in the level's own precision
   constexpr int NW = TBK / 32;
   const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
   for (int r = warp; r < RY; r += NW) {
@@ -323,10 +323,7 @@ __device__ __forceinline__ void tile_sweeps(c2<T>* __restrict__ uout, int po, co
         lvl::cp_async<sizeof(c2<T>)>(su + q, uin + ju + i);
       else
         su[q] = mk<T>(0, 0);
-      if constexpr (async_f)
-        lvl::cp_async<sizeof(c2<T>)>(sf + q, f + jf + i);
-      else
-        sf[q] = ldc<T>(f, jf + i);
+      lvl::cp_async<sizeof(c2<T>)>(sf + q, f + jf + i);
       lvl::cp_async<sizeof(T)>(sk + q, kh + jk + i);
     }
   }
@@ -353,33 +350,6 @@ __device__ __forceinline__ void tile_sweeps(c2<T>* __restrict__ uout, int po, co
     }
   }
 }
-
-// FP32 tiles are held to 56 registers a thread, so that a 1024-thread block leaves room for the
-// deferred solution update (k_update_x, one 128-thread block per SM) beside it; the FP64 tiles
-// (256 threads) need more.
-template <class F2, class G, bool POST>
-__global__ void __maxnreg__(56) kacz_sweep_tile_kernel(float2* __restrict__ uout, int po,
-                                                       const float2* __restrict__ uin, int pu,
-                                                       const F2* __restrict__ f, int pf, const float* __restrict__ kh,
-                                                       int pk, int n, float bA, const int* __restrict__ stop, Inst bi) {
-  tile_sweeps<float, F2, G, POST>(uout, po, uin, pu, f, pf, kh, pk, n, bA, stop, bi);
-}
-template <class G, bool POST>
-__global__ void __launch_bounds__(G::TBK) kacz_sweep_tile64_kernel(double2* __restrict__ uout, int po,
-                                                                   const double2* __restrict__ uin, int pu,
-                                                                   const double2* __restrict__ f, int pf,
-                                                                   const double* __restrict__ kh, int pk, int n,
-                                                                   double bA, const int* __restrict__ stop, Inst bi) {
-  tile_sweeps<double, double2, G, POST>(uout, po, uin, pu, f, pf, kh, pk, n, bA, stop, bi);
-}
-template <class T, class F2, class G, bool POST>
-struct TileKernel {
-  static constexpr auto fn = kacz_sweep_tile_kernel<F2, G, POST>;
-};
-template <class G, bool POST>
-struct TileKernel<double, double2, G, POST> {
-  static constexpr auto fn = kacz_sweep_tile64_kernel<G, POST>;
-};
 
 template <class T>
 size_t level_smem(int n) {
@@ -633,53 +603,27 @@ cudaError_t launch_cluster_kernel(void (*kernel)(Args...), int c, size_t smem, c
 
 }  // namespace
 
-template <class T, class F2, class G, bool POST>
-cudaError_t tile_attr() {
-  static bool done = false;
-  if (done) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(TileKernel<T, F2, G, POST>::fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)tile_smem<T, G>());
-  if (!e) done = true;
-  return e;
-}
-
-template <class T, class F2, class G>
-cudaError_t tile_launch(void* uout, int po, const void* uin, int pu, const void* f, int pf, const void* kh, int pk,
-                        int n, double bA, bool post, const int* stop, cudaStream_t s, const Inst& bi) {
-  cudaError_t e = post ? tile_attr<T, F2, G, true>() : tile_attr<T, F2, G, false>();
-  if (e) return e;
-  dim3 grid((n + G::KT) / G::KT, (n + G::KT) / G::KT, bi.count);
-  if (post)
-    pdl_launch(TileKernel<T, F2, G, true>::fn, grid, G::TBK, tile_smem<T, G>(), s, (c2<T>*)uout, po,
-               (const c2<T>*)uin, pu, (const F2*)f, pf, (const T*)kh, pk, n, (T)bA, stop, bi);
-  else
-    pdl_launch(TileKernel<T, F2, G, false>::fn, grid, G::TBK, tile_smem<T, G>(), s, (c2<T>*)uout, po,
-               (const c2<T>*)uin, pu, (const F2*)f, pf, (const T*)kh, pk, n, (T)bA, stop, bi);
+template <bool POST>
+cudaError_t tile_launch(double2* uout, int po, const double2* uin, int pu, const double2* f, int pf, const double* kh,
+                        int pk, int n, double bA, const int* stop, cudaStream_t s, const Inst& bi) {
+  static bool ready = false;
+  if (!ready) {
+    cudaError_t e = cudaFuncSetAttribute(kacz_sweep_tile64_kernel<POST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)tile_smem());
+    if (e) return e;
+    ready = true;
+  }
+  const int t = (n + TileOne::KT) / TileOne::KT;
+  pdl_launch(kacz_sweep_tile64_kernel<POST>, dim3(t, t, bi.count), TileOne::TBK, tile_smem(), s, uout, po, uin, pu, f, pf,
+             kh, pk, n, bA, stop, bi);
   return cudaGetLastError();
 }
 
-int kacz_tile_sweeps_per_launch(bool fp32, int n, int nu) {
-  // two sweeps per launch on FP32 levels of at least 256 intervals: with the two-sweep halo,
-  // 64-node tiles (n_l >= 1024) read 1.03 region nodes per output and sweep and 32-node tiles
-  // (n_l = 256 .. 1023, where 64-node tiles are too few to fill the GPU) 1.75, against 2.06 for
-  // one sweep on 32-node tiles. The launches ping-pong between two arrays and must end in u from an
-  // input in u, so their number has to be even: nu a multiple of 4.
-  return (fp32 && n >= 256 && nu % 4 == 0) ? 2 : 1;
-}
-
-cudaError_t launch_kacz_sweep_tile(bool fp32, void* uout, int po, const void* uin, int pu, const void* f, int pf,
-                                   bool f64_src, const void* kh, int pk, int n, double bA, bool post, int sweeps,
-                                   const int* stop, cudaStream_t s, const Inst& bi) {
-  if (!fp32)
-    return tile_launch<double, double2, TileOne>(uout, po, uin, pu, f, pf, kh, pk, n, bA, post, stop, s, bi);
-  if (sweeps == 2 && n >= 1024)
-    return f64_src ? tile_launch<float, double2, TileTwo>(uout, po, uin, pu, f, pf, kh, pk, n, bA, post, stop, s, bi)
-                   : tile_launch<float, float2, TileTwo>(uout, po, uin, pu, f, pf, kh, pk, n, bA, post, stop, s, bi);
-  if (sweeps == 2)
-    return f64_src ? tile_launch<float, double2, TileTwoS>(uout, po, uin, pu, f, pf, kh, pk, n, bA, post, stop, s, bi)
-                   : tile_launch<float, float2, TileTwoS>(uout, po, uin, pu, f, pf, kh, pk, n, bA, post, stop, s, bi);
-  return f64_src ? tile_launch<float, double2, TileOne>(uout, po, uin, pu, f, pf, kh, pk, n, bA, post, stop, s, bi)
-                 : tile_launch<float, float2, TileOne>(uout, po, uin, pu, f, pf, kh, pk, n, bA, post, stop, s, bi);
+cudaError_t launch_kacz_sweep_tile64(double2* uout, int po, const double2* uin, int pu, const double2* f, int pf,
+                                     const double* kh, int pk, int n, double bA, bool post, const int* stop,
+                                     cudaStream_t s, const Inst& bi) {
+  return post ? tile_launch<true>(uout, po, uin, pu, f, pf, kh, pk, n, bA, stop, s, bi)
+              : tile_launch<false>(uout, po, uin, pu, f, pf, kh, pk, n, bA, stop, s, bi);
 }
 
 namespace {
