@@ -1969,8 +1969,8 @@ static size_t ray_layout(int n, int m, RayBlocks* B, double2** ph, unsigned char
   B->y = (double2*)take(vec);
   B->e = (double2*)take(vec);
   B->dz = (double2*)take(vec);
-  B->fcol = (double2*)take(sizeof(double2) * Bs);
-  B->perm = (int*)take(sizeof(int) * Bs);
+  B->fcol = (double2*)take(sizeof(double2) * 2 * Bs);
+  B->perm = (int*)take(sizeof(int) * 2 * Bs);
   B->status = (int*)take(sizeof(int));
   *ph = (double2*)take(sizeof(double2) * 8 * (size_t)(n + 1) * (n + 1));
   return off;

@@ -301,10 +301,10 @@ cudaError_t launch_apply_fp64(double2* v, const double2* u, const double* kh, co
 struct RayBlocks {
   int n = 0, m = 0, Nr = 0, Bs = 0;
   double2 *L = nullptr, *D = nullptr, *U = nullptr;     // assembled blocks (kept)
-  double2 *Sinv = nullptr, *G = nullptr, *W = nullptr;  // S_J^{-1}, L_J S_{J-1}^{-1}, S_J^{-1} U_J
+  double2 *Sinv = nullptr, *G = nullptr, *W = nullptr;  // S_J^{-1} and the products towards and from the middle row (hz_ray.cu)
   double2 *g = nullptr, *z = nullptr, *y = nullptr, *e = nullptr, *dz = nullptr;  // solve vectors
-  double2* fcol = nullptr;  // Bs: pivot column of the current Gauss-Jordan step
-  int* perm = nullptr;      // Bs: pivot rows of the current inversion
+  double2* fcol = nullptr;  // 2 Bs: pivot columns of the current Gauss-Jordan steps (two matrices at once)
+  int* perm = nullptr;      // 2 Bs: pivot rows of the current inversions
   int* status = nullptr;    // device int: set to 1 by a zero or non-finite pivot column
 };
 cudaError_t launch_ray_phases(double2* ph, int n, double k, cudaStream_t s);

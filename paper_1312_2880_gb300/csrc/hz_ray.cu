@@ -9,9 +9,16 @@
 // The ray operator couples ray nodes at most one apart, so ordered by rows of ray nodes it is
 // block tridiagonal: block row J holds the 8 (nc + 1) unknowns of ray row J (node-major, eight
 // directions inner), with blocks L_J (row J - 1), D_J and U_J (row J + 1). It is factored once by
-// block LU: S_0 = D_0, S_J = D_J - L_J S_{J-1}^{-1} U_{J-1}, each S_J inverted by Gauss-Jordan
-// elimination with row pivoting; the solve keeps S_J^{-1}, G_J = L_J S_{J-1}^{-1} and
-// W_J = S_J^{-1} U_J, and runs one step of iterative refinement on the block residual.
+// a two-sided block LU that eliminates from both ends towards the middle row Mid = Nr / 2:
+//   J < Mid: S_0 = D_0,      S_J = D_J - L_J S_{J-1}^{-1} U_{J-1}   (from the row below)
+//   J > Mid: S_{Nr-1} = D_{Nr-1}, S_J = D_J - U_J S_{J+1}^{-1} L_{J+1}   (from the row above)
+//   S_Mid = D_Mid - L_Mid S_{Mid-1}^{-1} U_{Mid-1} - U_Mid S_{Mid+1}^{-1} L_{Mid+1},
+// each S_J inverted by Gauss-Jordan elimination with row pivoting. The solve keeps S_J^{-1}, the
+// products that carry a row towards the middle (G: L_J S_{J-1}^{-1} in slot J, U_J S_{J+1}^{-1} in
+// slot J + 1) and back (W: S_J^{-1} U_J below the middle, S_J^{-1} L_J above), and runs one step of
+// iterative refinement on the block residual. The two chains are independent, so every step of the
+// factorisation and of the substitutions works on two block rows at once: half the dependent
+// steps of a one-sided elimination, which are what bounds the solve beside the FP64 pipe.
 //
 // Every kernel here is launched with programmatic stream serialization and starts with pdl_enter()
 // (hz_common.cuh): it waits for its predecessor before reading anything.
@@ -192,9 +199,16 @@ __global__ void ray_prolong_add_kernel(double2* x, const double2* z, const doubl
 // of largest |S[i][k]| (i >= k; the first on ties) is swapped into row k and recorded in perm[k];
 // column k is saved in fcol; row k is scaled by 1 / pivot with the pivot's own entry replaced by
 // 1 / pivot. A zero or non-finite pivot column sets *status = 1 (the inverse is then meaningless).
-__global__ void __launch_bounds__(1024) ray_gj_pivot_kernel(double2* S, int Bs, int k, double2* fcol, int* perm,
+// Block b of the launch works on the b-th of up to two matrices (with its own fcol and perm).
+struct Pair {
+  double2* p[2];
+};
+__global__ void __launch_bounds__(1024) ray_gj_pivot_kernel(Pair m, int Bs, int k, double2* fcol, int* perm,
                                                             int* status) {
   pdl_enter();
+  double2* S = blockIdx.x ? m.p[1] : m.p[0];
+  fcol += blockIdx.x * Bs;
+  perm += blockIdx.x * Bs;
   __shared__ double sv[32];
   __shared__ int si[32];
   __shared__ int piv;
@@ -259,8 +273,10 @@ __global__ void __launch_bounds__(1024) ray_gj_pivot_kernel(double2* S, int Bs, 
 }
 
 // Rows i != k: S[i][c] = (c == k ? 0 : S[i][c]) - fcol[i] S[k][c]  (row k is only read).
-__global__ void ray_gj_elim_kernel(double2* S, int Bs, int k, const double2* fcol) {
+__global__ void ray_gj_elim_kernel(Pair m, int Bs, int k, const double2* fcol) {
   pdl_enter();
+  double2* S = blockIdx.z ? m.p[1] : m.p[0];
+  fcol += blockIdx.z * Bs;
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   const int i = blockIdx.y;
   if (c >= Bs || i == k) return;
@@ -273,8 +289,10 @@ __global__ void ray_gj_elim_kernel(double2* S, int Bs, int k, const double2* fco
 }
 
 // Undo the row interchanges on the inverse: columns k and perm[k] swapped, k = Bs-1 .. 0.
-__global__ void ray_gj_unpermute_kernel(double2* S, int Bs, const int* perm) {
+__global__ void ray_gj_unpermute_kernel(Pair m, int Bs, const int* perm) {
   pdl_enter();
+  double2* S = blockIdx.y ? m.p[1] : m.p[0];
+  perm += blockIdx.y * Bs;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= Bs) return;
   double2* row = S + (long long)i * Bs;
@@ -290,9 +308,19 @@ __global__ void ray_gj_unpermute_kernel(double2* S, int Bs, const int* perm) {
 
 // C = A B (acc 0) or C = C - A B (acc 1) for Bs x Bs row-major blocks; C aliases neither A nor B.
 // A 32 x 32 tile of C per block of 256 threads, each thread 2 x 2 entries, k in steps of 16.
-__global__ void __launch_bounds__(256) ray_gemm_kernel(double2* C, const double2* A, const double2* B, int Bs,
-                                                       int acc) {
+// The z-th of up to two products.
+struct GemmJob {
+  double2* C;
+  const double2 *A, *B;
+};
+struct GemmJobs {
+  GemmJob j[2];
+};
+__global__ void __launch_bounds__(256) ray_gemm_kernel(GemmJobs jobs, int Bs, int acc) {
   pdl_enter();
+  const GemmJob job = blockIdx.z ? jobs.j[1] : jobs.j[0];
+  double2* C = job.C;
+  const double2 *A = job.A, *B = job.B;
   __shared__ double2 As[32][17];
   __shared__ double2 Bsh[16][33];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -332,53 +360,70 @@ __global__ void __launch_bounds__(256) ray_gemm_kernel(double2* C, const double2
     }
 }
 
-// out_b = base_b + sgn M_b x_b for b = blockIdx.y (M_b advances Bs^2 entries, the vectors Bs);
-// base may be null (zero) or equal to out; x aliases neither. One block of GEMV_THREADS per row
-// (blockIdx.x): GB300's FP64 pipe is narrow, so a row is spread over four warps to keep every SM
-// sub-partition busy, and each complex product is accumulated with four FMAs.
-constexpr int GEMV_THREADS = 128;
-__global__ void __launch_bounds__(GEMV_THREADS) ray_gemv_kernel(double2* out, const double2* base, const double2* M,
-                                                                const double2* x, int Bs, double sgn) {
-  pdl_enter();
-  const int row = blockIdx.x;
-  const long long b = blockIdx.y;
-  const double2* Mr = M + b * Bs * (long long)Bs + (long long)row * Bs;
-  const double2* xb = x + b * Bs;
+// out = base + sgn (M x + M2 x2) for job blockIdx.y (base and M2 may be null; base may equal out), or,
+// with BATCH, job 0 advanced to block row blockIdx.y. One warp per row.
+//
+// Bound by the FP64 pipe (four FMAs a complex element, 77 cycles a warp instruction on a sub-partition:
+// 4.1 us for the two 520 x 520 products of a step at n = 512) and by the latency of the chain. A row's
+// elements are factors, fixed since set-up, so a warp loads its first 32 GEMV_PRE of them before it
+// waits for the preceding launch, and the launch after it may start as soon as every block has begun:
+// the factors' trip from HBM overlaps the step before. The real and imaginary parts are reduced
+// together in the two halves of the warp (five additions where two shuffle trees took ten: at 77
+// cycles each, four warps per row with a tree apiece spent a third of a step's FP64 time there, and
+// 128 threads on 520 columns left one warp twice the work of the others). A solve at n = 512 took
+// 2.23 ms with the one-sided elimination and four warps per row, 1.86 ms now; at n = 256 0.71 and
+// 0.50 ms; the factorisation 1.21 s and 0.77 s.
+constexpr int GEMV_WARPS = 4, GEMV_PRE = 17;
+struct GemvJob {
+  double2* out;
+  const double2 *base, *M, *x, *M2, *x2;
+};
+struct GemvJobs {
+  GemvJob j[2];
+};
+template <bool BATCH>
+__global__ void __launch_bounds__(32 * GEMV_WARPS) ray_gemv_kernel(GemvJobs jobs, int Bs, double sgn) {
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  const GemvJob job = !BATCH && blockIdx.y ? jobs.j[1] : jobs.j[0];
+  const long long b = BATCH ? blockIdx.y : 0;
+  const int row = blockIdx.x * GEMV_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const bool live = row < Bs;
+  const double2* Mr = job.M + b * Bs * (long long)Bs + (long long)(live ? row : 0) * Bs;
+  double2 a[GEMV_PRE];
+#pragma unroll
+  for (int q = 0; q < GEMV_PRE; ++q) {
+    const int c = lane + 32 * q;
+    a[q] = c < Bs ? Mr[c] : make_double2(0.0, 0.0);
+  }
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  if (!live) return;
   double re = 0.0, im = 0.0;
-  for (int c0 = threadIdx.x; c0 < Bs; c0 += 4 * GEMV_THREADS) {
-    double2 a[4], v[4];
+  auto acc = [&](double2 m, double2 v) {
+    re = fma(m.x, v.x, re);
+    re = fma(-m.y, v.y, re);
+    im = fma(m.x, v.y, im);
+    im = fma(m.y, v.x, im);
+  };
+  const double2* x = job.x + b * Bs;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int c = c0 + GEMV_THREADS * u;
-      a[u] = c < Bs ? Mr[c] : make_double2(0.0, 0.0);
-      v[u] = c < Bs ? xb[c] : make_double2(0.0, 0.0);
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      re = fma(a[u].x, v[u].x, re);
-      re = fma(-a[u].y, v[u].y, re);
-      im = fma(a[u].x, v[u].y, im);
-      im = fma(a[u].y, v[u].x, im);
-    }
+  for (int q = 0; q < GEMV_PRE; ++q) {
+    const int c = lane + 32 * q;
+    if (32 * q < Bs) acc(a[q], c < Bs ? __ldcg(x + c) : make_double2(0.0, 0.0));
   }
-  re = warp_sum(re);
-  im = warp_sum(im);
-  __shared__ double red[2][GEMV_THREADS / 32];
-  const int warp = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) {
-    red[0][warp] = re;
-    red[1][warp] = im;
+  for (int c = lane + 32 * GEMV_PRE; c < Bs; c += 32) acc(Mr[c], __ldcg(x + c));
+  if (!BATCH && job.M2) {
+    const double2* M2r = job.M2 + (long long)row * Bs;
+    for (int c = lane; c < Bs; c += 32) acc(M2r[c], __ldcg(job.x2 + c));
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double sr = 0.0, si = 0.0;
+  // lanes 0 .. 15 reduce the real part, 16 .. 31 the imaginary part
+  const bool hi = lane >= 16;
+  double v = hi ? im : re;
+  v += __shfl_xor_sync(0xffffffffu, hi ? re : im, 16);
 #pragma unroll
-    for (int w = 0; w < GEMV_THREADS / 32; ++w) {
-      sr += red[0][w];
-      si += red[1][w];
-    }
-    const double2 o = base ? base[b * Bs + row] : make_double2(0.0, 0.0);
-    out[b * Bs + row] = make_double2(o.x + sgn * sr, o.y + sgn * si);
+  for (int o = 8; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((lane & 15) == 0) {
+    const double* base = job.base ? reinterpret_cast<const double*>(job.base + b * Bs + row) + hi : nullptr;
+    reinterpret_cast<double*>(job.out + b * Bs + row)[hi] = fma(sgn, v, base ? __ldcg(base) : 0.0);
   }
 }
 
@@ -406,10 +451,11 @@ __global__ void __launch_bounds__(128) ray_block_residual_kernel(double2* e, con
   e[t] = make_double2(g[t].x - re, g[t].y - im);
 }
 
-__global__ void ray_copy_kernel(double2* dst, const double2* src, int cnt) {
+// dst = src on entries [0, cnt) and [last, last + cnt) (blockIdx.y).
+__global__ void ray_copy_kernel(double2* dst, const double2* src, int cnt, int last) {
   pdl_enter();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < cnt) dst[i] = src[i];
+  if (i < cnt) dst[blockIdx.y * last + i] = src[blockIdx.y * last + i];
 }
 
 constexpr int RED_BLOCKS = 512, RED_THREADS = 256;
@@ -486,57 +532,92 @@ cudaError_t launch_ray_prolong_add(double2* x, const double2* z, const double2* 
 
 namespace {
 
-cudaError_t gj_inverse(double2* S, int Bs, double2* fcol, int* perm, int* status, cudaStream_t s) {
-  const dim3 eg(blocks_for(Bs, 128), Bs);
+cudaError_t gj_inverse(const Pair& S, int count, int Bs, double2* fcol, int* perm, int* status, cudaStream_t s) {
+  const dim3 eg(blocks_for(Bs, 128), Bs, count);
   for (int k = 0; k < Bs; ++k) {
-    cudaError_t e = pdl_launch(ray_gj_pivot_kernel, dim3(1), dim3(1024), 0, s, S, Bs, k, fcol, perm, status);
+    cudaError_t e = pdl_launch(ray_gj_pivot_kernel, dim3(count), dim3(1024), 0, s, S, Bs, k, fcol, perm, status);
     if (e == cudaSuccess) e = pdl_launch(ray_gj_elim_kernel, eg, dim3(128), 0, s, S, Bs, k, (const double2*)fcol);
     if (e != cudaSuccess) return e;
   }
-  return pdl_launch(ray_gj_unpermute_kernel, dim3(blocks_for(Bs, 128)), dim3(128), 0, s, S, Bs, (const int*)perm);
+  return pdl_launch(ray_gj_unpermute_kernel, dim3(blocks_for(Bs, 128), count), dim3(128), 0, s, S, Bs, (const int*)perm);
 }
 
-cudaError_t gemm(double2* C, const double2* A, const double2* Bm, int Bs, int acc, cudaStream_t s) {
-  const dim3 g(blocks_for(Bs, 32), blocks_for(Bs, 32));
-  return pdl_launch(ray_gemm_kernel, g, dim3(256), 0, s, C, A, Bm, Bs, acc);
+cudaError_t gemm(const GemmJobs& jobs, int count, int Bs, int acc, cudaStream_t s) {
+  const dim3 g(blocks_for(Bs, 32), blocks_for(Bs, 32), count);
+  return pdl_launch(ray_gemm_kernel, g, dim3(256), 0, s, jobs, Bs, acc);
 }
 
-cudaError_t gemv(double2* out, const double2* base, const double2* M, const double2* x, int Bs, int batch, double sgn,
-                 cudaStream_t s) {
-  return pdl_launch(ray_gemv_kernel, dim3(Bs, batch), dim3(GEMV_THREADS), 0, s, out, base, M, x, Bs, sgn);
+cudaError_t gemv(const GemvJobs& jobs, int count, int Bs, double sgn, cudaStream_t s) {
+  return pdl_launch(ray_gemv_kernel<false>, dim3(blocks_for(Bs, GEMV_WARPS), count), dim3(32 * GEMV_WARPS), 0, s, jobs,
+                    Bs, sgn);
 }
 
-// z = (block LU)^{-1} g; y is scratch of one vector.
+// z = (block LU)^{-1} g; y is scratch of one vector. Both ends move to the middle row, every row is
+// multiplied by its inverse, and the middle is carried back to both ends.
 cudaError_t block_substitute(const RayBlocks& B, double2* z, const double2* g, double2* y, cudaStream_t s) {
-  const int Bs = B.Bs, Nr = B.Nr;
+  const int Bs = B.Bs, Nr = B.Nr, mid = Nr / 2, up = Nr - 1 - mid;  // `up` rows above the middle
   const long long bs2 = (long long)Bs * Bs;
-  cudaError_t e = pdl_launch(ray_copy_kernel, dim3(blocks_for(Bs, 128)), dim3(128), 0, s, y, g, Bs);
-  for (int J = 1; J < Nr && e == cudaSuccess; ++J)
-    e = gemv(y + (long long)J * Bs, g + (long long)J * Bs, B.G + J * bs2, y + (long long)(J - 1) * Bs, Bs, 1, -1.0, s);
-  if (e == cudaSuccess) e = gemv(z, nullptr, B.Sinv, y, Bs, Nr, 1.0, s);
-  for (int J = Nr - 2; J >= 0 && e == cudaSuccess; --J)
-    e = gemv(z + (long long)J * Bs, z + (long long)J * Bs, B.W + J * bs2, z + (long long)(J + 1) * Bs, Bs, 1, -1.0, s);
+  auto at = [&](auto* v, int J) { return v + (long long)J * Bs; };
+  cudaError_t e = pdl_launch(ray_copy_kernel, dim3(blocks_for(Bs, 128), 2), dim3(128), 0, s, y, g, Bs, (Nr - 1) * Bs);
+  for (int k = 1; k < mid && e == cudaSuccess; ++k) {
+    const int J = k, T = Nr - 1 - k;  // y_J = g_J - G_J y_{J-1}, y_T = g_T - G_{T+1} y_{T+1}
+    GemvJobs j = {{{at(y, J), at(g, J), B.G + J * bs2, at(y, J - 1), nullptr, nullptr},
+                   {at(y, T), at(g, T), B.G + (T + 1) * bs2, at(y, T + 1), nullptr, nullptr}}};
+    e = gemv(j, k < up ? 2 : 1, Bs, -1.0, s);
+  }
+  if (e == cudaSuccess) {
+    GemvJobs j = {{{at(y, mid), at(g, mid), B.G + mid * bs2, at(y, mid - 1), up ? B.G + (mid + 1) * bs2 : nullptr,
+                    up ? at(y, mid + 1) : nullptr}, {}}};
+    e = gemv(j, 1, Bs, -1.0, s);
+  }
+  if (e == cudaSuccess) {
+    GemvJobs j = {{{z, nullptr, B.Sinv, y, nullptr, nullptr}, {}}};
+    e = pdl_launch(ray_gemv_kernel<true>, dim3(blocks_for(Bs, GEMV_WARPS), Nr), dim3(32 * GEMV_WARPS), 0, s, j, Bs, 1.0);
+  }
+  for (int k = 1; k <= mid && e == cudaSuccess; ++k) {
+    const int J = mid - k, T = mid + k;  // z_J -= W_J z_{J+1}, z_T -= W_T z_{T-1}
+    GemvJobs j = {{{at(z, J), at(z, J), B.W + J * bs2, at(z, J + 1), nullptr, nullptr},
+                   {at(z, T), at(z, T), B.W + T * bs2, at(z, T - 1), nullptr, nullptr}}};
+    e = gemv(j, k <= up ? 2 : 1, Bs, -1.0, s);
+  }
   return e;
 }
 
 }  // namespace
 
 cudaError_t ray_factor(const RayBlocks& B, cudaStream_t s) {
-  const int Bs = B.Bs, Nr = B.Nr;
+  const int Bs = B.Bs, Nr = B.Nr, mid = Nr / 2, up = Nr - 1 - mid;
   const long long bs2 = (long long)Bs * Bs;
+  auto blk = [&](double2* a, int J) { return a + J * bs2; };
+  // What row J's elimination adds towards the middle: below it W_J, then S_{J+1} -= L_{J+1} W_J and
+  // G_{J+1}; above it W_J, then S_{J-1} -= U_{J-1} W_J and the product in slot J.
+  auto w_of = [&](int J) {
+    return J < mid ? GemmJob{blk(B.W, J), blk(B.Sinv, J), blk(B.U, J)} : GemmJob{blk(B.W, J), blk(B.Sinv, J), blk(B.L, J)};
+  };
+  auto s_of = [&](int J) {
+    return J < mid ? GemmJob{blk(B.Sinv, J + 1), blk(B.L, J + 1), blk(B.W, J)}
+                   : GemmJob{blk(B.Sinv, J - 1), blk(B.U, J - 1), blk(B.W, J)};
+  };
+  auto g_of = [&](int J) {
+    return J < mid ? GemmJob{blk(B.G, J + 1), blk(B.L, J + 1), blk(B.Sinv, J)}
+                   : GemmJob{blk(B.G, J), blk(B.U, J - 1), blk(B.Sinv, J)};
+  };
   cudaError_t e = cudaMemcpyAsync(B.Sinv, B.D, sizeof(double2) * (size_t)(bs2 * Nr), cudaMemcpyDeviceToDevice, s);
-  if (e != cudaSuccess) return e;
-  e = gj_inverse(B.Sinv, Bs, B.fcol, B.perm, B.status, s);
-  if (e != cudaSuccess) return e;
-  for (int J = 1; J < Nr; ++J) {
-    double2* Sprev = B.Sinv + (J - 1) * bs2;
-    double2* Sj = B.Sinv + J * bs2;
-    if ((e = gemm(B.W + (J - 1) * bs2, Sprev, B.U + (J - 1) * bs2, Bs, 0, s)) != cudaSuccess) return e;
-    if ((e = gemm(Sj, B.L + J * bs2, B.W + (J - 1) * bs2, Bs, 1, s)) != cudaSuccess) return e;
-    if ((e = gemm(B.G + J * bs2, B.L + J * bs2, Sprev, Bs, 0, s)) != cudaSuccess) return e;
-    if ((e = gj_inverse(Sj, Bs, B.fcol, B.perm, B.status, s)) != cudaSuccess) return e;
+  for (int k = 0; k < mid && e == cudaSuccess; ++k) {
+    const int J = k, T = Nr - 1 - k, count = k < up ? 2 : 1;
+    e = gj_inverse(Pair{{blk(B.Sinv, J), blk(B.Sinv, T)}}, count, Bs, B.fcol, B.perm, B.status, s);
+    if (e == cudaSuccess) e = gemm(GemmJobs{{w_of(J), w_of(T)}}, count, Bs, 0, s);
+    if (e == cudaSuccess) e = gemm(GemmJobs{{g_of(J), g_of(T)}}, count, Bs, 0, s);
+    // both ends reach the middle row in the last steps: its two updates one after the other
+    if (e == cudaSuccess && count == 2 && J + 1 == T - 1) {
+      e = gemm(GemmJobs{{s_of(J), {}}}, 1, Bs, 1, s);
+      if (e == cudaSuccess) e = gemm(GemmJobs{{s_of(T), {}}}, 1, Bs, 1, s);
+    } else if (e == cudaSuccess) {
+      e = gemm(GemmJobs{{s_of(J), s_of(T)}}, count, Bs, 1, s);
+    }
   }
-  return cudaSuccess;
+  if (e == cudaSuccess) e = gj_inverse(Pair{{blk(B.Sinv, mid), nullptr}}, 1, Bs, B.fcol, B.perm, B.status, s);
+  return e;
 }
 
 cudaError_t ray_coarse_solve(const RayBlocks& B, double2* z, const double2* g, cudaStream_t s) {
