@@ -46,6 +46,7 @@ struct Level {
   int pk = 0;
   void* u = nullptr;  // working precision complex
   void* f = nullptr;  // working precision complex (levels >= 1)
+  double* inv = nullptr;  // FP64: stored reciprocals of the relaxation (Inst::inv), pitch `pitch`
   void* u2 = nullptr; // result of the fused post-smoothing pass (levels >= 1)
   int var_down = 0, var_up = 0;  // fused-pass variants (picked by the tile autotuner)
   int kform = 0;                 // hz_kacz_form of a Kaczmarz level (set up by plan_kaczmarz)
@@ -59,7 +60,7 @@ struct Plan {
   std::vector<int> n, pitch;
   size_t total = 0;
   // offsets
-  std::vector<size_t> off_kh, off_u, off_f, off_u2;
+  std::vector<size_t> off_kh, off_u, off_f, off_u2, off_inv;
   size_t off_kh64 = 0, off_d = 0, off_vec = 0, vec_bytes = 0, off_ainv = 0, off_work = 0, off_state = 0, off_partials = 0,
          off_hist = 0, off_status = 0, off_sync = 0, sync_bytes = 0;
   int nvec = 11;
@@ -105,6 +106,7 @@ bool make_plan(int n, const hz_hierarchy_opts& o, Plan* P, std::string* err) {
   P->off_u.assign(L, 0);
   P->off_f.assign(L, 0);
   P->off_u2.assign(L, 0);
+  P->off_inv.assign(L, 0);
   for (int l = 0; l < L; ++l) {
     int nl = n >> l;
     P->n[l] = nl;
@@ -114,6 +116,10 @@ bool make_plan(int n, const hz_hierarchy_opts& o, Plan* P, std::string* err) {
     if (l > 0 || P->fp32) {  // level 0 in FP64 reads the FP64 k h array directly
       P->off_kh[l] = off;
       off = align256(off + cells * re);
+    }
+    if (!P->fp32 && l < L - 1) {
+      P->off_inv[l] = off;
+      off = align256(off + cells * 8);
     }
     P->off_u[l] = off;
     off = align256(off + cells * ce * B);
@@ -327,6 +333,8 @@ const void* kh_of(const hz_problem* P, int l, int* pk) {
 // Launch instances: every right-hand side of the batch (solves) or instance 0 (step entry points).
 Inst inst_for(const hz_problem* P, int l, bool all) {
   Inst bi;
+  bi.inv = P->lv[l].inv;
+  bi.pi = P->lv[l].pitch;
   if (!all || P->plan.batch == 1) return bi;
   const Plan& pl = P->plan;
   bi.count = pl.batch;
@@ -1358,6 +1366,12 @@ hz_status hz_setup_hierarchy(hz_problem* P, const hz_hierarchy_opts* opts, void*
     L.u2 = (l > 0 || pl.off_u2[0]) ? (void*)(A + pl.off_u2[l]) : nullptr;
     int stride = 1 << l;
     if (L.kh) CK(launch_inject_kh(fp32, L.kh, L.pk, P->kh64, n, stride, L.n, (double)stride, s));
+    if (!fp32 && l < pl.levels - 1) {
+      L.inv = (double*)(A + pl.off_inv[l]);
+      int pk;
+      const double* kh = (const double*)kh_of(P, l, &pk);
+      CK(launch_level_inverse(L.inv, L.pitch, kh, pk, L.n, op_beta(P, L.relax_op), L.smoother == HZ_SMOOTH_KACZMARZ, s));
+    }
   }
   // Krylov vectors and scratch.
   KrylovVecs& k = P->kv;

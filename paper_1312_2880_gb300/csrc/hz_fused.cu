@@ -172,34 +172,24 @@ __device__ __forceinline__ void prolong_smooth_inner(O2* __restrict__ out, int p
   }
 }
 
-template <class T, class F2>
-__global__ void __launch_bounds__(FT) smooth_restrict_kernel(c2<T>* __restrict__ u, int pu, c2<T>* __restrict__ fc,
-                                                              int pc, const F2* __restrict__ f, int pf,
-                                                              const T* __restrict__ kh, int pk, int n, T bA, T bB,
-                                                              const int* __restrict__ stop, Inst bi) {
-  pdl_enter();
-  if (stop && stop[blockIdx.z * bi.stop_stride]) return;
-  u += blockIdx.z * bi.su;
-  fc += blockIdx.z * bi.sc;
-  f += blockIdx.z * bi.sf;
+// The general tile: every node tested against the grid (FP32 tiles at the boundary, all FP64 tiles).
+// KA, KB: kinds of the relaxation and residual diagonals (xr::DIAG_*).
+template <class T, class F2, int KA, int KB>
+__device__ __forceinline__ void smooth_restrict_body(c2<T>* __restrict__ u, int pu, c2<T>* __restrict__ fc, int pc,
+                                                     const F2* __restrict__ f, int pf, const T* __restrict__ kh,
+                                                     int pk, int n, T bA, T bB, const Inst& bi, c2<T>* su, c2<T>* sf,
+                                                     T* sk, int gx, int gy) {
   constexpr int W = TileShape<T>::W, HH = TileShape<T>::H;
   constexpr int RW = W + 5, RH = HH + 5, RN = RW * RH, HW = (RW + 1) / 2;
-  extern __shared__ __align__(16) unsigned char smem[];
-  c2<T>* su = reinterpret_cast<c2<T>*>(smem);
-  c2<T>* sf = su + RN;
-  T* sk = reinterpret_cast<T*>(sf + RN);
-  const int x0 = blockIdx.x * W, y0 = blockIdx.y * HH;
-  const int gx = x0 - 3, gy = y0 - 3;
-  if (interior_path<T>() && gx >= 1 && gy >= 1 && gx + RW <= n && gy + RH <= n) {
-    smooth_restrict_inner<T, F2>(u, pu, fc, pc, f, pf, kh, pk, bA, bB, su, sf, sk, gx, gy);
-    return;
-  }
+  T* si = sk + (sizeof(T) == 8 ? RN : 0);  // FP64: the stored 1 / |d|^2
+  const int x0 = gx + 3, y0 = gy + 3;
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
   for (int q = tid; q < RN; q += FT) {
     int r = q / RW, c = q - r * RW, i = gx + c, j = gy + r;
     if (in_grid(i, j, n)) {
       sf[q] = ldc<T>(f, (long long)j * pf + i);
       sk[q] = kh[(long long)j * pk + i];
+      if constexpr (sizeof(T) == 8) si[q] = bi.inv[(long long)j * bi.pi + i];
     }
   }
   __syncthreads();
@@ -210,8 +200,8 @@ __global__ void __launch_bounds__(FT) smooth_restrict_kernel(c2<T>* __restrict__
     int c = 2 * m + ((0 - gx - j) & 1);
     int i = gx + c;
     if (c < RW && in_grid(i, j, n)) {
-      int sides = (i == 0) + (i == n) + (j == 0) + (j == n);
-      su[r * RW + c] = xr::cdiv<T>(sf[r * RW + c], xr::diag<T>(sk[r * RW + c], sides, bA));
+      const T sides2 = (T)(2 * ((i == 0) + (i == n) + (j == 0) + (j == n)));
+      su[r * RW + c] = xr::cdiv_k<T, KA>(sf[r * RW + c], xr::diag_k<T, KA>(sk[r * RW + c], sides2, bA), si[r * RW + c]);
     }
   }
   __syncthreads();
@@ -224,7 +214,7 @@ __global__ void __launch_bounds__(FT) smooth_restrict_kernel(c2<T>* __restrict__
     if (r >= 1 && r <= RH - 2 && c >= 1 && c <= RW - 2 && in_grid(i, j, n)) {
       Nbr b = neighbours(i, j, n);
       c2<T> s = nb_sum<T>(su, RW, c, r, i, j, n, gx, gy);
-      su[r * RW + c] = xr::gs<T>(sf[r * RW + c], s, xr::diag<T>(sk[r * RW + c], b.sides, bA));
+      su[r * RW + c] = xr::gs_k<T, KA>(sf[r * RW + c], s, xr::diag_k<T, KA>(sk[r * RW + c], (T)(2 * b.sides), bA), si[r * RW + c]);
     }
   }
   __syncthreads();
@@ -240,7 +230,7 @@ __global__ void __launch_bounds__(FT) smooth_restrict_kernel(c2<T>* __restrict__
     if (r >= 2 && r <= RH - 3 && c >= 2 && c <= RW - 3 && in_grid(i, j, n)) {
       Nbr b = neighbours(i, j, n);
       c2<T> s = nb_sum<T>(su, RW, c, r, i, j, n, gx, gy);
-      sf[q] = xr::resid<T>(sf[q], su[q], s, xr::diag<T>(sk[q], b.sides, bB));
+      sf[q] = xr::resid_k<T, KB>(sf[q], su[q], s, xr::diag_k<T, KB>(sk[q], (T)(2 * b.sides), bB));
     }
   }
   __syncthreads();
@@ -253,36 +243,22 @@ __global__ void __launch_bounds__(FT) smooth_restrict_kernel(c2<T>* __restrict__
   }
 }
 
-template <class T, class F2, class O2>
-__global__ void __launch_bounds__(FT) prolong_smooth_kernel(O2* __restrict__ out, int po, const c2<T>* __restrict__ upre,
-                                                             int pu, const c2<T>* __restrict__ ec, int pc,
-                                                             const F2* __restrict__ f, int pf,
-                                                             const T* __restrict__ kh, int pk, int n, T bA,
-                                                             const int* __restrict__ stop, Inst bi) {
-  pdl_enter();
-  if (stop && stop[blockIdx.z * bi.stop_stride]) return;
-  out += blockIdx.z * bi.so;
-  upre += blockIdx.z * bi.su;
-  ec += blockIdx.z * bi.sc;
-  f += blockIdx.z * bi.sf;
+template <class T, class F2, class O2, int KA>
+__device__ __forceinline__ void prolong_smooth_body(O2* __restrict__ out, int po, const c2<T>* __restrict__ upre,
+                                                    int pu, const c2<T>* __restrict__ ec, int pc,
+                                                    const F2* __restrict__ f, int pf, const T* __restrict__ kh, int pk,
+                                                    int n, T bA, const Inst& bi, c2<T>* su, c2<T>* sf, T* sk, int gx,
+                                                    int gy) {
   constexpr int W = TileShape<T>::W, HH = TileShape<T>::H;
   constexpr int RW = W + 4, RH = HH + 4, RN = RW * RH, HW = RW / 2;
-  extern __shared__ __align__(16) unsigned char smem[];
-  c2<T>* su = reinterpret_cast<c2<T>*>(smem);
-  c2<T>* sf = su + RN;
-  T* sk = reinterpret_cast<T*>(sf + RN);
-  const int x0 = blockIdx.x * W, y0 = blockIdx.y * HH;
-  const int gx = x0 - 2, gy = y0 - 2;
-  if (interior_path<T>() && gx >= 1 && gy >= 1 && gx + RW <= n && gy + RH <= n) {
-    prolong_smooth_inner<T, F2, O2>(out, po, upre, pu, ec, pc, f, pf, kh, pk, bA, su, sf, sk, gx, gy);
-    return;
-  }
+  T* si = sk + (sizeof(T) == 8 ? RN : 0);  // FP64: the stored 1 / |d|^2
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
   for (int q = tid; q < RN; q += FT) {
     int r = q / RW, c = q - r * RW, i = gx + c, j = gy + r;
     if (in_grid(i, j, n)) {
       sf[q] = ldc<T>(f, (long long)j * pf + i);
       sk[q] = kh[(long long)j * pk + i];
+      if constexpr (sizeof(T) == 8) si[q] = bi.inv[(long long)j * bi.pi + i];
     }
   }
   // u_pre + P e, one parity class (i mod 2, j mod 2) after the other (gx and gy are even), so that
@@ -311,7 +287,7 @@ __global__ void __launch_bounds__(FT) prolong_smooth_kernel(O2* __restrict__ out
     if (r >= 1 && r <= RH - 2 && c >= 1 && c <= RW - 2 && in_grid(i, j, n)) {
       Nbr b = neighbours(i, j, n);
       c2<T> s = nb_sum<T>(su, RW, c, r, i, j, n, gx, gy);
-      su[r * RW + c] = xr::gs<T>(sf[r * RW + c], s, xr::diag<T>(sk[r * RW + c], b.sides, bA));
+      su[r * RW + c] = xr::gs_k<T, KA>(sf[r * RW + c], s, xr::diag_k<T, KA>(sk[r * RW + c], (T)(2 * b.sides), bA), si[r * RW + c]);
     }
   }
   __syncthreads();
@@ -324,7 +300,7 @@ __global__ void __launch_bounds__(FT) prolong_smooth_kernel(O2* __restrict__ out
     if (r >= 2 && r < 2 + HH && c >= 2 && c < 2 + W && in_grid(i, j, n)) {
       Nbr b = neighbours(i, j, n);
       c2<T> s = nb_sum<T>(su, RW, c, r, i, j, n, gx, gy);
-      su[r * RW + c] = xr::gs<T>(sf[r * RW + c], s, xr::diag<T>(sk[r * RW + c], b.sides, bA));
+      su[r * RW + c] = xr::gs_k<T, KA>(sf[r * RW + c], s, xr::diag_k<T, KA>(sk[r * RW + c], (T)(2 * b.sides), bA), si[r * RW + c]);
     }
   }
   __syncthreads();
@@ -334,13 +310,85 @@ __global__ void __launch_bounds__(FT) prolong_smooth_kernel(O2* __restrict__ out
   }
 }
 
+template <class T, class F2>
+__global__ void __launch_bounds__(FT) smooth_restrict_kernel(c2<T>* __restrict__ u, int pu, c2<T>* __restrict__ fc,
+                                                              int pc, const F2* __restrict__ f, int pf,
+                                                              const T* __restrict__ kh, int pk, int n, T bA, T bB,
+                                                              const int* __restrict__ stop, Inst bi) {
+  pdl_enter();
+  if (stop && stop[blockIdx.z * bi.stop_stride]) return;
+  u += blockIdx.z * bi.su;
+  fc += blockIdx.z * bi.sc;
+  f += blockIdx.z * bi.sf;
+  constexpr int W = TileShape<T>::W, HH = TileShape<T>::H;
+  constexpr int RW = W + 5, RH = HH + 5, RN = RW * RH;
+  extern __shared__ __align__(16) unsigned char smem[];
+  c2<T>* su = reinterpret_cast<c2<T>*>(smem);
+  c2<T>* sf = su + RN;
+  T* sk = reinterpret_cast<T*>(sf + RN);
+  const int x0 = blockIdx.x * W, y0 = blockIdx.y * HH;
+  const int gx = x0 - 3, gy = y0 - 3;
+  if (interior_path<T>() && gx >= 1 && gy >= 1 && gx + RW <= n && gy + RH <= n) {
+    smooth_restrict_inner<T, F2>(u, pu, fc, pc, f, pf, kh, pk, bA, bB, su, sf, sk, gx, gy);
+    return;
+  }
+  if constexpr (sizeof(T) == 8) {
+    if (gx >= 1 && gy >= 1 && gx + RW <= n && gy + RH <= n) {  // every node strictly inside the square
+      if (bA == (T)0 && bB == (T)0)
+        smooth_restrict_body<T, F2, xr::DIAG_REAL, xr::DIAG_REAL>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, bi, su, sf, sk, gx, gy);
+      else if (bB == (T)0)
+        smooth_restrict_body<T, F2, xr::DIAG_INNER, xr::DIAG_REAL>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, bi, su, sf, sk, gx, gy);
+      else
+        smooth_restrict_body<T, F2, xr::DIAG_INNER, xr::DIAG_INNER>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, bi, su, sf, sk, gx, gy);
+      return;
+    }
+  }
+  smooth_restrict_body<T, F2, xr::DIAG_ANY, xr::DIAG_ANY>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, bi, su, sf, sk, gx, gy);
+}
+
+template <class T, class F2, class O2>
+__global__ void __launch_bounds__(FT) prolong_smooth_kernel(O2* __restrict__ out, int po, const c2<T>* __restrict__ upre,
+                                                             int pu, const c2<T>* __restrict__ ec, int pc,
+                                                             const F2* __restrict__ f, int pf,
+                                                             const T* __restrict__ kh, int pk, int n, T bA,
+                                                             const int* __restrict__ stop, Inst bi) {
+  pdl_enter();
+  if (stop && stop[blockIdx.z * bi.stop_stride]) return;
+  out += blockIdx.z * bi.so;
+  upre += blockIdx.z * bi.su;
+  ec += blockIdx.z * bi.sc;
+  f += blockIdx.z * bi.sf;
+  constexpr int W = TileShape<T>::W, HH = TileShape<T>::H;
+  constexpr int RW = W + 4, RH = HH + 4, RN = RW * RH;
+  extern __shared__ __align__(16) unsigned char smem[];
+  c2<T>* su = reinterpret_cast<c2<T>*>(smem);
+  c2<T>* sf = su + RN;
+  T* sk = reinterpret_cast<T*>(sf + RN);
+  const int x0 = blockIdx.x * W, y0 = blockIdx.y * HH;
+  const int gx = x0 - 2, gy = y0 - 2;
+  if (interior_path<T>() && gx >= 1 && gy >= 1 && gx + RW <= n && gy + RH <= n) {
+    prolong_smooth_inner<T, F2, O2>(out, po, upre, pu, ec, pc, f, pf, kh, pk, bA, su, sf, sk, gx, gy);
+    return;
+  }
+  if constexpr (sizeof(T) == 8) {
+    if (gx >= 1 && gy >= 1 && gx + RW <= n && gy + RH <= n) {
+      if (bA == (T)0)
+        prolong_smooth_body<T, F2, O2, xr::DIAG_REAL>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, bi, su, sf, sk, gx, gy);
+      else
+        prolong_smooth_body<T, F2, O2, xr::DIAG_INNER>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, bi, su, sf, sk, gx, gy);
+      return;
+    }
+  }
+  prolong_smooth_body<T, F2, O2, xr::DIAG_ANY>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, bi, su, sf, sk, gx, gy);
+}
+
 template <class T>
 constexpr size_t sr_smem() {
-  return (size_t)(TileShape<T>::W + 5) * (TileShape<T>::H + 5) * (2 * sizeof(c2<T>) + sizeof(T));
+  return (size_t)(TileShape<T>::W + 5) * (TileShape<T>::H + 5) * (2 * sizeof(c2<T>) + (sizeof(T) == 8 ? 2 : 1) * sizeof(T));
 }
 template <class T>
 constexpr size_t ps_smem() {
-  return (size_t)(TileShape<T>::W + 4) * (TileShape<T>::H + 4) * (2 * sizeof(c2<T>) + sizeof(T));
+  return (size_t)(TileShape<T>::W + 4) * (TileShape<T>::H + 4) * (2 * sizeof(c2<T>) + (sizeof(T) == 8 ? 2 : 1) * sizeof(T));
 }
 
 template <class T, class F2>

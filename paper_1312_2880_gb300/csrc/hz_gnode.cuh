@@ -15,11 +15,17 @@ namespace gnode {
 // boundary carries coefficient 2 and receives 2 delta.
 template <class T, class F2>
 __device__ __forceinline__ void kacz_row(c2<T>* __restrict__ u, int pu, const F2* __restrict__ f, int pf,
-                                         const T* __restrict__ kh, int pk, int n, int i, int j, T beta) {
+                                         const T* __restrict__ kh, int pk, int n, int i, int j, T beta,
+                                         const double* __restrict__ stored = nullptr, int pi = 0) {
   const Nbr b = neighbours(i, j, n);
   c2<T> d;
   T inv;
-  lvl::row_consts<T>(kh[(long long)j * pk + i], i, j, n, beta, &d, &inv);
+  if (sizeof(T) == 8 && stored) {
+    d = xr::diag<T>(kh[(long long)j * pk + i], lvl::sides_at(i, j, n), beta);
+    inv = (T)stored[(long long)j * pi + i];
+  } else {
+    lvl::row_consts<T>(kh[(long long)j * pk + i], i, j, n, beta, &d, &inv);
+  }
   c2<T>* row = u + (long long)j * pu;
   lvl::act_nodes<T>(row + i, row + b.iw, row + b.ie, u + (long long)b.js * pu + i, u + (long long)b.jn * pu + i,
                     ldc<T>(f, (long long)j * pf + i), d, inv);

@@ -38,6 +38,10 @@ struct Inst {
   int count = 1;
   long long su = 0, sf = 0, sc = 0, so = 0;
   int stop_stride = 0;
+  // FP64 levels: the reciprocals that relaxation needs at every node, stored once per problem (pitch
+  // pi): 1 / |d|^2 on Gauss-Seidel levels, 1 / |a_p|^2 (lvl::row_consts) on Kaczmarz levels.
+  const double* inv = nullptr;
+  int pi = 0;
 };
 
 // ---------------------------------------------------------------- V-cycle kernel launchers
@@ -164,6 +168,9 @@ cudaError_t launch_export(bool fp32, double2* dst, int pd, const void* src, int 
                           const int* stop, cudaStream_t s);
 cudaError_t launch_inject_kh(bool fp32, void* kh, int pk, const double* k0, int n0, int stride, int nl, double H,
                              cudaStream_t s);
+// The reciprocals of Inst::inv on an FP64 level.
+cudaError_t launch_level_inverse(double* inv, int pi, const double* kh, int pk, int n, double beta, bool kaczmarz,
+                                 cudaStream_t s);
 // Dense inverse of the coarsest scaled operator, stored transposed in the working precision.
 // work: 2 * m * m double2 scratch, m = (nc+1)^2. status: device int, 0 on success, 1 if singular.
 cudaError_t launch_coarse_setup(bool fp32, void* ainvT, double2* work, const void* kh, int pk, int nc, double beta,

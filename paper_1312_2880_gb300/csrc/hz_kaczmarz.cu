@@ -45,7 +45,7 @@ struct TileGeo {
   static constexpr int RX = KT_ + 2 * HX, RY = KT_ + HN + HF, REG = RX * RY;
 };
 using TileOne = TileGeo<32, 1, 256>;  // one sweep per launch: 44 x 48 regions
-constexpr size_t tile_smem() { return (size_t)TileOne::REG * (2 * sizeof(double2) + sizeof(double)); }
+constexpr size_t tile_smem() { return (size_t)TileOne::REG * (2 * sizeof(double2) + 2 * sizeof(double)); }
 
 // Actions of phase ph (of P = 5S; R = P - 1 - ph phases follow it) that can still reach the
 // tile's outputs. Propagating dependencies back from the outputs through the colour phases on an
@@ -87,12 +87,11 @@ __device__ __forceinline__ int mod5(int x) { return ((x % 5) + 5) % 5; }
 
 // Phase PH of a tile: each thread takes up to two slots, reads both supports before updating
 // either (same-colour supports are disjoint), then writes both back. The row constants come from
-// k H as in the whole-level forms (lvl::row_consts; strictly inside the square, no boundary term)
-// and the arithmetic is lvl::act_update, so a tiled sweep gives the same bits as the whole-level
+// k H and the stored 1 / |a_p|^2 (the values of lvl::row_consts) and the arithmetic is lvl::act_update, so a tiled sweep gives the same bits as the whole-level
 // and cluster forms.
 template <class T, class G, bool POST, bool INNER, int PH>
-__device__ __forceinline__ void tile_phase(c2<T>* su, const c2<T>* sf, const T* sk, const unsigned char* c0row,
-                                           int gx, int gy, int n, T beta) {
+__device__ __forceinline__ void tile_phase(c2<T>* su, const c2<T>* sf, const T* sk, const T* si,
+                                           const unsigned char* c0row, int gx, int gy, int n, T beta) {
   using PR = PhaseRect<G, POST>;
   constexpr int colour = POST ? 4 - PH % 5 : PH % 5;
   constexpr int xlo = PR::xlo(PH), xhi = PR::xhi(PH), ylo = PR::ylo(PH), per = PR::per(PH), slots = PR::slots(PH);
@@ -128,7 +127,7 @@ __device__ __forceinline__ void tile_phase(c2<T>* su, const c2<T>* sf, const T* 
       A.on = p + (A.j < n ? W : -W);
     }
   }
-  T kh[NS];
+  T kh[NS], inv[NS];
 #pragma unroll
   for (int s = 0; s < NS; ++s) {
     TileAct<T>& A = a[s];
@@ -140,21 +139,15 @@ __device__ __forceinline__ void tile_phase(c2<T>* su, const c2<T>* sf, const T* 
       A.un = su[A.on];
       A.f = sf[A.op];
       kh[s] = sk[A.op];
+      inv[s] = si[A.op];
     }
   }
 #pragma unroll
   for (int s = 0; s < NS; ++s) {
     TileAct<T>& A = a[s];
     if (A.ok) {
-      c2<T> d;
-      T inv;
-      if constexpr (INNER) {
-        d = xr::diag<T>(kh[s], 0, beta);
-        inv = xr::rcp(xr::add(xr::cabs2<T>(d), (T)4));
-      } else {
-        lvl::row_consts<T>(kh[s], A.i, A.j, n, beta, &d, &inv);
-      }
-      lvl::act_update<T>(A.up, A.uw, A.ue, A.us, A.un, A.f, d, inv, A.mx, A.my);
+      const c2<T> d = xr::diag<T>(kh[s], INNER ? 0 : lvl::sides_at(A.i, A.j, n), beta);
+      lvl::act_update<T>(A.up, A.uw, A.ue, A.us, A.un, A.f, d, inv[s], A.mx, A.my);
     }
   }
 #pragma unroll
@@ -172,9 +165,9 @@ __device__ __forceinline__ void tile_phase(c2<T>* su, const c2<T>* sf, const T* 
 
 // All phases of a launch in order, a barrier after each.
 template <class T, class G, bool POST, bool INNER, int... PH>
-__device__ __forceinline__ void tile_phases(c2<T>* su, const c2<T>* sf, const T* sk, const unsigned char* c0row,
-                                            int gx, int gy, int n, T beta, std::integer_sequence<int, PH...>) {
-  ((tile_phase<T, G, POST, INNER, PH>(su, sf, sk, c0row, gx, gy, n, beta), __syncthreads()), ...);
+__device__ __forceinline__ void tile_phases(c2<T>* su, const c2<T>* sf, const T* sk, const T* si,
+                                            const unsigned char* c0row, int gx, int gy, int n, T beta, std::integer_sequence<int, PH...>) {
+  ((tile_phase<T, G, POST, INNER, PH>(su, sf, sk, si, c0row, gx, gy, n, beta), __syncthreads()), ...);
 }
 
 // ------------------------------------------------------------------ whole level in one block
@@ -302,6 +295,7 @@ __global__ void __launch_bounds__(TileOne::TBK) kacz_sweep_tile64_kernel(double2
   c2<T>* su = reinterpret_cast<c2<T>*>(smem);
   c2<T>* sf = su + REG;
   T* sk = reinterpret_cast<T*>(sf + REG);
+  T* si = sk + REG;  // the stored 1 / |a_p|^2
   __shared__ unsigned char c0row[RY];  // column residue of colour 0 in each region row
   const int x0 = blockIdx.x * KT, y0 = blockIdx.y * KT;
   // sweeps in the order 0..4 (pre) need the near halo below the tile, 4..0 (post) above it
@@ -325,6 +319,7 @@ __global__ void __launch_bounds__(TileOne::TBK) kacz_sweep_tile64_kernel(double2
         su[q] = mk<T>(0, 0);
       lvl::cp_async<sizeof(c2<T>)>(sf + q, f + jf + i);
       lvl::cp_async<sizeof(T)>(sk + q, kh + jk + i);
+      lvl::cp_async<sizeof(T)>(si + q, bi.inv + (long long)j * bi.pi + i);
     }
   }
   for (int r = threadIdx.x; r < RY; r += TBK) c0row[r] = (unsigned char)mod5(-2 * (gy + r) - gx);
@@ -335,9 +330,9 @@ __global__ void __launch_bounds__(TileOne::TBK) kacz_sweep_tile64_kernel(double2
   const bool inner = gx + PR::xlo(0) >= 1 && gx + PR::xhi(0) <= n - 1 && gy + PR::ylo(0) >= 1 &&
                      gy + PR::yhi(0) <= n - 1;
   if (inner)
-    tile_phases<T, G, POST, true>(su, sf, sk, c0row, gx, gy, n, bA, std::make_integer_sequence<int, PR::P>{});
+    tile_phases<T, G, POST, true>(su, sf, sk, si, c0row, gx, gy, n, bA, std::make_integer_sequence<int, PR::P>{});
   else
-    tile_phases<T, G, POST, false>(su, sf, sk, c0row, gx, gy, n, bA, std::make_integer_sequence<int, PR::P>{});
+    tile_phases<T, G, POST, false>(su, sf, sk, si, c0row, gx, gy, n, bA, std::make_integer_sequence<int, PR::P>{});
   // the tile's own KT x KT nodes (those inside the square) back to global memory, rows by warp
   for (int r = below + warp; r < below + KT; r += NW) {
     const int j = gy + r;
@@ -452,6 +447,18 @@ struct ClusterLevel {
   }
 };
 
+// Row constants of a band's node: in FP64 the reciprocal is read (it is half of their instructions).
+template <class T>
+__device__ __forceinline__ void cluster_consts(const ClusterLevel<T>& L, int q, T kh, int i, int j, int n, T bA,
+                                               const Inst& bi) {
+  if (sizeof(T) == 8 && bi.inv) {
+    L.sd[q] = xr::diag<T>(kh, lvl::sides_at(i, j, n), bA);
+    L.sinv[q] = (T)bi.inv[(long long)j * bi.pi + i];
+  } else {
+    lvl::row_consts<T>(kh, i, j, n, bA, &L.sd[q], &L.sinv[q]);
+  }
+}
+
 template <class T>
 __device__ __forceinline__ void cluster_act(cgx::cluster_group& cl, const ClusterLevel<T>& L, int i, int j) {
   const int n = L.n;
@@ -502,7 +509,7 @@ __global__ void __launch_bounds__(KC_THREADS) kacz_cluster_pre_kernel(c2<T>* __r
     const int j = L.r0 + q / w, i = q % w;
     L.su[q] = mk<T>(0, 0);
     L.sf[q] = f[(long long)j * pf + i];
-    lvl::row_consts<T>(kh[(long long)j * pk + i], i, j, n, bA, &L.sd[q], &L.sinv[q]);
+    cluster_consts<T>(L, q, kh[(long long)j * pk + i], i, j, n, bA, bi);
   }
   cl.sync();
   cluster_sweeps<T>(cl, L, nu, false);
@@ -554,7 +561,7 @@ __global__ void __launch_bounds__(KC_THREADS) kacz_cluster_post_kernel(c2<T>* __
     const c2<T>* e0 = ec + (long long)(j >> 1) * pc;
     L.su[q] = xr::cadd<T>(u[(long long)j * pu + i], xr::bilinear<T>(e0, e0 + pc, i >> 1, i & 1, j & 1));
     L.sf[q] = f[(long long)j * pf + i];
-    lvl::row_consts<T>(kh[(long long)j * pk + i], i, j, n, bA, &L.sd[q], &L.sinv[q]);
+    cluster_consts<T>(L, q, kh[(long long)j * pk + i], i, j, n, bA, bi);
   }
   cl.sync();
   cluster_sweeps<T>(cl, L, nu, true);

@@ -60,8 +60,13 @@ template <class T>
 __device__ __forceinline__ c2<T> add2(c2<T> a, c2<T> b) { return xr::cadd<T>(a, b); }
 template <class T>
 __device__ __forceinline__ c2<T> scl2(c2<T> a, T s) { return xr::cscale<T>(a, s); }
-template <class T>
-__device__ __forceinline__ c2<T> diag(T k, T two_sides, T beta) { return xr::diag2<T>(k, two_sides, beta); }
+// What a strip's code knows about its nodes: EDGE, columns mirrored at the grid's edge; and the kinds
+// (xr::DIAG_*) of the relaxation and the residual diagonals.
+template <bool EDGE_, int KA_, int KB_>
+struct Mode {
+  static constexpr bool EDGE = EDGE_;
+  static constexpr int KA = KA_, KB = KB_;
+};
 
 // ------------------------------------------------------------------ per-lane async copies
 __device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
@@ -174,8 +179,11 @@ template <class T> __host__ __device__ constexpr int kpair_bytes() { return 2 * 
 //   full-weighting row sum (coarse row J completes at fine row 2J + 1).
 constexpr int SR_W = 58;
 constexpr int SR_R = 8;            // row slots per warp
-// bytes per slot: f pairs (16 B per lane in FP32, 32 in FP64), then k pairs (8, 16)
-template <class Real> __host__ __device__ constexpr int sr_slot() { return 32 * (pair_bytes<Real>() + kpair_bytes<Real>()); }
+// bytes per slot: f pairs (16 B per lane in FP32, 32 in FP64), then k pairs (8, 16), in FP64 then the
+// stored 1 / |d|^2 pairs (16)
+template <class Real> __host__ __device__ constexpr int ipair_bytes() { return sizeof(Real) == 8 ? 16 : 0; }
+template <class Real> __host__ __device__ constexpr int sr_inv_off() { return 32 * (pair_bytes<Real>() + kpair_bytes<Real>()); }
+template <class Real> __host__ __device__ constexpr int sr_slot() { return sr_inv_off<Real>() + 32 * ipair_bytes<Real>(); }
 
 template <class Real>
 struct SRArgs {
@@ -189,6 +197,8 @@ struct SRArgs {
   int pk;
   int n;
   Real bA, bB;
+  const double* inv;
+  int pi;
 };
 
 template <class Real>
@@ -208,13 +218,18 @@ __device__ __forceinline__ void sr_issue(unsigned char* ring, const SRArgs<Real>
                               q.m0, q.m1);
     copy_kpair<Real, EDGE>(smem_addr(slot + 32 * pair_bytes<Real>() + kpair_bytes<Real>() * threadIdx.x),
                            A.kh + (long long)mj * A.pk, q.c0, q.m0, q.m1);
+    if constexpr (sizeof(Real) == 8)
+      copy_kpair<Real, EDGE>(smem_addr(slot + sr_inv_off<Real>() + ipair_bytes<Real>() * threadIdx.x),
+                             A.inv + (long long)mj * A.pi, q.c0, q.m0, q.m1);
   }
   cp_commit();  // one group per row index, empty past the segment, so the wait count stays fixed
 }
 
-template <class Real, int Q, bool EDGE, bool VF>
+template <class Real, int Q, class M, bool VF>
 __device__ __forceinline__ void sr_stage(SRState<Real>& S, unsigned char* ring, const SRArgs<Real>& A, int t, int T, int y0,
                                          int row_end, int gx, const Lane<Real>& q) {
+  constexpr bool EDGE = M::EDGE;
+  constexpr int KA = M::KA, KB = M::KB;
   if (t >= T) return;
   cp_wait<SR_R - 2>();  // rows up to t have landed (t + R - 1 groups committed)
   {
@@ -225,13 +240,19 @@ __device__ __forceinline__ void sr_stage(SRState<Real>& S, unsigned char* ring, 
   // global row y0 - 3 + t has the parity of t + 1: red is column 0 of the pair on odd t
   constexpr int er = (Q & 1) ? 0 : 1;
   const int j0 = y0 - 3 + t;
+  // stored reciprocal of this lane's column c in row t or t - 1 (both slots are still filled)
+  auto inv = [&](int row, int c) -> Real {
+    if constexpr (sizeof(Real) == 8)
+      return reinterpret_cast<const Real*>(ring + (row % SR_R) * sr_slot<Real>() + sr_inv_off<Real>())[2 * threadIdx.x + c];
+    return (Real)0;
+  };
   {  // red at row t (zero guess)
     L2c<Real>& U = S.U[Q];
     const Real rs = sides2<Real>(j0, A.n);
     if (er == 0)
-      U.a = xr::cdiv<Real>(S.F[Q].a, diag<Real>(S.K[Q].x, q.sc0 + rs, A.bA));
+      U.a = xr::cdiv_k<Real, KA>(S.F[Q].a, xr::diag_k<Real, KA>(S.K[Q].x, q.sc0 + rs, A.bA), inv(t, 0));
     else
-      U.b = xr::cdiv<Real>(S.F[Q].b, diag<Real>(S.K[Q].y, q.sc1 + rs, A.bA));
+      U.b = xr::cdiv_k<Real, KA>(S.F[Q].b, xr::diag_k<Real, KA>(S.K[Q].y, q.sc1 + rs, A.bA), inv(t, 1));
   }
   if (t >= 1) {  // black at row t-1, column er
     constexpr int q1 = (Q + 3) & 3, q2 = (Q + 2) & 3;
@@ -239,10 +260,10 @@ __device__ __forceinline__ void sr_stage(SRState<Real>& S, unsigned char* ring, 
     L2c<Real>& U = S.U[q1];
     if (er == 1) {
       const c2<Real> nb = xr::nb4<Real>(U.a, shfl_down2<Real>(U.a), S.U[q2].b, S.U[Q].b);
-      U.b = xr::gs<Real>(S.F[q1].b, nb, diag<Real>(S.K[q1].y, q.sc1 + rs, A.bA));
+      U.b = xr::gs_k<Real, KA>(S.F[q1].b, nb, xr::diag_k<Real, KA>(S.K[q1].y, q.sc1 + rs, A.bA), inv(t - 1, 1));
     } else {
       const c2<Real> nb = xr::nb4<Real>(shfl_up2<Real>(U.b), U.b, S.U[q2].a, S.U[Q].a);
-      U.a = xr::gs<Real>(S.F[q1].a, nb, diag<Real>(S.K[q1].x, q.sc0 + rs, A.bA));
+      U.a = xr::gs_k<Real, KA>(S.F[q1].a, nb, xr::diag_k<Real, KA>(S.K[q1].x, q.sc0 + rs, A.bA), inv(t - 1, 0));
     }
     const int jo = j0 - 1;
     if (jo >= y0 && jo < row_end) store_pair<Real, true>(A.u + (long long)jo * A.pu, q.c0, gx + 4, min(gx + 61, A.n), U);
@@ -252,10 +273,10 @@ __device__ __forceinline__ void sr_stage(SRState<Real>& S, unsigned char* ring, 
     const Real rs = sides2<Real>(j0 - 2, A.n);
     const L2c<Real>& U = S.U[q2];
     L2c<Real> R;
-    R.a = xr::resid<Real>(S.F[q2].a, U.a, xr::nb4<Real>(shfl_up2<Real>(U.b), U.b, S.U[q3].a, S.U[q1].a),
-                           diag<Real>(S.K[q2].x, q.sc0 + rs, A.bB));
-    R.b = xr::resid<Real>(S.F[q2].b, U.b, xr::nb4<Real>(U.a, shfl_down2<Real>(U.a), S.U[q3].b, S.U[q1].b),
-                           diag<Real>(S.K[q2].y, q.sc1 + rs, A.bB));
+    R.a = xr::resid_k<Real, KB>(S.F[q2].a, U.a, xr::nb4<Real>(shfl_up2<Real>(U.b), U.b, S.U[q3].a, S.U[q1].a),
+                           xr::diag_k<Real, KB>(S.K[q2].x, q.sc0 + rs, A.bB));
+    R.b = xr::resid_k<Real, KB>(S.F[q2].b, U.b, xr::nb4<Real>(U.a, shfl_down2<Real>(U.a), S.U[q3].b, S.U[q1].b),
+                           xr::diag_k<Real, KB>(S.K[q2].y, q.sc1 + rs, A.bB));
     // the row sum (w + e) + 2 c at this lane's coarse column (2I = c0), then across rows; row
     // j0 - 2 is even (2J) on odd t, odd (2J + 1) on even t
     const c2<Real> h = xr::fw3<Real>(shfl_up2<Real>(R.b), R.a, R.b);
@@ -275,8 +296,9 @@ __device__ __forceinline__ void sr_stage(SRState<Real>& S, unsigned char* ring, 
   sr_issue<Real, EDGE, VF>(ring, A, t + SR_R - 1, T, y0, q);
 }
 
-template <class Real, bool EDGE, bool VF>
+template <class Real, class M, bool VF>
 __device__ __forceinline__ void sr_run(unsigned char* ring, const SRArgs<Real>& A, int gx, int y0, int row_end) {
+  constexpr bool EDGE = M::EDGE;
   const Lane<Real> q = lane_of<Real>(gx, A.n);
   const int T = row_end - y0 + 6;
   SRState<Real> S;
@@ -288,10 +310,10 @@ __device__ __forceinline__ void sr_run(unsigned char* ring, const SRArgs<Real>& 
   // t mod 4), so no register moves rotate the windows between iterations
 #pragma unroll 1
   for (int t0 = 0; t0 < T; t0 += 4) {
-    sr_stage<Real, 0, EDGE, VF>(S, ring, A, t0 + 0, T, y0, row_end, gx, q);
-    sr_stage<Real, 1, EDGE, VF>(S, ring, A, t0 + 1, T, y0, row_end, gx, q);
-    sr_stage<Real, 2, EDGE, VF>(S, ring, A, t0 + 2, T, y0, row_end, gx, q);
-    sr_stage<Real, 3, EDGE, VF>(S, ring, A, t0 + 3, T, y0, row_end, gx, q);
+    sr_stage<Real, 0, M, VF>(S, ring, A, t0 + 0, T, y0, row_end, gx, q);
+    sr_stage<Real, 1, M, VF>(S, ring, A, t0 + 1, T, y0, row_end, gx, q);
+    sr_stage<Real, 2, M, VF>(S, ring, A, t0 + 2, T, y0, row_end, gx, q);
+    sr_stage<Real, 3, M, VF>(S, ring, A, t0 + 3, T, y0, row_end, gx, q);
   }
   cp_wait<0>();
 }
@@ -311,10 +333,22 @@ __global__ void __launch_bounds__(32 * WPB) smooth_restrict_stream_kernel(SRArgs
   const int gx = strip * SR_W - 4;
   const int y0 = blockIdx.y * seg_rows;
   const int row_end = min(y0 + seg_rows, A.n + 1);
-  if (gx >= 0 && gx + 63 <= A.n)
-    sr_run<Real, false, VF>(ring, A, gx, y0, row_end);
-  else
-    sr_run<Real, true, VF>(ring, A, gx, y0, row_end);
+  // FP64 strips and segments strictly inside the square (every loaded node) take the code for their
+  // operators: all warps of a launch share bA and bB, so there is no divergence. (FP32 is not bound
+  // by its arithmetic: the same specialisation left smooth_restrict at n = 4096 at 78 us.)
+  const bool cols = gx >= 0 && gx + 63 <= A.n;
+  if (sizeof(Real) == 8 && cols && gx >= 1 && gx + 63 < A.n && y0 - 3 >= 1 && row_end + 2 < A.n) {
+    if (A.bA == (Real)0 && A.bB == (Real)0)
+      sr_run<Real, Mode<false, xr::DIAG_REAL, xr::DIAG_REAL>, VF>(ring, A, gx, y0, row_end);
+    else if (A.bB == (Real)0)
+      sr_run<Real, Mode<false, xr::DIAG_INNER, xr::DIAG_REAL>, VF>(ring, A, gx, y0, row_end);
+    else
+      sr_run<Real, Mode<false, xr::DIAG_INNER, xr::DIAG_INNER>, VF>(ring, A, gx, y0, row_end);
+  } else if (cols) {
+    sr_run<Real, Mode<false, xr::DIAG_ANY, xr::DIAG_ANY>, VF>(ring, A, gx, y0, row_end);
+  } else {
+    sr_run<Real, Mode<true, xr::DIAG_ANY, xr::DIAG_ANY>, VF>(ring, A, gx, y0, row_end);
+  }
 }
 
 // ------------------------------------------------------------------ prolong + post-smooth
@@ -330,7 +364,9 @@ constexpr int PS_R = 8;            // row slots per warp
 template <class Real> __host__ __device__ constexpr int ps_upre_off() { return 32 * pair_bytes<Real>(); }
 template <class Real> __host__ __device__ constexpr int ps_k_off() { return 64 * pair_bytes<Real>(); }
 template <class Real> __host__ __device__ constexpr int ps_e_off() { return ps_k_off<Real>() + 32 * kpair_bytes<Real>(); }
-template <class Real> __host__ __device__ constexpr int ps_slot() { return ps_e_off<Real>() + 32 * (int)sizeof(c2<Real>); }
+// in FP64 then the stored 1 / |d|^2 pairs
+template <class Real> __host__ __device__ constexpr int ps_inv_off() { return ps_e_off<Real>() + 32 * (int)sizeof(c2<Real>); }
+template <class Real> __host__ __device__ constexpr int ps_slot() { return ps_inv_off<Real>() + 32 * ipair_bytes<Real>(); }
 
 template <class Real>
 struct PSArgs {
@@ -346,6 +382,8 @@ struct PSArgs {
   int pk;
   int n;
   Real bA;
+  const double* inv;
+  int pi;
 };
 
 template <class Real>
@@ -353,7 +391,8 @@ struct PSState {
   L2c<Real> F[4];
   c2<Real> K[4];
   L2c<Real> U[4];
-  c2<Real> Ee;  // coarse e under the last even row
+  c2<Real> I[4];  // stored 1 / |d|^2 (FP64)
+  c2<Real> Ee;    // coarse e under the last even row
 };
 
 // Copies of loaded row t (< T) and, on even rows, of the coarse row under it (also for t == T,
@@ -372,6 +411,9 @@ __device__ __forceinline__ void ps_issue(unsigned char* ring, const PSArgs<Real>
                                   A.upre + (long long)mj * A.pu, q.c0, q.m0, q.m1);
       copy_kpair<Real, EDGE>(smem_addr(slot + ps_k_off<Real>() + kpair_bytes<Real>() * threadIdx.x),
                              A.kh + (long long)mj * A.pk, q.c0, q.m0, q.m1);
+      if constexpr (sizeof(Real) == 8)
+        copy_kpair<Real, EDGE>(smem_addr(slot + ps_inv_off<Real>() + ipair_bytes<Real>() * threadIdx.x),
+                               A.inv + (long long)mj * A.pi, q.c0, q.m0, q.m1);
     }
     if (!(j & 1))
       cp_elem<sizeof(c2<Real>)>(smem_addr(slot + ps_e_off<Real>() + (int)sizeof(c2<Real>) * threadIdx.x),
@@ -380,14 +422,18 @@ __device__ __forceinline__ void ps_issue(unsigned char* ring, const PSArgs<Real>
   cp_commit();
 }
 
-template <class Real, int Q, bool EDGE, bool V>
+template <class Real, int Q, class M, bool V>
 __device__ __forceinline__ void ps_stage(PSState<Real>& S, unsigned char* ring, const PSArgs<Real>& A, int t, int T, int y0,
                                          int row_end, int gx, const Lane<Real>& q, int ci) {
+  constexpr bool EDGE = M::EDGE;
+  constexpr int KA = M::KA;
   if (t >= T) return;
   cp_wait<PS_R - 3>();  // rows up to t + 1 have landed (t + R - 1 groups committed)
   const unsigned char* slot = ring + (t % PS_R) * ps_slot<Real>();
   S.F[Q] = lds_pair<Real>(slot + pair_bytes<Real>() * threadIdx.x);
   S.K[Q] = *reinterpret_cast<const c2<Real>*>(slot + ps_k_off<Real>() + kpair_bytes<Real>() * threadIdx.x);
+  if constexpr (sizeof(Real) == 8)
+    S.I[Q] = *reinterpret_cast<const c2<Real>*>(slot + ps_inv_off<Real>() + ipair_bytes<Real>() * threadIdx.x);
   // global row y0 - 2 + t has the parity of t: red is column 0 of the pair on even t
   constexpr int er = (Q & 1) ? 1 : 0;
   const int j0 = y0 - 2 + t;
@@ -412,10 +458,10 @@ __device__ __forceinline__ void ps_stage(PSState<Real>& S, unsigned char* ring, 
     L2c<Real>& U = S.U[q1];
     if (er == 1) {
       const c2<Real> nb = xr::nb4<Real>(U.a, shfl_down2<Real>(U.a), S.U[q2].b, S.U[Q].b);
-      U.b = xr::gs<Real>(S.F[q1].b, nb, diag<Real>(S.K[q1].y, q.sc1 + rs, A.bA));
+      U.b = xr::gs_k<Real, KA>(S.F[q1].b, nb, xr::diag_k<Real, KA>(S.K[q1].y, q.sc1 + rs, A.bA), S.I[q1].y);
     } else {
       const c2<Real> nb = xr::nb4<Real>(shfl_up2<Real>(U.b), U.b, S.U[q2].a, S.U[Q].a);
-      U.a = xr::gs<Real>(S.F[q1].a, nb, diag<Real>(S.K[q1].x, q.sc0 + rs, A.bA));
+      U.a = xr::gs_k<Real, KA>(S.F[q1].a, nb, xr::diag_k<Real, KA>(S.K[q1].x, q.sc0 + rs, A.bA), S.I[q1].x);
     }
   }
   if (t >= 2) {  // red at row t-2, column er (its neighbours are updated black nodes)
@@ -424,10 +470,10 @@ __device__ __forceinline__ void ps_stage(PSState<Real>& S, unsigned char* ring, 
     L2c<Real>& U = S.U[q2];
     if (er == 0) {
       const c2<Real> nb = xr::nb4<Real>(shfl_up2<Real>(U.b), U.b, S.U[q3].a, S.U[q1].a);
-      U.a = xr::gs<Real>(S.F[q2].a, nb, diag<Real>(S.K[q2].x, q.sc0 + rs, A.bA));
+      U.a = xr::gs_k<Real, KA>(S.F[q2].a, nb, xr::diag_k<Real, KA>(S.K[q2].x, q.sc0 + rs, A.bA), S.I[q2].x);
     } else {
       const c2<Real> nb = xr::nb4<Real>(U.a, shfl_down2<Real>(U.a), S.U[q3].b, S.U[q1].b);
-      U.b = xr::gs<Real>(S.F[q2].b, nb, diag<Real>(S.K[q2].y, q.sc1 + rs, A.bA));
+      U.b = xr::gs_k<Real, KA>(S.F[q2].b, nb, xr::diag_k<Real, KA>(S.K[q2].y, q.sc1 + rs, A.bA), S.I[q2].y);
     }
     const int jo = j0 - 2;
     if (jo >= y0 && jo < row_end)
@@ -437,22 +483,23 @@ __device__ __forceinline__ void ps_stage(PSState<Real>& S, unsigned char* ring, 
   ps_issue<Real, EDGE, V>(ring, A, t + PS_R - 1, T, y0, q, ci);
 }
 
-template <class Real, bool EDGE, bool V>
+template <class Real, class M, bool V>
 __device__ __forceinline__ void ps_run(unsigned char* ring, const PSArgs<Real>& A, int gx, int y0, int row_end) {
+  constexpr bool EDGE = M::EDGE;
   const Lane<Real> q = lane_of<Real>(gx, A.n);
   const int ci = mirror_index(q.c0 >> 1, A.n >> 1);  // this lane's coarse column
   const int T = row_end - y0 + 4;
   PSState<Real> S;
 #pragma unroll
-  for (int k = 0; k < 4; ++k) S.U[k].a = S.U[k].b = mk<Real>(0, 0);
+  for (int k = 0; k < 4; ++k) S.U[k].a = S.U[k].b = S.I[k] = mk<Real>(0, 0);
   S.Ee = mk<Real>(0, 0);
   for (int t = 0; t < PS_R - 1; ++t) ps_issue<Real, EDGE, V>(ring, A, t, T, y0, q, ci);
 #pragma unroll 1
   for (int t0 = 0; t0 < T; t0 += 4) {  // as in sr_run: row t in window slot t mod 4
-    ps_stage<Real, 0, EDGE, V>(S, ring, A, t0 + 0, T, y0, row_end, gx, q, ci);
-    ps_stage<Real, 1, EDGE, V>(S, ring, A, t0 + 1, T, y0, row_end, gx, q, ci);
-    ps_stage<Real, 2, EDGE, V>(S, ring, A, t0 + 2, T, y0, row_end, gx, q, ci);
-    ps_stage<Real, 3, EDGE, V>(S, ring, A, t0 + 3, T, y0, row_end, gx, q, ci);
+    ps_stage<Real, 0, M, V>(S, ring, A, t0 + 0, T, y0, row_end, gx, q, ci);
+    ps_stage<Real, 1, M, V>(S, ring, A, t0 + 1, T, y0, row_end, gx, q, ci);
+    ps_stage<Real, 2, M, V>(S, ring, A, t0 + 2, T, y0, row_end, gx, q, ci);
+    ps_stage<Real, 3, M, V>(S, ring, A, t0 + 3, T, y0, row_end, gx, q, ci);
   }
   cp_wait<0>();
 }
@@ -473,10 +520,17 @@ __global__ void __launch_bounds__(32 * WPB) prolong_smooth_stream_kernel(PSArgs<
   const int gx = strip * PS_W - 2;
   const int y0 = blockIdx.y * seg_rows;
   const int row_end = min(y0 + seg_rows, A.n + 1);
-  if (gx >= 0 && gx + 63 <= A.n)
-    ps_run<Real, false, V>(ring, A, gx, y0, row_end);
-  else
-    ps_run<Real, true, V>(ring, A, gx, y0, row_end);
+  const bool cols = gx >= 0 && gx + 63 <= A.n;
+  if (sizeof(Real) == 8 && cols && gx >= 1 && gx + 63 < A.n && y0 - 2 >= 1 && row_end + 1 < A.n) {
+    if (A.bA == (Real)0)
+      ps_run<Real, Mode<false, xr::DIAG_REAL, 0>, V>(ring, A, gx, y0, row_end);
+    else
+      ps_run<Real, Mode<false, xr::DIAG_INNER, 0>, V>(ring, A, gx, y0, row_end);
+  } else if (cols) {
+    ps_run<Real, Mode<false, xr::DIAG_ANY, 0>, V>(ring, A, gx, y0, row_end);
+  } else {
+    ps_run<Real, Mode<true, xr::DIAG_ANY, 0>, V>(ring, A, gx, y0, row_end);
+  }
 }
 
 bool aligned16(const void* p, long long pitch, long long stride) {
@@ -495,7 +549,7 @@ cudaError_t allow_smem(K kernel, size_t bytes, bool& done) {
 template <class Real>
 cudaError_t sr_stream(void* u, int pu, void* fc, int pc, const void* f, int pf, const void* kh, int pk, int n,
                       double bA, double bB, int seg_rows, const int* stop, cudaStream_t s, const Inst& bi) {
-  SRArgs<Real> A{(c2<Real>*)u, pu, (c2<Real>*)fc, pc, (const c2<Real>*)f, pf, (const Real*)kh, pk, n, (Real)bA, (Real)bB};
+  SRArgs<Real> A{(c2<Real>*)u, pu, (c2<Real>*)fc, pc, (const c2<Real>*)f, pf, (const Real*)kh, pk, n, (Real)bA, (Real)bB, bi.inv, bi.pi};
   const int strips = (n + 1 + SR_W - 1) / SR_W, segs = (n + 1 + seg_rows - 1) / seg_rows;
   dim3 grid((strips + WPB - 1) / WPB, segs, bi.count);
   constexpr size_t sm = (size_t)WPB * SR_R * sr_slot<Real>();
@@ -516,7 +570,7 @@ cudaError_t ps_stream(void* out, int po, const void* upre, int pu, const void* e
                       const void* kh, int pk, int n, double bA, int seg_rows, const int* stop, cudaStream_t s,
                       const Inst& bi) {
   PSArgs<Real> A{(c2<Real>*)out, po, (const c2<Real>*)upre, pu, (const c2<Real>*)ec, pc, (const c2<Real>*)f, pf,
-                 (const Real*)kh, pk, n, (Real)bA};
+                 (const Real*)kh, pk, n, (Real)bA, bi.inv, bi.pi};
   const int strips = (n + 1 + PS_W - 1) / PS_W, segs = (n + 1 + seg_rows - 1) / seg_rows;
   dim3 grid((strips + WPB - 1) / WPB, segs, bi.count);
   constexpr size_t sm = (size_t)WPB * PS_R * ps_slot<Real>();

@@ -122,7 +122,7 @@ __global__ void kacz_colour_kernel(c2<T>* __restrict__ u, int pu, const F2* __re
   if (j > n) return;
   int i = ((colour - 2 * j) % 5 + 5) % 5 + 5 * m;
   if (i > n) return;
-  gnode::kacz_row<T, F2>(u, pu, f, pf, kh, pk, n, i, j, beta);
+  gnode::kacz_row<T, F2>(u, pu, f, pf, kh, pk, n, i, j, beta, bi.inv, bi.pi);
 }
 
 // ---------------------------------------------------------------- transfers (Sec. 5)
@@ -312,6 +312,22 @@ __global__ void inject_kh_kernel(T* __restrict__ kh, int pk, const double* __res
   kh[(long long)J * pk + I] = (T)(k0[(long long)stride * J * (n0 + 1) + (long long)stride * I] * H);
 }
 
+__global__ void level_inverse_kernel(double* __restrict__ inv, int pi, const double* __restrict__ kh, int pk, int n,
+                                     double beta, bool kaczmarz) {
+  pdl_enter();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = blockIdx.y * blockDim.y + threadIdx.y;
+  if (i > n || j > n) return;
+  const double k = kh[(long long)j * pk + i];
+  double2 d;
+  double v;
+  if (kaczmarz)
+    lvl::row_consts<double>(k, i, j, n, beta, &d, &v);
+  else
+    v = xr::rcp(xr::cabs2<double>(xr::diag<double>(k, lvl::sides_at(i, j, n), beta)));
+  inv[(long long)j * pi + i] = v;
+}
+
 template <class T, class F2>
 cudaError_t gs_colour_t(void* u, int pu, const void* f, int pf, const void* kh, int pk, int n, int colour, double beta,
                         const int* stop, cudaStream_t s, const Inst& bi, double omega) {
@@ -449,6 +465,12 @@ cudaError_t launch_inject_kh(bool fp32, void* kh, int pk, const double* k0, int 
     pdl_launch(inject_kh_kernel<float>, grid2(nl + 1, nl + 1), dim3(BX, BY), 0, s, (float*)kh, pk, k0, n0, stride, nl, H);
   else
     pdl_launch(inject_kh_kernel<double>, grid2(nl + 1, nl + 1), dim3(BX, BY), 0, s, (double*)kh, pk, k0, n0, stride, nl, H);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_level_inverse(double* inv, int pi, const double* kh, int pk, int n, double beta, bool kaczmarz,
+                                 cudaStream_t s) {
+  pdl_launch(level_inverse_kernel, grid2(n + 1, n + 1), dim3(BX, BY), 0, s, inv, pi, kh, pk, n, beta, kaczmarz);
   return cudaGetLastError();
 }
 
