@@ -1077,14 +1077,20 @@ bool opts_ok(const hz_hierarchy_opts& o) {
 
 // ------------------------------------------------------------------ coarse tail
 // The largest tail that fits TAIL_MAX_SMEM: levels lt .. L-1 (lt >= 1), each a one-sweep
-// Gauss-Seidel level or a Kaczmarz level, the last the coarsest.
+// Gauss-Seidel level or a Kaczmarz level, the last the coarsest. Only where one block is the faster
+// way: its FP64 pipe makes every level above 16 intervals slower than launches over several SMs (FP64
+// iteration at n = 64 193 us with levels 32 .. 8 in the tail, 158 without one; n = 512 1104 and 1015;
+// n = 240 848 and 812), and so is a coarsest solve of many unknowns (FP32 iteration at n = 864, 784
+// unknowns: 488 us with the tail, 363 with coarse_solve_kernel over 49 blocks; at 256 unknowns 212 both ways).
+constexpr int TAIL_MAX_N64 = 16, TAIL_MAX_COARSE32 = 256, TAIL_MAX_COARSE64 = 100;
 void plan_tail(hz_problem* P) {
   P->tail_start = -1;
   const int L = P->plan.levels;
   if (!P->opts.coarse_tail || L < 3) return;
   const bool fp32 = P->plan.fp32;
+  if (P->plan.m_coarse > (fp32 ? TAIL_MAX_COARSE32 : TAIL_MAX_COARSE64)) return;
   for (int lt = 1; lt <= L - 2; ++lt) {
-    if (L - lt > TAIL_MAX_LEVELS) continue;
+    if (L - lt > TAIL_MAX_LEVELS || (!fp32 && P->lv[lt].n > TAIL_MAX_N64)) continue;
     bool ok = true;
     TailArgs A{};
     A.count = L - lt;

@@ -162,20 +162,68 @@ __global__ void prolong_add_kernel(c2<T>* __restrict__ u, int pu, const c2<T>* _
 
 // ---------------------------------------------------------------- coarsest grid
 
-// u = A_c^{-1} f~ with the dense inverse stored transposed (column c contiguous), one block.
+// u = A_c^{-1} f~ with the dense inverse stored transposed (column c contiguous). A row's sum runs over
+// the columns in order (lvl::coarse_row's, so that every form gives the same bits): a chain of m
+// additions, 77 cycles each on the FP64 pipe. A block takes 16 rows, one lane of a warp per row and
+// component; warp 0 does the additions while the other warps form the products of the next chunk of
+// columns in shared memory (in FP64 the warps that share no sub-partition with it), so a launch costs
+// the additions alone and the rows spread over the SMs. One block for all rows was bound by its FP64
+// pipe, or by one load latency per eight columns: m = 81 25 us, m = 256 114 us, m = 1024 1720 us (FP64)
+// and 177 us (FP32).
+constexpr int CS_ROWS = 16;
+template <class T> struct CoarseChunk;  // columns per producer warp and chunk, producer warps
+template <> struct CoarseChunk<double> { static constexpr int PER = 8, WARPS = 6; };
+template <> struct CoarseChunk<float> { static constexpr int PER = 16, WARPS = 7; };
 template <class T>
-__global__ void coarse_solve_kernel(c2<T>* __restrict__ u, int pu, const c2<T>* __restrict__ f, int pf,
-                                    const c2<T>* __restrict__ ainvT, int nc, const int* __restrict__ stop, Inst bi) {
+__global__ void __launch_bounds__(256) coarse_solve_kernel(c2<T>* __restrict__ u, int pu, const c2<T>* __restrict__ f,
+                                                           int pf, const c2<T>* __restrict__ ainvT, int nc,
+                                                           const int* __restrict__ stop, Inst bi) {
+  constexpr int PER = CoarseChunk<T>::PER, NW = CoarseChunk<T>::WARPS, CH = PER * NW;
+  __shared__ T prod[2][CH][32];
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  c2<T>* fs = reinterpret_cast<c2<T>*>(smem_raw);
+  const int w = nc + 1, m = w * w;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, comp = lane & 1;
+  const int row = blockIdx.x * CS_ROWS + (lane >> 1), r = min(row, m - 1);
+  // producer index: FP64 warps 1, 2, 3, 5, 6, 7 (warps 0 and 4 share the adding warp's sub-partition)
+  const int pw = sizeof(T) == 8 ? (warp % 4 == 0 ? -1 : warp < 4 ? warp - 1 : warp - 2) : warp - 1;
+  c2<T> a[PER];
+  auto fetch = [&](int c0) {
+    if (pw < 0) return;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) a[q] = ainvT[(long long)min(c0 + pw * PER + q, m - 1) * m + r];
+  };
+  fetch(0);  // the inverse is fixed since set-up: fetched before the wait for the preceding kernel
   pdl_enter();
   if (stop && stop[blockIdx.z * bi.stop_stride]) return;
   u += blockIdx.z * bi.su;
   f += blockIdx.z * bi.su;
-  extern __shared__ unsigned char smem_raw[];
-  c2<T>* fs = reinterpret_cast<c2<T>*>(smem_raw);
-  int w = nc + 1, m = w * w;
   for (int q = threadIdx.x; q < m; q += blockDim.x) fs[q] = f[(long long)(q / w) * pf + q % w];
   __syncthreads();
-  for (int r = threadIdx.x; r < m; r += blockDim.x) u[(long long)(r / w) * pu + r % w] = lvl::coarse_row<T>(ainvT, fs, m, r);
+  T acc = (T)0;
+  for (int c0 = 0, k = 0; c0 < m + CH; c0 += CH, ++k) {
+    if (pw >= 0 && c0 < m) {  // products of columns c0 .. c0 + CH - 1 (xr::cmul's component)
+#pragma unroll
+      for (int q = 0; q < PER; ++q) {
+        const c2<T> v = fs[min(c0 + pw * PER + q, m - 1)];
+        const T t = xr::mul(a[q].y, comp ? v.x : v.y);
+        prod[k & 1][pw * PER + q][lane] = xr::fma(a[q].x, comp ? v.y : v.x, comp ? t : -t);
+      }
+      if (c0 + CH < m) fetch(c0 + CH);
+    }
+    if (warp == 0 && k > 0) {  // the previous chunk's additions, in column order
+      const int cnt = min(CH, m - (c0 - CH));
+      const T(*p)[32] = prod[(k - 1) & 1];
+      if (cnt == CH) {
+#pragma unroll 16
+        for (int q = 0; q < CH; ++q) acc = xr::add(acc, p[q][lane]);
+      } else {
+        for (int q = 0; q < cnt; ++q) acc = xr::add(acc, p[q][lane]);
+      }
+    }
+    __syncthreads();
+  }
+  if (warp == 0 && row < m) reinterpret_cast<T*>(u + (long long)(row / w) * pu + row % w)[comp] = acc;
 }
 
 // Dense scaled operator of the coarsest level (row-major, m x m) next to the identity, then
@@ -428,15 +476,14 @@ cudaError_t launch_prolong_add(bool fp32, void* u, int pu, const void* ec, int p
 
 cudaError_t launch_coarse_solve(bool fp32, void* u, int pu, const void* f, int pf, const void* ainvT, int nc,
                                 const int* stop, cudaStream_t s, const Inst& bi) {
-  int m = (nc + 1) * (nc + 1);
-  int threads = m < 256 ? ((m + 31) / 32) * 32 : 256;
-  dim3 g(1, 1, bi.count);
+  const int m = (nc + 1) * (nc + 1);
+  const dim3 g((m + CS_ROWS - 1) / CS_ROWS, 1, bi.count);
   if (fp32)
-    pdl_launch(coarse_solve_kernel<float>, g, threads, m * sizeof(float2), s, (float2*)u, pu, (const float2*)f, pf,
-                                                                       (const float2*)ainvT, nc, stop, bi);
+    pdl_launch(coarse_solve_kernel<float>, g, 256, m * sizeof(float2), s, (float2*)u, pu, (const float2*)f, pf,
+               (const float2*)ainvT, nc, stop, bi);
   else
-    pdl_launch(coarse_solve_kernel<double>, g, threads, m * sizeof(double2), s, (double2*)u, pu, (const double2*)f, pf,
-                                                                         (const double2*)ainvT, nc, stop, bi);
+    pdl_launch(coarse_solve_kernel<double>, g, 256, m * sizeof(double2), s, (double2*)u, pu, (const double2*)f, pf,
+               (const double2*)ainvT, nc, stop, bi);
   return cudaGetLastError();
 }
 
