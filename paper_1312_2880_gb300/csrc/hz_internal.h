@@ -103,12 +103,20 @@ cudaError_t launch_kacz_level_post(bool fp32, void* u, int pu, const void* ec, i
                                    const void* kh, int pk, int n, double bA, int nu, const int* stop, cudaStream_t s, const Inst& bi = Inst());
 // Whole level over a thread-block cluster (row bands, distributed shared memory; up to 16 blocks).
 bool kacz_cluster_fits(bool fp32, int n);
+// (FP32 levels, and FP64 levels: hz_kcluster.cu)
 cudaError_t launch_kacz_cluster_pre(bool fp32, void* u, int pu, void* fc, int pc, const void* f, int pf, const void* kh,
                                     int pk, int n, double bA, double bB, int nu, const int* stop, cudaStream_t s,
                                     const Inst& bi = Inst());
 cudaError_t launch_kacz_cluster_post(bool fp32, void* u, int pu, const void* ec, int pc, const void* f, int pf,
                                      const void* kh, int pk, int n, double bA, int nu, const int* stop, cudaStream_t s,
                                      const Inst& bi = Inst());
+bool kacz_cluster64_fits(int n);
+cudaError_t launch_kacz_cluster64_pre(double2* u, int pu, double2* fc, int pc, const double2* f, int pf,
+                                      const double* kh, int pk, int n, double bA, double bB, int nu, const int* stop,
+                                      cudaStream_t s, const Inst& bi);
+cudaError_t launch_kacz_cluster64_post(double2* u, int pu, const double2* ec, int pc, const double2* f, int pf,
+                                       const double* kh, int pk, int n, double bA, int nu, const int* stop,
+                                       cudaStream_t s, const Inst& bi);
 // Whole level in global memory by one persistent cooperative launch per pass (hz_kgrid.cu); one
 // instance (batch 1). Each block owns a band of grid rows and publishes its progress (phases
 // done) in its counter; before a phase it waits, with a bounded number of polls, for the two

@@ -13,9 +13,9 @@
 //   the dependency cone of the sweep (6 columns each side, 6 and 10 rows), so the tile interior holds
 //   exactly the sequential sweep's values; each phase acts only on the part of the region that can
 //   still reach the tile. Out of place. (FP32 levels run whole passes in tiles: hz_kpass.cu.)
-// kacz_cluster_*: the kacz_level_* operations with the level split into row bands over a
+// kacz_cluster_*: the kacz_level_* operations with an FP32 level split into row bands over a
 //   thread-block cluster of up to 16 blocks (distributed shared memory, one cluster barrier per
-//   colour), for levels too large for one block or, in FP64, too slow on one SM's FP64 pipe.
+//   colour), for levels too large for one block with an odd number of sweeps (FP64: hz_kcluster.cu).
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -411,8 +411,7 @@ cudaError_t launch_kacz_level_post(bool fp32, void* u, int pu, const void* ec, i
 // action on a band's first or last row reads and updates one node of the neighbouring band
 // through distributed shared memory; rows of one colour have disjoint supports, so no node is
 // touched twice in a colour, and a cluster barrier separates the colours. Same operations as the
-// one-block form (hz_level.cuh), spread over C SMs: for the FP64 form this is C times the FP64
-// rate of one SM on the Kaczmarz level.
+// one-block form (hz_level.cuh), spread over C SMs.
 namespace {
 
 namespace cgx = cooperative_groups;
@@ -446,18 +445,6 @@ struct ClusterLevel {
     return base + (j - owner * rows) * w;
   }
 };
-
-// Row constants of a band's node: in FP64 the reciprocal is read (it is half of their instructions).
-template <class T>
-__device__ __forceinline__ void cluster_consts(const ClusterLevel<T>& L, int q, T kh, int i, int j, int n, T bA,
-                                               const Inst& bi) {
-  if (sizeof(T) == 8 && bi.inv) {
-    L.sd[q] = xr::diag<T>(kh, lvl::sides_at(i, j, n), bA);
-    L.sinv[q] = (T)bi.inv[(long long)j * bi.pi + i];
-  } else {
-    lvl::row_consts<T>(kh, i, j, n, bA, &L.sd[q], &L.sinv[q]);
-  }
-}
 
 template <class T>
 __device__ __forceinline__ void cluster_act(cgx::cluster_group& cl, const ClusterLevel<T>& L, int i, int j) {
@@ -509,7 +496,7 @@ __global__ void __launch_bounds__(KC_THREADS) kacz_cluster_pre_kernel(c2<T>* __r
     const int j = L.r0 + q / w, i = q % w;
     L.su[q] = mk<T>(0, 0);
     L.sf[q] = f[(long long)j * pf + i];
-    cluster_consts<T>(L, q, kh[(long long)j * pk + i], i, j, n, bA, bi);
+    lvl::row_consts<T>(kh[(long long)j * pk + i], i, j, n, bA, &L.sd[q], &L.sinv[q]);
   }
   cl.sync();
   cluster_sweeps<T>(cl, L, nu, false);
@@ -561,7 +548,7 @@ __global__ void __launch_bounds__(KC_THREADS) kacz_cluster_post_kernel(c2<T>* __
     const c2<T>* e0 = ec + (long long)(j >> 1) * pc;
     L.su[q] = xr::cadd<T>(u[(long long)j * pu + i], xr::bilinear<T>(e0, e0 + pc, i >> 1, i & 1, j & 1));
     L.sf[q] = f[(long long)j * pf + i];
-    cluster_consts<T>(L, q, kh[(long long)j * pk + i], i, j, n, bA, bi);
+    lvl::row_consts<T>(kh[(long long)j * pk + i], i, j, n, bA, &L.sd[q], &L.sinv[q]);
   }
   cl.sync();
   cluster_sweeps<T>(cl, L, nu, true);
@@ -679,45 +666,33 @@ ClusterShape cluster_shape(int n) {
 
 }  // namespace
 
-bool kacz_cluster_fits(bool fp32, int n) { return (fp32 ? cluster_shape<float>(n) : cluster_shape<double>(n)).c > 0; }
+bool kacz_cluster_fits(bool fp32, int n) { return fp32 ? cluster_shape<float>(n).c > 0 : kacz_cluster64_fits(n); }
 
 cudaError_t launch_kacz_cluster_pre(bool fp32, void* u, int pu, void* fc, int pc, const void* f, int pf, const void* kh,
                                     int pk, int n, double bA, double bB, int nu, const int* stop, cudaStream_t s,
                                     const Inst& bi) {
-  cudaError_t e;
-  if (fp32) {
-    const ClusterShape C = cluster_shape<float>(n);
-    if (!C.c) return cudaErrorInvalidValue;
-    e = launch_cluster_kernel<float>(kacz_cluster_pre_kernel<float>, C.c, C.smem, s, bi, (float2*)u, pu, (float2*)fc,
-                                     pc, (const float2*)f, pf, (const float*)kh, pk, n, (float)bA, (float)bB, nu, C.rows,
-                                     stop, bi);
-  } else {
-    const ClusterShape C = cluster_shape<double>(n);
-    if (!C.c) return cudaErrorInvalidValue;
-    e = launch_cluster_kernel<double>(kacz_cluster_pre_kernel<double>, C.c, C.smem, s, bi, (double2*)u, pu,
-                                      (double2*)fc, pc, (const double2*)f, pf, (const double*)kh, pk, n, bA, bB, nu,
-                                      C.rows, stop, bi);
-  }
+  if (!fp32)
+    return launch_kacz_cluster64_pre((double2*)u, pu, (double2*)fc, pc, (const double2*)f, pf, (const double*)kh, pk, n,
+                                     bA, bB, nu, stop, s, bi);
+  const ClusterShape C = cluster_shape<float>(n);
+  if (!C.c) return cudaErrorInvalidValue;
+  cudaError_t e = launch_cluster_kernel<float>(kacz_cluster_pre_kernel<float>, C.c, C.smem, s, bi, (float2*)u, pu,
+                                               (float2*)fc, pc, (const float2*)f, pf, (const float*)kh, pk, n, (float)bA,
+                                               (float)bB, nu, C.rows, stop, bi);
   return e ? e : cudaGetLastError();
 }
 
 cudaError_t launch_kacz_cluster_post(bool fp32, void* u, int pu, const void* ec, int pc, const void* f, int pf,
                                      const void* kh, int pk, int n, double bA, int nu, const int* stop, cudaStream_t s,
                                      const Inst& bi) {
-  cudaError_t e;
-  if (fp32) {
-    const ClusterShape C = cluster_shape<float>(n);
-    if (!C.c) return cudaErrorInvalidValue;
-    e = launch_cluster_kernel<float>(kacz_cluster_post_kernel<float>, C.c, C.smem, s, bi, (float2*)u, pu,
-                                     (const float2*)ec, pc, (const float2*)f, pf, (const float*)kh, pk, n, (float)bA,
-                                     nu, C.rows, stop, bi);
-  } else {
-    const ClusterShape C = cluster_shape<double>(n);
-    if (!C.c) return cudaErrorInvalidValue;
-    e = launch_cluster_kernel<double>(kacz_cluster_post_kernel<double>, C.c, C.smem, s, bi, (double2*)u, pu,
-                                      (const double2*)ec, pc, (const double2*)f, pf, (const double*)kh, pk, n, bA, nu,
-                                      C.rows, stop, bi);
-  }
+  if (!fp32)
+    return launch_kacz_cluster64_post((double2*)u, pu, (const double2*)ec, pc, (const double2*)f, pf, (const double*)kh, pk,
+                                      n, bA, nu, stop, s, bi);
+  const ClusterShape C = cluster_shape<float>(n);
+  if (!C.c) return cudaErrorInvalidValue;
+  cudaError_t e = launch_cluster_kernel<float>(kacz_cluster_post_kernel<float>, C.c, C.smem, s, bi, (float2*)u, pu,
+                                               (const float2*)ec, pc, (const float2*)f, pf, (const float*)kh, pk, n,
+                                               (float)bA, nu, C.rows, stop, bi);
   return e ? e : cudaGetLastError();
 }
 
