@@ -163,6 +163,39 @@ __device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b);
 __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma(double a, double b, double c) { return __fma_rn(a, b, c); }
+// The correctly rounded FP64 sum a + b on the integer pipe (the bits of __dadd_rn, from the IEEE 754
+// formats): order by magnitude, align the smaller significand below the larger with ten guard bits and
+// a sticky bit, add or subtract, normalise, round to nearest even. About 50 instructions of the
+// integer pipe against 77 cycles of the FP64 pipe, which kernels bound by the latter leave idle:
+// there, some of the additions done here run beside the rest. Zeros, subnormal operands or results,
+// infinities, NaN and exact cancellation take the hardware addition.
+// Out of line: in line, the compiler predicates this addition and issues it for every warp.
+static __device__ __noinline__ double add_hw(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double add_int(double a, double b) {
+  unsigned ah = (unsigned)__double2hiint(a), al = (unsigned)__double2loint(a);
+  unsigned bh = (unsigned)__double2hiint(b), bl = (unsigned)__double2loint(b);
+  const unsigned long long ua = ((unsigned long long)(ah & 0x7fffffffu) << 32) | al;
+  const unsigned long long ub = ((unsigned long long)(bh & 0x7fffffffu) << 32) | bl;
+  if (ub > ua) {
+    unsigned t = ah; ah = bh; bh = t;
+    t = al; al = bl; bl = t;
+  }
+  const int ea = (int)(ah >> 20) & 0x7ff, eb = (int)(bh >> 20) & 0x7ff;
+  const unsigned long long ma = ((unsigned long long)__funnelshift_l(al, (ah & 0xfffffu) | 0x100000u, 10) << 32) | (al << 10);
+  const unsigned long long mb = ((unsigned long long)__funnelshift_l(bl, (bh & 0xfffffu) | 0x100000u, 10) << 32) | (bl << 10);
+  const int d = min(ea - eb, 63);
+  unsigned long long t = mb >> d;
+  t |= (t << d) != mb ? 1ull : 0ull;
+  const long long neg = (long long)(int)(ah ^ bh) >> 31;  // all ones: a difference
+  unsigned long long r = ma + ((t ^ (unsigned long long)neg) - (unsigned long long)neg);
+  const int lz = __clzll((long long)r), e = ea + 1 - lz;
+  if (eb == 0 || ea == 0x7ff || (unsigned)(e - 1) >= 0x7feu || r == 0) return add_hw(a, b);
+  r <<= lz;
+  const unsigned long long p = r >> 11;
+  const unsigned up = ((unsigned)r & 0x7ffu) + ((unsigned)p & 1u) > 0x400u ? 1u : 0u;
+  const unsigned long long q = p + up + ((unsigned long long)(unsigned)(e - 1) << 52);
+  return __hiloint2double((int)((unsigned)(q >> 32) | (ah & 0x80000000u)), (int)(unsigned)q);
+}
 // FP32: the hardware reciprocal approximation (rcp.approx, about 1 ulp); the divisors here are
 // |d|^2 of a Helmholtz diagonal, never denormal. FP64: the correctly rounded reciprocal.
 __device__ __forceinline__ float rcp(float a) {
@@ -225,6 +258,15 @@ template <class T>
 __device__ __forceinline__ c2<T> nb4(c2<T> w, c2<T> e, c2<T> s, c2<T> n) {
   return cadd<T>(cadd<T>(w, e), cadd<T>(s, n));
 }
+// The same with MIX of its six FP64 additions on the integer pipe (add_int; 0, 1, 2, 4 or 6).
+template <int MIX>
+__device__ __forceinline__ double2 nb4_mix(double2 w, double2 e, double2 s, double2 n) {
+  const double hx = MIX >= 1 ? add_int(w.x, e.x) : add(w.x, e.x), hy = MIX >= 2 ? add_int(w.y, e.y) : add(w.y, e.y);
+  const double vx = MIX >= 4 ? add_int(s.x, n.x) : add(s.x, n.x), vy = MIX >= 4 ? add_int(s.y, n.y) : add(s.y, n.y);
+  return MIX >= 6 ? mk<double>(add_int(hx, vx), add_int(hy, vy)) : mk<double>(add(hx, vx), add(hy, vy));
+}
+template <int MIX>
+__device__ __forceinline__ float2 nb4_mix(float2 w, float2 e, float2 s, float2 n) { return nb4<float>(w, e, s, n); }
 // Gauss-Seidel point update (f - nb) / d and residual f - (d u + nb).
 template <class T>
 __device__ __forceinline__ c2<T> gs(c2<T> f, c2<T> nb, c2<T> d) { return cdiv<T>(csub<T>(f, nb), d); }

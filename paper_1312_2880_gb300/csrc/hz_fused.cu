@@ -21,6 +21,10 @@ namespace hz {
 
 namespace {
 
+// FP64 neighbour sums on levels of at least MIX_MIN_N intervals: MIX_TILE of the six additions on the
+// integer pipe (xr::nb4_mix). n = 1024 smooth_restrict 118, 112, 107, 101 us with 0, 2, 4, 6 there, n = 512
+// 41, 38, 36, 34; smaller levels are bound by latency and lose (n = 64 FP64 solve 588 us with 0, 626 with 4).
+constexpr int MIX_TILE = 4, MIX_MIN_N = 256;
 constexpr int FT = 256;  // threads per block
 
 // Owned fine nodes of a tile (W x H). FP64 tiles are small: the FP64 passes are bound by each
@@ -40,10 +44,10 @@ struct TileShape<double> {
 
 __device__ __forceinline__ bool in_grid(int i, int j, int n) { return (unsigned)i <= (unsigned)n && (unsigned)j <= (unsigned)n; }
 
-template <class T>
+template <class T, int MIX>
 __device__ __forceinline__ c2<T> nb_sum(const c2<T>* s, int rw, int c, int r, int i, int j, int n, int gx, int gy) {
   Nbr b = neighbours(i, j, n);
-  return xr::nb4<T>(s[r * rw + (b.iw - gx)], s[r * rw + (b.ie - gx)], s[(b.js - gy) * rw + c],
+  return xr::nb4_mix<MIX>(s[r * rw + (b.iw - gx)], s[r * rw + (b.ie - gx)], s[(b.js - gy) * rw + c],
                     s[(b.jn - gy) * rw + c]);
 }
 
@@ -173,8 +177,8 @@ __device__ __forceinline__ void prolong_smooth_inner(O2* __restrict__ out, int p
 }
 
 // The general tile: every node tested against the grid (FP32 tiles at the boundary, all FP64 tiles).
-// KA, KB: kinds of the relaxation and residual diagonals (xr::DIAG_*).
-template <class T, class F2, int KA, int KB>
+// KA, KB: kinds of the relaxation and residual diagonals (xr::DIAG_*); MIX: see MIX_TILE.
+template <class T, class F2, int MIX, int KA, int KB>
 __device__ __forceinline__ void smooth_restrict_body(c2<T>* __restrict__ u, int pu, c2<T>* __restrict__ fc, int pc,
                                                      const F2* __restrict__ f, int pf, const T* __restrict__ kh,
                                                      int pk, int n, T bA, T bB, const Inst& bi, c2<T>* su, c2<T>* sf,
@@ -213,7 +217,7 @@ __device__ __forceinline__ void smooth_restrict_body(c2<T>* __restrict__ u, int 
     int i = gx + c;
     if (r >= 1 && r <= RH - 2 && c >= 1 && c <= RW - 2 && in_grid(i, j, n)) {
       Nbr b = neighbours(i, j, n);
-      c2<T> s = nb_sum<T>(su, RW, c, r, i, j, n, gx, gy);
+      c2<T> s = nb_sum<T, MIX>(su, RW, c, r, i, j, n, gx, gy);
       su[r * RW + c] = xr::gs_k<T, KA>(sf[r * RW + c], s, xr::diag_k<T, KA>(sk[r * RW + c], (T)(2 * b.sides), bA), si[r * RW + c]);
     }
   }
@@ -229,7 +233,7 @@ __device__ __forceinline__ void smooth_restrict_body(c2<T>* __restrict__ u, int 
     int r = q / RW, c = q - r * RW, i = gx + c, j = gy + r;
     if (r >= 2 && r <= RH - 3 && c >= 2 && c <= RW - 3 && in_grid(i, j, n)) {
       Nbr b = neighbours(i, j, n);
-      c2<T> s = nb_sum<T>(su, RW, c, r, i, j, n, gx, gy);
+      c2<T> s = nb_sum<T, MIX>(su, RW, c, r, i, j, n, gx, gy);
       sf[q] = xr::resid_k<T, KB>(sf[q], su[q], s, xr::diag_k<T, KB>(sk[q], (T)(2 * b.sides), bB));
     }
   }
@@ -243,7 +247,7 @@ __device__ __forceinline__ void smooth_restrict_body(c2<T>* __restrict__ u, int 
   }
 }
 
-template <class T, class F2, class O2, int KA>
+template <class T, class F2, class O2, int MIX, int KA>
 __device__ __forceinline__ void prolong_smooth_body(O2* __restrict__ out, int po, const c2<T>* __restrict__ upre,
                                                     int pu, const c2<T>* __restrict__ ec, int pc,
                                                     const F2* __restrict__ f, int pf, const T* __restrict__ kh, int pk,
@@ -286,7 +290,7 @@ __device__ __forceinline__ void prolong_smooth_body(O2* __restrict__ out, int po
     int i = gx + c;
     if (r >= 1 && r <= RH - 2 && c >= 1 && c <= RW - 2 && in_grid(i, j, n)) {
       Nbr b = neighbours(i, j, n);
-      c2<T> s = nb_sum<T>(su, RW, c, r, i, j, n, gx, gy);
+      c2<T> s = nb_sum<T, MIX>(su, RW, c, r, i, j, n, gx, gy);
       su[r * RW + c] = xr::gs_k<T, KA>(sf[r * RW + c], s, xr::diag_k<T, KA>(sk[r * RW + c], (T)(2 * b.sides), bA), si[r * RW + c]);
     }
   }
@@ -299,7 +303,7 @@ __device__ __forceinline__ void prolong_smooth_body(O2* __restrict__ out, int po
     int i = gx + c;
     if (r >= 2 && r < 2 + HH && c >= 2 && c < 2 + W && in_grid(i, j, n)) {
       Nbr b = neighbours(i, j, n);
-      c2<T> s = nb_sum<T>(su, RW, c, r, i, j, n, gx, gy);
+      c2<T> s = nb_sum<T, MIX>(su, RW, c, r, i, j, n, gx, gy);
       su[r * RW + c] = xr::gs_k<T, KA>(sf[r * RW + c], s, xr::diag_k<T, KA>(sk[r * RW + c], (T)(2 * b.sides), bA), si[r * RW + c]);
     }
   }
@@ -310,7 +314,7 @@ __device__ __forceinline__ void prolong_smooth_body(O2* __restrict__ out, int po
   }
 }
 
-template <class T, class F2>
+template <class T, class F2, int MIX>
 __global__ void __launch_bounds__(FT) smooth_restrict_kernel(c2<T>* __restrict__ u, int pu, c2<T>* __restrict__ fc,
                                                               int pc, const F2* __restrict__ f, int pf,
                                                               const T* __restrict__ kh, int pk, int n, T bA, T bB,
@@ -335,18 +339,18 @@ __global__ void __launch_bounds__(FT) smooth_restrict_kernel(c2<T>* __restrict__
   if constexpr (sizeof(T) == 8) {
     if (gx >= 1 && gy >= 1 && gx + RW <= n && gy + RH <= n) {  // every node strictly inside the square
       if (bA == (T)0 && bB == (T)0)
-        smooth_restrict_body<T, F2, xr::DIAG_REAL, xr::DIAG_REAL>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, bi, su, sf, sk, gx, gy);
+        smooth_restrict_body<T, F2, MIX, xr::DIAG_REAL, xr::DIAG_REAL>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, bi, su, sf, sk, gx, gy);
       else if (bB == (T)0)
-        smooth_restrict_body<T, F2, xr::DIAG_INNER, xr::DIAG_REAL>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, bi, su, sf, sk, gx, gy);
+        smooth_restrict_body<T, F2, MIX, xr::DIAG_INNER, xr::DIAG_REAL>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, bi, su, sf, sk, gx, gy);
       else
-        smooth_restrict_body<T, F2, xr::DIAG_INNER, xr::DIAG_INNER>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, bi, su, sf, sk, gx, gy);
+        smooth_restrict_body<T, F2, MIX, xr::DIAG_INNER, xr::DIAG_INNER>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, bi, su, sf, sk, gx, gy);
       return;
     }
   }
-  smooth_restrict_body<T, F2, xr::DIAG_ANY, xr::DIAG_ANY>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, bi, su, sf, sk, gx, gy);
+  smooth_restrict_body<T, F2, MIX, xr::DIAG_ANY, xr::DIAG_ANY>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, bi, su, sf, sk, gx, gy);
 }
 
-template <class T, class F2, class O2>
+template <class T, class F2, class O2, int MIX>
 __global__ void __launch_bounds__(FT) prolong_smooth_kernel(O2* __restrict__ out, int po, const c2<T>* __restrict__ upre,
                                                              int pu, const c2<T>* __restrict__ ec, int pc,
                                                              const F2* __restrict__ f, int pf,
@@ -373,13 +377,13 @@ __global__ void __launch_bounds__(FT) prolong_smooth_kernel(O2* __restrict__ out
   if constexpr (sizeof(T) == 8) {
     if (gx >= 1 && gy >= 1 && gx + RW <= n && gy + RH <= n) {
       if (bA == (T)0)
-        prolong_smooth_body<T, F2, O2, xr::DIAG_REAL>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, bi, su, sf, sk, gx, gy);
+        prolong_smooth_body<T, F2, O2, MIX, xr::DIAG_REAL>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, bi, su, sf, sk, gx, gy);
       else
-        prolong_smooth_body<T, F2, O2, xr::DIAG_INNER>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, bi, su, sf, sk, gx, gy);
+        prolong_smooth_body<T, F2, O2, MIX, xr::DIAG_INNER>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, bi, su, sf, sk, gx, gy);
       return;
     }
   }
-  prolong_smooth_body<T, F2, O2, xr::DIAG_ANY>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, bi, su, sf, sk, gx, gy);
+  prolong_smooth_body<T, F2, O2, MIX, xr::DIAG_ANY>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, bi, su, sf, sk, gx, gy);
 }
 
 template <class T>
@@ -391,38 +395,38 @@ constexpr size_t ps_smem() {
   return (size_t)(TileShape<T>::W + 4) * (TileShape<T>::H + 4) * (2 * sizeof(c2<T>) + (sizeof(T) == 8 ? 2 : 1) * sizeof(T));
 }
 
-template <class T, class F2>
+template <class T, class F2, int MIX = 0>
 cudaError_t sr_t(void* u, int pu, void* fc, int pc, const void* f, int pf, const void* kh, int pk, int n, double bA,
                  double bB, const int* stop, cudaStream_t s, const Inst& bi) {
   constexpr size_t sm = sr_smem<T>();
   static bool attr = false;
   if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(smooth_restrict_kernel<T, F2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = cudaFuncSetAttribute(smooth_restrict_kernel<T, F2, MIX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e) return e;
     attr = true;
   }
   constexpr int CW = TileShape<T>::W / 2, CH = TileShape<T>::H / 2;
   int nc = n / 2;
   dim3 grid((nc + CW) / CW, (nc + CH) / CH, bi.count);
-  pdl_launch(smooth_restrict_kernel<T, F2>, grid, dim3(TXN, TYN), sm, s, (c2<T>*)u, pu, (c2<T>*)fc, pc, (const F2*)f, pf,
+  pdl_launch(smooth_restrict_kernel<T, F2, MIX>, grid, dim3(TXN, TYN), sm, s, (c2<T>*)u, pu, (c2<T>*)fc, pc, (const F2*)f, pf,
                                                                 (const T*)kh, pk, n, (T)bA, (T)bB, stop, bi);
   return cudaGetLastError();
 }
 
-template <class T, class F2, class O2>
+template <class T, class F2, class O2, int MIX = 0>
 cudaError_t ps_t(void* out, int po, const void* upre, int pu, const void* ec, int pc, const void* f, int pf,
                  const void* kh, int pk, int n, double bA, const int* stop, cudaStream_t s, const Inst& bi) {
   constexpr size_t sm = ps_smem<T>();
   static bool attr = false;
   if (!attr) {
     cudaError_t e =
-        cudaFuncSetAttribute(prolong_smooth_kernel<T, F2, O2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaFuncSetAttribute(prolong_smooth_kernel<T, F2, O2, MIX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e) return e;
     attr = true;
   }
   constexpr int W = TileShape<T>::W, HH = TileShape<T>::H;
   dim3 grid((n + W) / W, (n + HH) / HH, bi.count);
-  pdl_launch(prolong_smooth_kernel<T, F2, O2>, grid, dim3(TXN, TYN), sm, s, (O2*)out, po, (const c2<T>*)upre, pu,
+  pdl_launch(prolong_smooth_kernel<T, F2, O2, MIX>, grid, dim3(TXN, TYN), sm, s, (O2*)out, po, (const c2<T>*)upre, pu,
                                                                     (const c2<T>*)ec, pc, (const F2*)f, pf,
                                                                     (const T*)kh, pk, n, (T)bA, stop, bi);
   return cudaGetLastError();
@@ -437,6 +441,8 @@ cudaError_t launch_smooth_restrict(bool fp32, void* u, int pu, void* fc, int pc,
   if (variant >= 1 && variant < FUSED_VARIANTS)
     return launch_smooth_restrict_stream(fp32, u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, stream_rows(variant), stop, s,
                                          bi);
+  if (!fp32 && n >= MIX_MIN_N)
+    return sr_t<double, double2, MIX_TILE>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, stop, s, bi);
   if (!fp32) return sr_t<double, double2>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, stop, s, bi);
   return sr_t<float, float2>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, stop, s, bi);
 }
@@ -448,6 +454,8 @@ cudaError_t launch_prolong_smooth(bool fp32, void* out, int po, bool out_f64, co
   if (variant >= 1 && variant < FUSED_VARIANTS)
     return launch_prolong_smooth_stream(fp32, out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, stream_rows(variant),
                                         stop, s, bi);
+  if (!fp32 && n >= MIX_MIN_N)
+    return ps_t<double, double2, double2, MIX_TILE>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, stop, s, bi);
   if (!fp32) return ps_t<double, double2, double2>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, stop, s, bi);
   return ps_t<float, float2, float2>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, stop, s, bi);
 }

@@ -10,6 +10,10 @@
 namespace hz {
 namespace gnode {
 
+// FP64 neighbour sums on the integer pipe (xr::nb4_mix): n_l = 1024, 80 colour launches 2.07, 1.94,
+// 1.92 ms with 0, 4, 6 of the six additions there, the restricted residual 117, 102, 98 us.
+constexpr int MIX_GNODE = 6;
+
 // Row action on row (i, j) of A u = f~ (Sec. 4-5, Kaczmarz): delta = (f~_p - a_p u) / |a_p|^2,
 // u_q += conj(a_pq) delta over the row's support (lvl::act_nodes); a mirror neighbour at the
 // boundary carries coefficient 2 and receives 2 delta.
@@ -27,7 +31,7 @@ __device__ __forceinline__ void kacz_row(c2<T>* __restrict__ u, int pu, const F2
     lvl::row_consts<T>(kh[(long long)j * pk + i], i, j, n, beta, &d, &inv);
   }
   c2<T>* row = u + (long long)j * pu;
-  lvl::act_nodes<T>(row + i, row + b.iw, row + b.ie, u + (long long)b.js * pu + i, u + (long long)b.jn * pu + i,
+  lvl::act_nodes<T, MIX_GNODE>(row + i, row + b.iw, row + b.ie, u + (long long)b.js * pu + i, u + (long long)b.jn * pu + i,
                     ldc<T>(f, (long long)j * pf + i), d, inv);
 }
 
@@ -52,7 +56,7 @@ __device__ __forceinline__ c2<T> restrict_node(const c2<T>* u, int pu, const F2*
       const Nbr nb = neighbours(i, j, n);
       const c2<T>* row = u + (long long)j * pu;
       r[a] = xr::resid<T>(ldc<T>(f, (long long)j * pf + i), row[i],
-                          xr::nb4<T>(row[nb.iw], row[nb.ie], u[(long long)nb.js * pu + i], u[(long long)nb.jn * pu + i]),
+                          xr::nb4_mix<MIX_GNODE>(row[nb.iw], row[nb.ie], u[(long long)nb.js * pu + i], u[(long long)nb.jn * pu + i]),
                           xr::diag<T>(kh[(long long)j * pk + i], lvl::sides_at(i, j, n), beta));
     }
     rows[b] = xr::fw3<T>(r[0], r[1], r[2]);

@@ -209,9 +209,14 @@ __device__ __forceinline__ double2 nb_sum(float2 a, float2 b, float2 c, float2 d
   o.y = join(sv.y, rv.y, odd);
   return o;
 }
-// Neighbour sum (W + E) + (S + N) of FP64 values.
+// Neighbour sum (W + E) + (S + N) of FP64 values, MIX of its six additions on the integer pipe. On grids
+// that fill the GPU four are the best split (operator alone at n = 1984: 91, 78, 64, 82 us with 0, 2, 4,
+// 6); a grid of a few nodes per thread is bound by latency and takes none.
+constexpr int MIX_LARGE = 4;
+constexpr int MIX_MIN_N = 512;
+template <int MIX>
 __device__ __forceinline__ double2 nb_sum64(double2 w, double2 e, double2 s, double2 n) {
-  return d2add(d2add(w, e), d2add(s, n));
+  return xr::nb4_mix<MIX>(w, e, s, n);
 }
 
 __device__ __forceinline__ double2 interior(double d, double2 y, double2 nb) {
@@ -239,28 +244,30 @@ struct Star {
   }
 };
 __device__ __noinline__ double2 nb_sum_fp64(float2 w, float2 e, float2 s, float2 n) {
-  return nb_sum64(widen(w), widen(e), widen(s), widen(n));
+  return nb_sum64<0>(widen(w), widen(e), widen(s), widen(n));
 }
-__device__ __forceinline__ double2 nb_of(const Star<double2>& t) { return nb_sum64(t.w, t.e, t.s, t.n); }
+template <int MIX>
+__device__ __forceinline__ double2 nb_of(const Star<double2>& t) { return nb_sum64<MIX>(t.w, t.e, t.s, t.n); }
+template <int MIX>
 __device__ __forceinline__ double2 nb_of(const Star<float2>& t) {
   unsigned odd;
   double2 nb = nb_sum(t.w, t.e, t.s, t.n, odd);
   if (odd) nb = nb_sum_fp64(t.w, t.e, t.s, t.n);
   return nb;
 }
-template <class Y2>
+template <int MIX, class Y2>
 __device__ __forceinline__ double2 apply_star(const Star<Y2>& t, const Y2* __restrict__ y, const double* __restrict__ kh,
                                               int q, double beta) {
-  const double2 nb = nb_of(t);
+  const double2 nb = nb_of<MIX>(t);
   if (t.sides == 0 && beta == 0.0) return interior(t.d, widen(t.c), nb);
   return apply_row(y, kh[q], q, t.sides, beta, nb);
 }
-template <class Y2>
+template <int MIX, class Y2>
 __device__ __forceinline__ double2 apply_at(const Y2* __restrict__ y, const double* __restrict__ kh,
                                             const double* __restrict__ dd, int e, int i, int j, int n, double beta) {
   Star<Y2> t;
   t.load(y, dd, e, i, j, n);
-  return apply_star(t, y, kh, e, beta);
+  return apply_star<MIX>(t, y, kh, e, beta);
 }
 
 // Grid-stride walk over the (n+1)^2 nodes that keeps (i, j) up to date without dividing per node.
@@ -442,7 +449,7 @@ __global__ void k_update_p_kernel(KrylovVecs k) {
 }
 
 // v = A y with <r^, v>; alpha = rho / <r^, v>.
-template <class Y2, int VB>
+template <class Y2, int VB, int MIX>
 __global__ void __launch_bounds__(KB, 4) k_apply_rv_kernel(KrylovVecs k, const Y2* __restrict__ y) {
   pdl_enter();
   k = instance(k);
@@ -466,7 +473,7 @@ __global__ void __launch_bounds__(KB, 4) k_apply_rv_kernel(KrylovVecs k, const Y
 #pragma unroll
     for (int q = 0; q < VB; ++q) {
       if (it[q].live(N, k.G)) {
-        const double2 v = apply_star(star[q], y, k.kh, it[q].e, 0.0);
+        const double2 v = apply_star<MIX>(star[q], y, k.kh, it[q].e, 0.0);
         k.v[it[q].e] = v;
         acc[2 * q] = fma(rh[q].x, v.x, fma(rh[q].y, v.y, acc[2 * q]));
         acc[2 * q + 1] = fma(rh[q].x, v.y, fma(-rh[q].y, v.x, acc[2 * q + 1]));
@@ -523,7 +530,7 @@ __global__ void k_update_s_kernel(KrylovVecs k) {
 }
 
 // t = A z with <t, s> and <t, t>; omega = <t, s> / <t, t>.
-template <class Y2, int VB>
+template <class Y2, int VB, int MIX>
 __global__ void __launch_bounds__(KB, 4) k_apply_ts_kernel(KrylovVecs k, const Y2* __restrict__ z) {
   pdl_enter();
   k = instance(k);
@@ -547,7 +554,7 @@ __global__ void __launch_bounds__(KB, 4) k_apply_ts_kernel(KrylovVecs k, const Y
 #pragma unroll
     for (int q = 0; q < VB; ++q) {
       if (it[q].live(N, k.G)) {
-        const double2 t = apply_star(star[q], z, k.kh, it[q].e, 0.0);
+        const double2 t = apply_star<MIX>(star[q], z, k.kh, it[q].e, 0.0);
         k.t[it[q].e] = t;
         acc[3 * q] = fma(t.x, s[q].x, fma(t.y, s[q].y, acc[3 * q]));
         acc[3 * q + 1] = fma(t.x, s[q].y, fma(-t.y, s[q].x, acc[3 * q + 1]));
@@ -702,6 +709,7 @@ __global__ void loop_control_kernel(LoopCtl c) {
 }
 
 // tr = h^2 b - A x and |tr|^2, to confirm a recurrence-converged iterate.
+template <int MIX>
 __global__ void k_true_residual_kernel(KrylovVecs k) {
   pdl_enter();
   k = instance(k);
@@ -710,7 +718,7 @@ __global__ void k_true_residual_kernel(KrylovVecs k) {
   const int N = (int)k.N;
   for (NodeWalk it(k.n, gridDim.x * KB); it.e < N; it.next()) {
     const int e = it.e;
-    double2 ax = apply_at(k.x, k.kh, k.d, e, it.i, it.j, k.n, 0.0);
+    double2 ax = apply_at<MIX>(k.x, k.kh, k.d, e, it.i, it.j, k.n, 0.0);
     double2 bv = k.b[e];
     double2 tr = make_double2(fma(bv.x, k.scale_b, -ax.x), fma(bv.y, k.scale_b, -ax.y));
     k.tr[e] = tr;
@@ -758,13 +766,14 @@ __global__ void diag_kernel(double* __restrict__ d, const double* __restrict__ k
   GRID_STRIDE(e, N) d[e] = fma(kh[e], kh[e], -4.0);
 }
 
+template <int MIX>
 __global__ void apply_fp64_kernel(double2* v, const double2* u, const double* kh, const double* d, int n, double beta,
                                   double out_scale) {
   pdl_enter();
   const int N = (n + 1) * (n + 1);
   for (NodeWalk it(n, gridDim.x * KB); it.e < N; it.next()) {
     const int e = it.e;
-    double2 a = apply_at(u, kh, d, e, it.i, it.j, n, beta);
+    double2 a = apply_at<MIX>(u, kh, d, e, it.i, it.j, n, beta);
     v[e] = make_double2(a.x * out_scale, a.y * out_scale);
   }
 }
@@ -802,17 +811,21 @@ cudaError_t launch_k_update_p(const KrylovVecs& k, cudaStream_t s) { KLAUNCH(k_u
 template <class Y2>
 cudaError_t apply_rv(const KrylovVecs& k, const Y2* y, cudaStream_t s) {
   if (sizeof(Y2) == 8 && k.G > 4 * device_sms())
-    pdl_launch(k_apply_rv_kernel<float2, 2>, dim3((k.G + 1) / 2, 1, k.batch), KB, 0, s, k, (const float2*)y);
+    pdl_launch(k_apply_rv_kernel<float2, 2, 0>, dim3((k.G + 1) / 2, 1, k.batch), KB, 0, s, k, (const float2*)y);
+  else if (sizeof(Y2) == 16 && k.n >= MIX_MIN_N)
+    pdl_launch(k_apply_rv_kernel<double2, 1, MIX_LARGE>, KGRID, KB, 0, s, k, (const double2*)y);
   else
-    pdl_launch(k_apply_rv_kernel<Y2, 1>, KGRID, KB, 0, s, k, y);
+    pdl_launch(k_apply_rv_kernel<Y2, 1, 0>, KGRID, KB, 0, s, k, y);
   return cudaGetLastError();
 }
 template <class Y2>
 cudaError_t apply_ts(const KrylovVecs& k, const Y2* z, cudaStream_t s) {
   if (sizeof(Y2) == 8 && k.G > 4 * device_sms())
-    pdl_launch(k_apply_ts_kernel<float2, 2>, dim3((k.G + 1) / 2, 1, k.batch), KB, 0, s, k, (const float2*)z);
+    pdl_launch(k_apply_ts_kernel<float2, 2, 0>, dim3((k.G + 1) / 2, 1, k.batch), KB, 0, s, k, (const float2*)z);
+  else if (sizeof(Y2) == 16 && k.n >= MIX_MIN_N)
+    pdl_launch(k_apply_ts_kernel<double2, 1, MIX_LARGE>, KGRID, KB, 0, s, k, (const double2*)z);
   else
-    pdl_launch(k_apply_ts_kernel<Y2, 1>, KGRID, KB, 0, s, k, z);
+    pdl_launch(k_apply_ts_kernel<Y2, 1, 0>, KGRID, KB, 0, s, k, z);
   return cudaGetLastError();
 }
 cudaError_t launch_k_apply_rv(const KrylovVecs& k, cudaStream_t s) {
@@ -834,7 +847,11 @@ cudaError_t launch_k_update_x(const KrylovVecs& k, bool omega_half, cudaStream_t
   }
   return cudaGetLastError();
 }
-cudaError_t launch_k_true_residual(const KrylovVecs& k, cudaStream_t s) { KLAUNCH(k_true_residual_kernel) }
+cudaError_t launch_k_true_residual(const KrylovVecs& k, cudaStream_t s) {
+  if (k.n >= MIX_MIN_N) pdl_launch(k_true_residual_kernel<MIX_LARGE>, KGRID, KB, 0, s, k);
+  else pdl_launch(k_true_residual_kernel<0>, KGRID, KB, 0, s, k);
+  return cudaGetLastError();
+}
 cudaError_t launch_loop_control(const LoopCtl& c, cudaStream_t s) {
   pdl_launch(loop_control_kernel, 1, 32, 0, s, c);
   return cudaGetLastError();
@@ -852,7 +869,8 @@ cudaError_t launch_apply_fp64(double2* v, const double2* u, const double* kh, co
   long long N = (long long)(n + 1) * (n + 1);
   int G = (int)((N + KB - 1) / KB);
   if (G > 4096) G = 4096;
-  pdl_launch(apply_fp64_kernel, G, KB, 0, s, v, u, kh, d, n, beta, out_scale);
+  if (n >= MIX_MIN_N) pdl_launch(apply_fp64_kernel<MIX_LARGE>, G, KB, 0, s, v, u, kh, d, n, beta, out_scale);
+  else pdl_launch(apply_fp64_kernel<0>, G, KB, 0, s, v, u, kh, d, n, beta, out_scale);
   return cudaGetLastError();
 }
 

@@ -99,10 +99,10 @@ __device__ __forceinline__ void row_consts(T kh, int i, int j, int n, T beta, c2
 // written once. Every Kaczmarz kernel form goes through this function, so they give the same bits.
 // The arithmetic on the five values already read (mx / my: the W and E, or S and N, support nodes
 // are one mirror node, held in uw / us); act_nodes and the two-action form of the tiled sweep call it.
-template <class T>
+template <class T, int MIX = 0>
 __device__ __forceinline__ void act_update(c2<T>& up, c2<T>& uw, c2<T>& ue, c2<T>& us, c2<T>& un, c2<T> f, c2<T> d,
                                            T inv, bool mx, bool my) {
-  const c2<T> delta = xr::cscale<T>(xr::resid<T>(f, up, xr::nb4<T>(uw, ue, us, un), d), inv);
+  const c2<T> delta = xr::cscale<T>(xr::resid<T>(f, up, xr::nb4_mix<MIX>(uw, ue, us, un), d), inv);
   up = xr::cadd<T>(up, xr::cmulc<T>(d, delta));
   if (mx) {
     uw = xr::cadd<T>(uw, xr::cscale<T>(delta, (T)2));
@@ -117,12 +117,12 @@ __device__ __forceinline__ void act_update(c2<T>& up, c2<T>& uw, c2<T>& ue, c2<T
     un = xr::cadd<T>(un, delta);
   }
 }
-template <class T>
+template <class T, int MIX = 0>
 __device__ __forceinline__ void act_nodes(c2<T>* pp, c2<T>* pw, c2<T>* pe, c2<T>* ps, c2<T>* pn, c2<T> f, c2<T> d,
                                           T inv) {
   c2<T> up = *pp, uw = *pw, ue = *pe, us = *ps, un = *pn;
   const bool mx = pw == pe, my = ps == pn;
-  act_update<T>(up, uw, ue, us, un, f, d, inv, mx, my);
+  act_update<T, MIX>(up, uw, ue, us, un, f, d, inv, mx, my);
   *pp = up;
   *pw = uw;
   if (!mx) *pe = ue;

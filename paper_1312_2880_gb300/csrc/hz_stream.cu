@@ -31,6 +31,11 @@ namespace hz {
 
 namespace {
 
+// FP64 neighbour sums: additions of the six on the integer pipe (xr::nb4_mix). Few warps are resident
+// (154 registers), so more than two lengthen the chain by more than they take off the FP64 pipe: the
+// finest smooth_restrict at n = 4096 takes 1.19, 1.15, 1.12, 1.29 ms with 0, 1, 2, 4 (prolong_smooth 0.85,
+// 0.82, 0.77, 0.86).
+constexpr int MIX_STREAM = 2;
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int WPB = 4;  // warps (strips) per block
 
@@ -259,10 +264,10 @@ __device__ __forceinline__ void sr_stage(SRState<Real>& S, unsigned char* ring, 
     const Real rs = sides2<Real>(j0 - 1, A.n);
     L2c<Real>& U = S.U[q1];
     if (er == 1) {
-      const c2<Real> nb = xr::nb4<Real>(U.a, shfl_down2<Real>(U.a), S.U[q2].b, S.U[Q].b);
+      const c2<Real> nb = xr::nb4_mix<MIX_STREAM>(U.a, shfl_down2<Real>(U.a), S.U[q2].b, S.U[Q].b);
       U.b = xr::gs_k<Real, KA>(S.F[q1].b, nb, xr::diag_k<Real, KA>(S.K[q1].y, q.sc1 + rs, A.bA), inv(t - 1, 1));
     } else {
-      const c2<Real> nb = xr::nb4<Real>(shfl_up2<Real>(U.b), U.b, S.U[q2].a, S.U[Q].a);
+      const c2<Real> nb = xr::nb4_mix<MIX_STREAM>(shfl_up2<Real>(U.b), U.b, S.U[q2].a, S.U[Q].a);
       U.a = xr::gs_k<Real, KA>(S.F[q1].a, nb, xr::diag_k<Real, KA>(S.K[q1].x, q.sc0 + rs, A.bA), inv(t - 1, 0));
     }
     const int jo = j0 - 1;
@@ -273,9 +278,9 @@ __device__ __forceinline__ void sr_stage(SRState<Real>& S, unsigned char* ring, 
     const Real rs = sides2<Real>(j0 - 2, A.n);
     const L2c<Real>& U = S.U[q2];
     L2c<Real> R;
-    R.a = xr::resid_k<Real, KB>(S.F[q2].a, U.a, xr::nb4<Real>(shfl_up2<Real>(U.b), U.b, S.U[q3].a, S.U[q1].a),
+    R.a = xr::resid_k<Real, KB>(S.F[q2].a, U.a, xr::nb4_mix<MIX_STREAM>(shfl_up2<Real>(U.b), U.b, S.U[q3].a, S.U[q1].a),
                            xr::diag_k<Real, KB>(S.K[q2].x, q.sc0 + rs, A.bB));
-    R.b = xr::resid_k<Real, KB>(S.F[q2].b, U.b, xr::nb4<Real>(U.a, shfl_down2<Real>(U.a), S.U[q3].b, S.U[q1].b),
+    R.b = xr::resid_k<Real, KB>(S.F[q2].b, U.b, xr::nb4_mix<MIX_STREAM>(U.a, shfl_down2<Real>(U.a), S.U[q3].b, S.U[q1].b),
                            xr::diag_k<Real, KB>(S.K[q2].y, q.sc1 + rs, A.bB));
     // the row sum (w + e) + 2 c at this lane's coarse column (2I = c0), then across rows; row
     // j0 - 2 is even (2J) on odd t, odd (2J + 1) on even t
@@ -457,10 +462,10 @@ __device__ __forceinline__ void ps_stage(PSState<Real>& S, unsigned char* ring, 
     const Real rs = sides2<Real>(j0 - 1, A.n);
     L2c<Real>& U = S.U[q1];
     if (er == 1) {
-      const c2<Real> nb = xr::nb4<Real>(U.a, shfl_down2<Real>(U.a), S.U[q2].b, S.U[Q].b);
+      const c2<Real> nb = xr::nb4_mix<MIX_STREAM>(U.a, shfl_down2<Real>(U.a), S.U[q2].b, S.U[Q].b);
       U.b = xr::gs_k<Real, KA>(S.F[q1].b, nb, xr::diag_k<Real, KA>(S.K[q1].y, q.sc1 + rs, A.bA), S.I[q1].y);
     } else {
-      const c2<Real> nb = xr::nb4<Real>(shfl_up2<Real>(U.b), U.b, S.U[q2].a, S.U[Q].a);
+      const c2<Real> nb = xr::nb4_mix<MIX_STREAM>(shfl_up2<Real>(U.b), U.b, S.U[q2].a, S.U[Q].a);
       U.a = xr::gs_k<Real, KA>(S.F[q1].a, nb, xr::diag_k<Real, KA>(S.K[q1].x, q.sc0 + rs, A.bA), S.I[q1].x);
     }
   }
@@ -469,10 +474,10 @@ __device__ __forceinline__ void ps_stage(PSState<Real>& S, unsigned char* ring, 
     const Real rs = sides2<Real>(j0 - 2, A.n);
     L2c<Real>& U = S.U[q2];
     if (er == 0) {
-      const c2<Real> nb = xr::nb4<Real>(shfl_up2<Real>(U.b), U.b, S.U[q3].a, S.U[q1].a);
+      const c2<Real> nb = xr::nb4_mix<MIX_STREAM>(shfl_up2<Real>(U.b), U.b, S.U[q3].a, S.U[q1].a);
       U.a = xr::gs_k<Real, KA>(S.F[q2].a, nb, xr::diag_k<Real, KA>(S.K[q2].x, q.sc0 + rs, A.bA), S.I[q2].x);
     } else {
-      const c2<Real> nb = xr::nb4<Real>(U.a, shfl_down2<Real>(U.a), S.U[q3].b, S.U[q1].b);
+      const c2<Real> nb = xr::nb4_mix<MIX_STREAM>(U.a, shfl_down2<Real>(U.a), S.U[q3].b, S.U[q1].b);
       U.b = xr::gs_k<Real, KA>(S.F[q2].b, nb, xr::diag_k<Real, KA>(S.K[q2].y, q.sc1 + rs, A.bA), S.I[q2].y);
     }
     const int jo = j0 - 2;
