@@ -398,17 +398,23 @@ bool kform_ok(const hz_problem* P, int l, int form) {
   return false;
 }
 // Default form: FP32 - one block if the level fits, else tiles, else (odd sweep counts) a cluster; FP64
-// - a cluster (the FP64 pipe of one SM bounds the one-block form), else tiles up to n_l = 512, else
-// colour launches (the tiles' halo recomputation is FP64 work, which outweighs the saved launches on
-// the largest levels). Measured per Bi-CGSTAB iteration (four passes): FP32 n_l = 128 cluster 114 us,
-// tiles 93 us; n_l = 256 215 and 105 us; FP64 n_l = 64 cluster 206 us,
-// colour launches 820 us; FP64 in the n = 4096 solve's graph: n_l = 1024 tiles 2.67 ms, colour
-// launches 2.39 ms; n_l = 512 0.94 and 1.21 ms; n_l = 256 0.58 and 0.92 ms. All forms give the
-// same bits.
+// - a cluster (the FP64 pipe of one SM bounds the one-block form) up to CLUSTER_BEST64 or, in a batch,
+// as far as it fits (its rows are acted on once, a tile's halo again by its neighbours), else tiles up to
+// TILE_MAX64, else colour launches (the halo's FP64 work outweighs the saved launches on the largest
+// levels). Measured per Bi-CGSTAB iteration (four passes): FP32 n_l = 128 cluster 114 us, tiles 93 us;
+// n_l = 256 215 and 105 us; FP64 n_l = 64 cluster 180 us, colour launches 880 us; FP64 iteration, cluster
+// and tiles: n_l = 128 681 and 712 us, 144 733 and 758, 160 845 and 822, 224 1297 and 994; in batches of
+// 16 n_l = 128 1.97 and 2.14 ms, 160 2.86 and 3.00, 224 4.92 and 4.87; FP64 tiles and colour launches:
+// n_l = 512 0.73 and 1.10 ms, 768 1.40 and 1.56, 1024 2.28 and 1.96 (a batch hides the launches: tiles up
+// to 512 there). All forms give the same bits.
 int default_kform(const hz_problem* P, int l) {
-  const int order32[] = {HZ_KACZ_LEVEL, HZ_KACZ_TILE, HZ_KACZ_CLUSTER}, order64[] = {HZ_KACZ_CLUSTER, HZ_KACZ_TILE};
-  const int* o = P->plan.fp32 ? order32 : order64;
-  const int cnt = P->plan.fp32 ? 3 : (P->lv[l].n <= 512 ? 2 : 1);
+  constexpr int CLUSTER_BEST64 = 144, TILE_MAX64 = 768, TILE_MAX64_BATCH = 512;
+  const bool one = P->plan.batch == 1;
+  const int n = P->lv[l].n;
+  const int order32[] = {HZ_KACZ_LEVEL, HZ_KACZ_TILE, HZ_KACZ_CLUSTER};
+  const int cluster_first[] = {HZ_KACZ_CLUSTER, HZ_KACZ_TILE}, tile_first[] = {HZ_KACZ_TILE, HZ_KACZ_CLUSTER};
+  const int* o = P->plan.fp32 ? order32 : one && n > CLUSTER_BEST64 ? tile_first : cluster_first;
+  const int cnt = P->plan.fp32 ? 3 : n <= (one ? TILE_MAX64 : TILE_MAX64_BATCH) ? 2 : 0;
   for (int q = 0; q < cnt; ++q)
     if (kform_ok(P, l, o[q])) return o[q];
   return HZ_KACZ_COLOUR;
@@ -436,8 +442,8 @@ cudaError_t kacz_tile_sweeps(hz_problem* P, int l, Src f, const void* first_in, 
   for (int k = 0; k < L.nu; ++k) {
     void* out = ((L.nu - 1 - k) % 2 == 0) ? L.u : L.u2;
     if ((e = mark(P, launch_kacz_sweep_tile64((double2*)out, L.pitch, (const double2*)in, L.pitch, (const double2*)f.f,
-                                              f.pf, (const double*)kh, pk, L.n, op_beta(P, L.relax_op), post, stop,
-                                              P->stream, bi),
+                                              f.pf, (const double*)kh, pk, L.n, op_beta(P, L.relax_op), post,
+                                              P->num_sms, stop, P->stream, bi),
                   HZ_K_KACZ_SWEEP, l)))
       return e;
     in = out;

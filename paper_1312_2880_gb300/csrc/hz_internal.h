@@ -135,9 +135,9 @@ cudaError_t launch_kacz_grid_pre(bool fp32, void* u, int pu, void* fc, int pc, c
 cudaError_t launch_kacz_grid_post(bool fp32, void* u, int pu, const void* ec, int pc, const void* f, int pf,
                                   const void* kh, int pk, int n, double bA, int nu, const int* stop, BandSync bs,
                                   cudaStream_t s);
-// One FP64 Kaczmarz sweep over halo tiles.
+// One FP64 Kaczmarz sweep over halo tiles; sms: the device's SM count (chooses the tile).
 cudaError_t launch_kacz_sweep_tile64(double2* uout, int po, const double2* uin, int pu, const double2* f, int pf,
-                                     const double* kh, int pk, int n, double bA, bool post, const int* stop,
+                                     const double* kh, int pk, int n, double bA, bool post, int sms, const int* stop,
                                      cudaStream_t s, const Inst& bi = Inst());
 // Coarse tail (hz_tail.cu): levels lt .. L-1 of the V-cycle in one block's shared memory.
 constexpr int TAIL_MAX_LEVELS = 12;

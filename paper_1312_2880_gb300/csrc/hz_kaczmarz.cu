@@ -44,8 +44,8 @@ struct TileGeo {
   static constexpr int HN = 6 * S_, HF = 10 * S_;  // halo rows on the near and the far side
   static constexpr int RX = KT_ + 2 * HX, RY = KT_ + HN + HF, REG = RX * RY;
 };
-using TileOne = TileGeo<32, 1, 256>;  // one sweep per launch: 44 x 48 regions
-constexpr size_t tile_smem() { return (size_t)TileOne::REG * (2 * sizeof(double2) + 2 * sizeof(double)); }
+template <class G>
+constexpr size_t tile_smem() { return (size_t)G::REG * (2 * sizeof(double2) + 2 * sizeof(double)); }
 
 // Actions of phase ph (of P = 5S; R = P - 1 - ph phases follow it) that can still reach the
 // tile's outputs. Propagating dependencies back from the outputs through the colour phases on an
@@ -274,15 +274,14 @@ __global__ void __launch_bounds__(LB) kacz_level_post_kernel(c2<T>* __restrict__
   lvl::for_nodes_blocked(n, [&](int, int i, int j, int p) { u[(long long)j * pu + i] = S.su[p]; });
 }
 
-template <bool POST>
-__global__ void __launch_bounds__(TileOne::TBK) kacz_sweep_tile64_kernel(double2* __restrict__ uout, int po,
+template <class G, bool POST>
+__global__ void __launch_bounds__(G::TBK) kacz_sweep_tile64_kernel(double2* __restrict__ uout, int po,
                                                                          const double2* __restrict__ uin, int pu,
                                                                          const double2* __restrict__ f, int pf,
                                                                          const double* __restrict__ kh, int pk, int n,
                                                                          double bA, const int* __restrict__ stop,
                                                                          Inst bi) {
   using T = double;
-  using G = TileOne;
   using PR = PhaseRect<G, POST>;
   static_assert(PR::fits(), "phase rectangles must keep their supports inside the tile region");
   constexpr int TBK = G::TBK, RX = G::RX, RY = G::RY, REG = G::REG, KT = G::KT;
@@ -597,27 +596,52 @@ cudaError_t launch_cluster_kernel(void (*kernel)(Args...), int c, size_t smem, c
 
 }  // namespace
 
-template <bool POST>
-cudaError_t tile_launch(double2* uout, int po, const double2* uin, int pu, const double2* f, int pf, const double* kh,
+template <class G, bool POST>
+cudaError_t tile_launch_t(double2* uout, int po, const double2* uin, int pu, const double2* f, int pf, const double* kh,
                         int pk, int n, double bA, const int* stop, cudaStream_t s, const Inst& bi) {
   static bool ready = false;
   if (!ready) {
-    cudaError_t e = cudaFuncSetAttribute(kacz_sweep_tile64_kernel<POST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)tile_smem());
+    cudaError_t e = cudaFuncSetAttribute(kacz_sweep_tile64_kernel<G, POST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)tile_smem<G>());
     if (e) return e;
     ready = true;
   }
-  const int t = (n + TileOne::KT) / TileOne::KT;
-  pdl_launch(kacz_sweep_tile64_kernel<POST>, dim3(t, t, bi.count), TileOne::TBK, tile_smem(), s, uout, po, uin, pu, f, pf,
+  const int t = (n + G::KT) / G::KT;
+  pdl_launch(kacz_sweep_tile64_kernel<G, POST>, dim3(t, t, bi.count), G::TBK, tile_smem<G>(), s, uout, po, uin, pu, f, pf,
              kh, pk, n, bA, stop, bi);
   return cudaGetLastError();
 }
 
+template <class G, class... A>
+cudaError_t tile_launch(bool post, A... args) {
+  return post ? tile_launch_t<G, true>(args...) : tile_launch_t<G, false>(args...);
+}
+
+// Tile edge: the sweep is bound by a tile's FP64 work (a warp instruction holds an SM's FP64 pipe about 77
+// cycles), so the smallest tile whose grid is at most one block per SM, which keeps every SM busy and
+// each one's work least; levels too large for that take 28, where two or three blocks share an SM and the
+// halo is still small. 16 sweeps (four passes) of 16, 20, 24, 28, 36, 44 in one wave: 278, 311, 377,
+// 410, 554, 730 us (32, the only edge before: 511, n_l = 512 in two waves 897); n_l = 768: 1888, 1601,
+// 1506, 1396, 1667, 1726 us (32: 1435).
+int tile64_edge(int n, int count, int sms) {
+  for (int k : {16, 20, 24, 28, 36, 44}) {
+    const long long t = (n + k) / k;
+    if (t * t * count <= sms) return k;
+  }
+  return 28;
+}
+
 cudaError_t launch_kacz_sweep_tile64(double2* uout, int po, const double2* uin, int pu, const double2* f, int pf,
-                                     const double* kh, int pk, int n, double bA, bool post, const int* stop,
+                                     const double* kh, int pk, int n, double bA, bool post, int sms, const int* stop,
                                      cudaStream_t s, const Inst& bi) {
-  return post ? tile_launch<true>(uout, po, uin, pu, f, pf, kh, pk, n, bA, stop, s, bi)
-              : tile_launch<false>(uout, po, uin, pu, f, pf, kh, pk, n, bA, stop, s, bi);
+  switch (tile64_edge(n, bi.count, sms)) {
+    case 16: return tile_launch<TileGeo<16, 1, 192>>(post, uout, po, uin, pu, f, pf, kh, pk, n, bA, stop, s, bi);
+    case 20: return tile_launch<TileGeo<20, 1, 256>>(post, uout, po, uin, pu, f, pf, kh, pk, n, bA, stop, s, bi);
+    case 24: return tile_launch<TileGeo<24, 1, 288>>(post, uout, po, uin, pu, f, pf, kh, pk, n, bA, stop, s, bi);
+    case 36: return tile_launch<TileGeo<36, 1, 256>>(post, uout, po, uin, pu, f, pf, kh, pk, n, bA, stop, s, bi);
+    case 44: return tile_launch<TileGeo<44, 1, 320>>(post, uout, po, uin, pu, f, pf, kh, pk, n, bA, stop, s, bi);
+    default: return tile_launch<TileGeo<28, 1, 352>>(post, uout, po, uin, pu, f, pf, kh, pk, n, bA, stop, s, bi);
+  }
 }
 
 namespace {
