@@ -325,6 +325,17 @@ __device__ __forceinline__ c2<T> fw_node(const c2<T>* r, int pr, int n, int I, i
   }
   return cscale<T>(fw3<T>(row[0], row[1], row[2]), (T)0.25);
 }
+// One component of fw_node<double>: r points at that component of the array's first value.
+__device__ __forceinline__ double fw_comp(const double* r, int pr, int n, int I, int J) {
+  const int w = 2 * reflect(2 * I - 1, n), c = 4 * I, e = 2 * reflect(2 * I + 1, n);
+  double row[3];
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    const double* rr = r + 2ll * reflect(2 * J + b - 1, n) * pr;
+    row[b] = fma(rr[c], 2.0, add(rr[w], rr[e]));
+  }
+  return mul(fma(row[1], 2.0, add(row[0], row[2])), 0.25);
+}
 // Bilinear interpolation of the coarse correction at fine node (2I + oi, 2J + oj) from coarse rows
 // e0 (J) and e1 (J + 1): coincident nodes copy, edge midpoints average two, centres four, in the
 // order ((e00 + e10) + (e01 + e11)) / 4.

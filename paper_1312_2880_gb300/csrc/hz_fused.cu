@@ -24,23 +24,20 @@ namespace {
 // FP64 neighbour sums on levels of at least MIX_MIN_N intervals: MIX_TILE of the six additions on the
 // integer pipe (xr::nb4_mix). n = 1024 smooth_restrict 118, 112, 107, 101 us with 0, 2, 4, 6 there, n = 512
 // 41, 38, 36, 34; smaller levels are bound by latency and lose (n = 64 FP64 solve 588 us with 0, 626 with 4).
-constexpr int MIX_TILE = 4, MIX_MIN_N = 256;
-constexpr int FT = 256;  // threads per block
+constexpr int MIX_TILE = 6, MIX_MIN_N = 256;
 
-// Owned fine nodes of a tile (W x H). FP64 tiles are small: the FP64 passes are bound by each
-// SM's FP64 pipe, so spreading a level over more blocks (and SMs) pays for the larger share of
-// halo nodes. Measured FP64 solves of the n = 512 wedge: 117.5 ms with 64 x 16 tiles everywhere,
+// Owned fine nodes of a tile (W x H) and threads of its block. FP64 tiles are small: the FP64 passes are
+// bound by each SM's FP64 pipe, so spreading a level over more blocks (and SMs) pays for the larger share
+// of halo nodes. Measured FP64 solves of the n = 512 wedge: 117.5 ms with 64 x 16 tiles everywhere,
 // 112.4 ms with 32 x 8 everywhere (116.9 and 121.6 ms with 32 x 8 only below n_l = 256 or 512).
-template <class T>
-struct TileShape;
-template <>
-struct TileShape<float> {
-  static constexpr int W = 64, H = 32;
+// TileFew: levels so small that its grid is one block per SM at most (few_tiles).
+template <int W_, int H_, int FT_>
+struct Tile {
+  static constexpr int W = W_, H = H_, FT = FT_;
 };
-template <>
-struct TileShape<double> {
-  static constexpr int W = 32, H = 8;
-};
+using Tile32 = Tile<64, 32, 256>;
+using Tile64 = Tile<32, 8, 256>;
+using TileFew = Tile<16, 4, 128>;
 
 __device__ __forceinline__ bool in_grid(int i, int j, int n) { return (unsigned)i <= (unsigned)n && (unsigned)j <= (unsigned)n; }
 
@@ -62,15 +59,16 @@ __device__ __forceinline__ c2<T> nb_sum(const c2<T>* s, int rw, int c, int r, in
 template <class T>
 __host__ __device__ constexpr bool interior_path() { return sizeof(T) == 4; }
 
-constexpr int TXN = 32, TYN = 8;
+constexpr int TXN = 32;
 
-template <class T, class F2>
+template <class T, class F2, class S>
 __device__ __forceinline__ void smooth_restrict_inner(c2<T>* __restrict__ u, int pu, c2<T>* __restrict__ fc, int pc,
                                                       const F2* __restrict__ f, int pf, const T* __restrict__ kh,
                                                       int pk, T bA, T bB, c2<T>* su, c2<T>* sf, T* sk, int gx,
                                                       int gy) {
-  constexpr int W = TileShape<T>::W, HH = TileShape<T>::H;
+  constexpr int W = S::W, HH = S::H;
   constexpr int RW = W + 5, RH = HH + 5;
+  constexpr int TYN = S::FT / TXN;
   const int tx = threadIdx.x, ty = threadIdx.y;
   for (int r = ty; r < RH; r += TYN) {
     const F2* fr = f + (long long)(gy + r) * pf + gx;
@@ -127,13 +125,14 @@ __device__ __forceinline__ void smooth_restrict_inner(c2<T>* __restrict__ u, int
   }
 }
 
-template <class T, class F2, class O2>
+template <class T, class F2, class O2, class S>
 __device__ __forceinline__ void prolong_smooth_inner(O2* __restrict__ out, int po, const c2<T>* __restrict__ upre,
                                                      int pu, const c2<T>* __restrict__ ec, int pc,
                                                      const F2* __restrict__ f, int pf, const T* __restrict__ kh,
                                                      int pk, T bA, c2<T>* su, c2<T>* sf, T* sk, int gx, int gy) {
-  constexpr int W = TileShape<T>::W, HH = TileShape<T>::H;
+  constexpr int W = S::W, HH = S::H;
   constexpr int RW = W + 4, RH = HH + 4;
+  constexpr int TYN = S::FT / TXN;
   const int tx = threadIdx.x, ty = threadIdx.y;
   for (int r = ty; r < RH; r += TYN) {
     const int j = gy + r, J = j >> 1, oj = j & 1;
@@ -178,17 +177,17 @@ __device__ __forceinline__ void prolong_smooth_inner(O2* __restrict__ out, int p
 
 // The general tile: every node tested against the grid (FP32 tiles at the boundary, all FP64 tiles).
 // KA, KB: kinds of the relaxation and residual diagonals (xr::DIAG_*); MIX: see MIX_TILE.
-template <class T, class F2, int MIX, int KA, int KB>
+template <class T, class F2, class S, int MIX, int KA, int KB>
 __device__ __forceinline__ void smooth_restrict_body(c2<T>* __restrict__ u, int pu, c2<T>* __restrict__ fc, int pc,
                                                      const F2* __restrict__ f, int pf, const T* __restrict__ kh,
                                                      int pk, int n, T bA, T bB, const Inst& bi, c2<T>* su, c2<T>* sf,
                                                      T* sk, int gx, int gy) {
-  constexpr int W = TileShape<T>::W, HH = TileShape<T>::H;
-  constexpr int RW = W + 5, RH = HH + 5, RN = RW * RH, HW = (RW + 1) / 2;
+  constexpr int W = S::W, HH = S::H;
+  constexpr int RW = W + 5, RH = HH + 5, RN = RW * RH, HW = (RW + 1) / 2, HB = (RW - 1) / 2;
   T* si = sk + (sizeof(T) == 8 ? RN : 0);  // FP64: the stored 1 / |d|^2
   const int x0 = gx + 3, y0 = gy + 3;
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-  for (int q = tid; q < RN; q += FT) {
+  for (int q = tid; q < RN; q += S::FT) {
     int r = q / RW, c = q - r * RW, i = gx + c, j = gy + r;
     if (in_grid(i, j, n)) {
       sf[q] = ldc<T>(f, (long long)j * pf + i);
@@ -198,7 +197,7 @@ __device__ __forceinline__ void smooth_restrict_body(c2<T>* __restrict__ u, int 
   }
   __syncthreads();
   // red nodes of the whole region: zero neighbours, u = f~ / d
-  for (int q = tid; q < RH * HW; q += FT) {
+  for (int q = tid; q < RH * HW; q += S::FT) {
     int r = q / HW, m = q - r * HW;
     int j = gy + r;
     int c = 2 * m + ((0 - gx - j) & 1);
@@ -210,12 +209,10 @@ __device__ __forceinline__ void smooth_restrict_body(c2<T>* __restrict__ u, int 
   }
   __syncthreads();
   // black nodes one in from the region edge
-  for (int q = tid; q < RH * HW; q += FT) {
-    int r = q / HW, m = q - r * HW;
-    int j = gy + r;
-    int c = 2 * m + ((1 - gx - j) & 1);
-    int i = gx + c;
-    if (r >= 1 && r <= RH - 2 && c >= 1 && c <= RW - 2 && in_grid(i, j, n)) {
+  for (int q = tid; q < (RH - 2) * HB; q += S::FT) {
+    const int rr = q / HB, m = q - rr * HB, r = rr + 1, j = gy + r;
+    const int c = 1 + 2 * m + ((gx + j) & 1), i = gx + c;
+    if (c <= RW - 2 && in_grid(i, j, n)) {
       Nbr b = neighbours(i, j, n);
       c2<T> s = nb_sum<T, MIX>(su, RW, c, r, i, j, n, gx, gy);
       su[r * RW + c] = xr::gs_k<T, KA>(sf[r * RW + c], s, xr::diag_k<T, KA>(sk[r * RW + c], (T)(2 * b.sides), bA), si[r * RW + c]);
@@ -223,15 +220,15 @@ __device__ __forceinline__ void smooth_restrict_body(c2<T>* __restrict__ u, int 
   }
   __syncthreads();
   // write the owned nodes; residual f~ - B u two in from the edge (into sf)
-  for (int q = tid; q < RN; q += FT) {
+  for (int q = tid; q < RN; q += S::FT) {
     int r = q / RW, c = q - r * RW, i = gx + c, j = gy + r;
     if (!in_grid(i, j, n)) continue;
     if (r >= 3 && r < 3 + HH && c >= 3 && c < 3 + W) u[(long long)j * pu + i] = su[q];
   }
   __syncthreads();
-  for (int q = tid; q < RN; q += FT) {
-    int r = q / RW, c = q - r * RW, i = gx + c, j = gy + r;
-    if (r >= 2 && r <= RH - 3 && c >= 2 && c <= RW - 3 && in_grid(i, j, n)) {
+  for (int t = tid; t < (RH - 4) * (RW - 4); t += S::FT) {
+    const int rr = t / (RW - 4), c = t - rr * (RW - 4) + 2, r = rr + 2, q = r * RW + c, i = gx + c, j = gy + r;
+    if (in_grid(i, j, n)) {
       Nbr b = neighbours(i, j, n);
       c2<T> s = nb_sum<T, MIX>(su, RW, c, r, i, j, n, gx, gy);
       sf[q] = xr::resid_k<T, KB>(sf[q], su[q], s, xr::diag_k<T, KB>(sk[q], (T)(2 * b.sides), bB));
@@ -240,24 +237,33 @@ __device__ __forceinline__ void smooth_restrict_body(c2<T>* __restrict__ u, int 
   __syncthreads();
   // full weighting onto the owned coarse nodes
   const int nc = n / 2;
-  for (int q = tid; q < (W / 2) * (HH / 2); q += FT) {
-    int J = y0 / 2 + q / (W / 2), I = x0 / 2 + q % (W / 2);
-    if (I > nc || J > nc) continue;
-    fc[(long long)J * pc + I] = xr::fw_node<T>(sf - gy * RW - gx, RW, n, I, J);
+  if constexpr (sizeof(T) == 8) {  // two lanes per node, one component each: half the chain on the FP64 pipe
+    for (int q = tid; q < 2 * (W / 2) * (HH / 2); q += S::FT) {
+      const int p = q >> 1, comp = q & 1, J = y0 / 2 + p / (W / 2), I = x0 / 2 + p % (W / 2);
+      if (I > nc || J > nc) continue;
+      reinterpret_cast<double*>(fc)[2 * ((long long)J * pc + I) + comp] =
+          xr::fw_comp(reinterpret_cast<const double*>(sf - gy * RW - gx) + comp, RW, n, I, J);
+    }
+  } else {
+    for (int q = tid; q < (W / 2) * (HH / 2); q += S::FT) {
+      int J = y0 / 2 + q / (W / 2), I = x0 / 2 + q % (W / 2);
+      if (I > nc || J > nc) continue;
+      fc[(long long)J * pc + I] = xr::fw_node<T>(sf - gy * RW - gx, RW, n, I, J);
+    }
   }
 }
 
-template <class T, class F2, class O2, int MIX, int KA>
+template <class T, class F2, class O2, class S, int MIX, int KA>
 __device__ __forceinline__ void prolong_smooth_body(O2* __restrict__ out, int po, const c2<T>* __restrict__ upre,
                                                     int pu, const c2<T>* __restrict__ ec, int pc,
                                                     const F2* __restrict__ f, int pf, const T* __restrict__ kh, int pk,
                                                     int n, T bA, const Inst& bi, c2<T>* su, c2<T>* sf, T* sk, int gx,
                                                     int gy) {
-  constexpr int W = TileShape<T>::W, HH = TileShape<T>::H;
-  constexpr int RW = W + 4, RH = HH + 4, RN = RW * RH, HW = RW / 2;
+  constexpr int W = S::W, HH = S::H;
+  constexpr int RW = W + 4, RH = HH + 4, RN = RW * RH, HB = (RW - 1) / 2;
   T* si = sk + (sizeof(T) == 8 ? RN : 0);  // FP64: the stored 1 / |d|^2
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-  for (int q = tid; q < RN; q += FT) {
+  for (int q = tid; q < RN; q += S::FT) {
     int r = q / RW, c = q - r * RW, i = gx + c, j = gy + r;
     if (in_grid(i, j, n)) {
       sf[q] = ldc<T>(f, (long long)j * pf + i);
@@ -268,7 +274,7 @@ __device__ __forceinline__ void prolong_smooth_body(O2* __restrict__ out, int po
   // u_pre + P e, one parity class (i mod 2, j mod 2) after the other (gx and gy are even), so that
   // a warp takes one interpolation case: a warp mixing the four cases would issue all of them
   constexpr int CE = (RW + 1) / 2, CO = RW / 2, RE = (RH + 1) / 2, RO = RH / 2;
-  for (int q = tid; q < RN; q += FT) {
+  for (int q = tid; q < RN; q += S::FT) {
     int oi, oj, t;
     if (q < CE * RE) { oi = 0; oj = 0; t = q; }
     else if (q < CE * RE + CO * RE) { oi = 1; oj = 0; t = q - CE * RE; }
@@ -283,12 +289,10 @@ __device__ __forceinline__ void prolong_smooth_body(O2* __restrict__ out, int po
   }
   __syncthreads();
   // black nodes one in from the region edge
-  for (int q = tid; q < RH * HW; q += FT) {
-    int r = q / HW, m = q - r * HW;
-    int j = gy + r;
-    int c = 2 * m + ((1 - gx - j) & 1);
-    int i = gx + c;
-    if (r >= 1 && r <= RH - 2 && c >= 1 && c <= RW - 2 && in_grid(i, j, n)) {
+  for (int q = tid; q < (RH - 2) * HB; q += S::FT) {
+    const int rr = q / HB, m = q - rr * HB, r = rr + 1, j = gy + r;
+    const int c = 1 + 2 * m + ((gx + j) & 1), i = gx + c;
+    if (c <= RW - 2 && in_grid(i, j, n)) {
       Nbr b = neighbours(i, j, n);
       c2<T> s = nb_sum<T, MIX>(su, RW, c, r, i, j, n, gx, gy);
       su[r * RW + c] = xr::gs_k<T, KA>(sf[r * RW + c], s, xr::diag_k<T, KA>(sk[r * RW + c], (T)(2 * b.sides), bA), si[r * RW + c]);
@@ -296,26 +300,24 @@ __device__ __forceinline__ void prolong_smooth_body(O2* __restrict__ out, int po
   }
   __syncthreads();
   // red nodes of the owned tile
-  for (int q = tid; q < RH * HW; q += FT) {
-    int r = q / HW, m = q - r * HW;
-    int j = gy + r;
-    int c = 2 * m + ((0 - gx - j) & 1);
-    int i = gx + c;
-    if (r >= 2 && r < 2 + HH && c >= 2 && c < 2 + W && in_grid(i, j, n)) {
+  for (int q = tid; q < HH * (W / 2); q += S::FT) {
+    const int rr = q / (W / 2), m = q - rr * (W / 2), r = rr + 2, j = gy + r;
+    const int c = 2 + 2 * m + ((gx + j) & 1), i = gx + c;
+    if (in_grid(i, j, n)) {
       Nbr b = neighbours(i, j, n);
       c2<T> s = nb_sum<T, MIX>(su, RW, c, r, i, j, n, gx, gy);
       su[r * RW + c] = xr::gs_k<T, KA>(sf[r * RW + c], s, xr::diag_k<T, KA>(sk[r * RW + c], (T)(2 * b.sides), bA), si[r * RW + c]);
     }
   }
   __syncthreads();
-  for (int q = tid; q < RN; q += FT) {
-    int r = q / RW, c = q - r * RW, i = gx + c, j = gy + r;
-    if (r >= 2 && r < 2 + HH && c >= 2 && c < 2 + W && in_grid(i, j, n)) stc<T>(out, (long long)j * po + i, su[q]);
+  for (int q = tid; q < HH * W; q += S::FT) {
+    const int r = q / W + 2, c = q % W + 2, i = gx + c, j = gy + r;
+    if (in_grid(i, j, n)) stc<T>(out, (long long)j * po + i, su[r * RW + c]);
   }
 }
 
-template <class T, class F2, int MIX>
-__global__ void __launch_bounds__(FT) smooth_restrict_kernel(c2<T>* __restrict__ u, int pu, c2<T>* __restrict__ fc,
+template <class T, class F2, class S, int MIX>
+__global__ void __launch_bounds__(S::FT) smooth_restrict_kernel(c2<T>* __restrict__ u, int pu, c2<T>* __restrict__ fc,
                                                               int pc, const F2* __restrict__ f, int pf,
                                                               const T* __restrict__ kh, int pk, int n, T bA, T bB,
                                                               const int* __restrict__ stop, Inst bi) {
@@ -324,7 +326,7 @@ __global__ void __launch_bounds__(FT) smooth_restrict_kernel(c2<T>* __restrict__
   u += blockIdx.z * bi.su;
   fc += blockIdx.z * bi.sc;
   f += blockIdx.z * bi.sf;
-  constexpr int W = TileShape<T>::W, HH = TileShape<T>::H;
+  constexpr int W = S::W, HH = S::H;
   constexpr int RW = W + 5, RH = HH + 5, RN = RW * RH;
   extern __shared__ __align__(16) unsigned char smem[];
   c2<T>* su = reinterpret_cast<c2<T>*>(smem);
@@ -333,25 +335,25 @@ __global__ void __launch_bounds__(FT) smooth_restrict_kernel(c2<T>* __restrict__
   const int x0 = blockIdx.x * W, y0 = blockIdx.y * HH;
   const int gx = x0 - 3, gy = y0 - 3;
   if (interior_path<T>() && gx >= 1 && gy >= 1 && gx + RW <= n && gy + RH <= n) {
-    smooth_restrict_inner<T, F2>(u, pu, fc, pc, f, pf, kh, pk, bA, bB, su, sf, sk, gx, gy);
+    smooth_restrict_inner<T, F2, S>(u, pu, fc, pc, f, pf, kh, pk, bA, bB, su, sf, sk, gx, gy);
     return;
   }
   if constexpr (sizeof(T) == 8) {
     if (gx >= 1 && gy >= 1 && gx + RW <= n && gy + RH <= n) {  // every node strictly inside the square
       if (bA == (T)0 && bB == (T)0)
-        smooth_restrict_body<T, F2, MIX, xr::DIAG_REAL, xr::DIAG_REAL>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, bi, su, sf, sk, gx, gy);
+        smooth_restrict_body<T, F2, S, MIX, xr::DIAG_REAL, xr::DIAG_REAL>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, bi, su, sf, sk, gx, gy);
       else if (bB == (T)0)
-        smooth_restrict_body<T, F2, MIX, xr::DIAG_INNER, xr::DIAG_REAL>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, bi, su, sf, sk, gx, gy);
+        smooth_restrict_body<T, F2, S, MIX, xr::DIAG_INNER, xr::DIAG_REAL>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, bi, su, sf, sk, gx, gy);
       else
-        smooth_restrict_body<T, F2, MIX, xr::DIAG_INNER, xr::DIAG_INNER>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, bi, su, sf, sk, gx, gy);
+        smooth_restrict_body<T, F2, S, MIX, xr::DIAG_INNER, xr::DIAG_INNER>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, bi, su, sf, sk, gx, gy);
       return;
     }
   }
-  smooth_restrict_body<T, F2, MIX, xr::DIAG_ANY, xr::DIAG_ANY>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, bi, su, sf, sk, gx, gy);
+  smooth_restrict_body<T, F2, S, MIX, xr::DIAG_ANY, xr::DIAG_ANY>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, bi, su, sf, sk, gx, gy);
 }
 
-template <class T, class F2, class O2, int MIX>
-__global__ void __launch_bounds__(FT) prolong_smooth_kernel(O2* __restrict__ out, int po, const c2<T>* __restrict__ upre,
+template <class T, class F2, class O2, class S, int MIX>
+__global__ void __launch_bounds__(S::FT) prolong_smooth_kernel(O2* __restrict__ out, int po, const c2<T>* __restrict__ upre,
                                                              int pu, const c2<T>* __restrict__ ec, int pc,
                                                              const F2* __restrict__ f, int pf,
                                                              const T* __restrict__ kh, int pk, int n, T bA,
@@ -362,7 +364,7 @@ __global__ void __launch_bounds__(FT) prolong_smooth_kernel(O2* __restrict__ out
   upre += blockIdx.z * bi.su;
   ec += blockIdx.z * bi.sc;
   f += blockIdx.z * bi.sf;
-  constexpr int W = TileShape<T>::W, HH = TileShape<T>::H;
+  constexpr int W = S::W, HH = S::H;
   constexpr int RW = W + 4, RH = HH + 4, RN = RW * RH;
   extern __shared__ __align__(16) unsigned char smem[];
   c2<T>* su = reinterpret_cast<c2<T>*>(smem);
@@ -371,65 +373,72 @@ __global__ void __launch_bounds__(FT) prolong_smooth_kernel(O2* __restrict__ out
   const int x0 = blockIdx.x * W, y0 = blockIdx.y * HH;
   const int gx = x0 - 2, gy = y0 - 2;
   if (interior_path<T>() && gx >= 1 && gy >= 1 && gx + RW <= n && gy + RH <= n) {
-    prolong_smooth_inner<T, F2, O2>(out, po, upre, pu, ec, pc, f, pf, kh, pk, bA, su, sf, sk, gx, gy);
+    prolong_smooth_inner<T, F2, O2, S>(out, po, upre, pu, ec, pc, f, pf, kh, pk, bA, su, sf, sk, gx, gy);
     return;
   }
   if constexpr (sizeof(T) == 8) {
     if (gx >= 1 && gy >= 1 && gx + RW <= n && gy + RH <= n) {
       if (bA == (T)0)
-        prolong_smooth_body<T, F2, O2, MIX, xr::DIAG_REAL>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, bi, su, sf, sk, gx, gy);
+        prolong_smooth_body<T, F2, O2, S, MIX, xr::DIAG_REAL>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, bi, su, sf, sk, gx, gy);
       else
-        prolong_smooth_body<T, F2, O2, MIX, xr::DIAG_INNER>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, bi, su, sf, sk, gx, gy);
+        prolong_smooth_body<T, F2, O2, S, MIX, xr::DIAG_INNER>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, bi, su, sf, sk, gx, gy);
       return;
     }
   }
-  prolong_smooth_body<T, F2, O2, MIX, xr::DIAG_ANY>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, bi, su, sf, sk, gx, gy);
+  prolong_smooth_body<T, F2, O2, S, MIX, xr::DIAG_ANY>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, bi, su, sf, sk, gx, gy);
 }
 
-template <class T>
+template <class T, class S>
 constexpr size_t sr_smem() {
-  return (size_t)(TileShape<T>::W + 5) * (TileShape<T>::H + 5) * (2 * sizeof(c2<T>) + (sizeof(T) == 8 ? 2 : 1) * sizeof(T));
+  return (size_t)(S::W + 5) * (S::H + 5) * (2 * sizeof(c2<T>) + (sizeof(T) == 8 ? 2 : 1) * sizeof(T));
 }
-template <class T>
+template <class T, class S>
 constexpr size_t ps_smem() {
-  return (size_t)(TileShape<T>::W + 4) * (TileShape<T>::H + 4) * (2 * sizeof(c2<T>) + (sizeof(T) == 8 ? 2 : 1) * sizeof(T));
+  return (size_t)(S::W + 4) * (S::H + 4) * (2 * sizeof(c2<T>) + (sizeof(T) == 8 ? 2 : 1) * sizeof(T));
 }
 
-template <class T, class F2, int MIX = 0>
+template <class T, class F2, class S, int MIX = 0>
 cudaError_t sr_t(void* u, int pu, void* fc, int pc, const void* f, int pf, const void* kh, int pk, int n, double bA,
                  double bB, const int* stop, cudaStream_t s, const Inst& bi) {
-  constexpr size_t sm = sr_smem<T>();
+  constexpr size_t sm = sr_smem<T, S>();
   static bool attr = false;
   if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(smooth_restrict_kernel<T, F2, MIX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = cudaFuncSetAttribute(smooth_restrict_kernel<T, F2, S, MIX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e) return e;
     attr = true;
   }
-  constexpr int CW = TileShape<T>::W / 2, CH = TileShape<T>::H / 2;
+  constexpr int CW = S::W / 2, CH = S::H / 2;
   int nc = n / 2;
   dim3 grid((nc + CW) / CW, (nc + CH) / CH, bi.count);
-  pdl_launch(smooth_restrict_kernel<T, F2, MIX>, grid, dim3(TXN, TYN), sm, s, (c2<T>*)u, pu, (c2<T>*)fc, pc, (const F2*)f, pf,
+  pdl_launch(smooth_restrict_kernel<T, F2, S, MIX>, grid, dim3(TXN, S::FT / TXN), sm, s, (c2<T>*)u, pu, (c2<T>*)fc, pc, (const F2*)f, pf,
                                                                 (const T*)kh, pk, n, (T)bA, (T)bB, stop, bi);
   return cudaGetLastError();
 }
 
-template <class T, class F2, class O2, int MIX = 0>
+template <class T, class F2, class O2, class S, int MIX = 0>
 cudaError_t ps_t(void* out, int po, const void* upre, int pu, const void* ec, int pc, const void* f, int pf,
                  const void* kh, int pk, int n, double bA, const int* stop, cudaStream_t s, const Inst& bi) {
-  constexpr size_t sm = ps_smem<T>();
+  constexpr size_t sm = ps_smem<T, S>();
   static bool attr = false;
   if (!attr) {
     cudaError_t e =
-        cudaFuncSetAttribute(prolong_smooth_kernel<T, F2, O2, MIX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaFuncSetAttribute(prolong_smooth_kernel<T, F2, O2, S, MIX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e) return e;
     attr = true;
   }
-  constexpr int W = TileShape<T>::W, HH = TileShape<T>::H;
+  constexpr int W = S::W, HH = S::H;
   dim3 grid((n + W) / W, (n + HH) / HH, bi.count);
-  pdl_launch(prolong_smooth_kernel<T, F2, O2, MIX>, grid, dim3(TXN, TYN), sm, s, (O2*)out, po, (const c2<T>*)upre, pu,
+  pdl_launch(prolong_smooth_kernel<T, F2, O2, S, MIX>, grid, dim3(TXN, S::FT / TXN), sm, s, (O2*)out, po, (const c2<T>*)upre, pu,
                                                                     (const c2<T>*)ec, pc, (const F2*)f, pf,
                                                                     (const T*)kh, pk, n, (T)bA, stop, bi);
   return cudaGetLastError();
+}
+
+// TileFew where its grid is at most one block per SM: latency bounds such levels, and a phase of a small
+// tile is one warp per FP64 pipe. n_l = 64 smooth_restrict 13.4 -> 11.2 us, prolong_smooth 11.1 -> 9.8 us;
+// n_l = 32 13.1 -> 10.6 and 11.2 -> 10.0 us.
+bool few_tiles(int n, int count) {
+  return (long long)((n + TileFew::W) / TileFew::W) * ((n + TileFew::H) / TileFew::H) * count <= device_sms();
 }
 
 }  // namespace
@@ -442,9 +451,11 @@ cudaError_t launch_smooth_restrict(bool fp32, void* u, int pu, void* fc, int pc,
     return launch_smooth_restrict_stream(fp32, u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, stream_rows(variant), stop, s,
                                          bi);
   if (!fp32 && n >= MIX_MIN_N)
-    return sr_t<double, double2, MIX_TILE>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, stop, s, bi);
-  if (!fp32) return sr_t<double, double2>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, stop, s, bi);
-  return sr_t<float, float2>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, stop, s, bi);
+    return sr_t<double, double2, Tile64, MIX_TILE>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, stop, s, bi);
+  if (!fp32 && few_tiles(n, bi.count))
+    return sr_t<double, double2, TileFew>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, stop, s, bi);
+  if (!fp32) return sr_t<double, double2, Tile64>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, stop, s, bi);
+  return sr_t<float, float2, Tile32>(u, pu, fc, pc, f, pf, kh, pk, n, bA, bB, stop, s, bi);
 }
 
 cudaError_t launch_prolong_smooth(bool fp32, void* out, int po, bool out_f64, const void* upre, int pu, const void* ec,
@@ -455,9 +466,11 @@ cudaError_t launch_prolong_smooth(bool fp32, void* out, int po, bool out_f64, co
     return launch_prolong_smooth_stream(fp32, out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, stream_rows(variant),
                                         stop, s, bi);
   if (!fp32 && n >= MIX_MIN_N)
-    return ps_t<double, double2, double2, MIX_TILE>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, stop, s, bi);
-  if (!fp32) return ps_t<double, double2, double2>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, stop, s, bi);
-  return ps_t<float, float2, float2>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, stop, s, bi);
+    return ps_t<double, double2, double2, Tile64, MIX_TILE>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, stop, s, bi);
+  if (!fp32 && few_tiles(n, bi.count))
+    return ps_t<double, double2, double2, TileFew>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, stop, s, bi);
+  if (!fp32) return ps_t<double, double2, double2, Tile64>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, stop, s, bi);
+  return ps_t<float, float2, float2, Tile32>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, stop, s, bi);
 }
 
 }  // namespace hz

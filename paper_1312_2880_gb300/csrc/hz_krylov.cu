@@ -780,7 +780,6 @@ __global__ void apply_fp64_kernel(double2* v, const double2* u, const double* kh
 
 }  // namespace
 
-namespace {
 int device_sms() {
   static int sms = 0;
   if (!sms) {
@@ -789,7 +788,6 @@ int device_sms() {
   }
   return sms;
 }
-}  // namespace
 
 #define KGRID dim3(k.G, 1, k.batch)
 #define KLAUNCH(name) pdl_launch(name, KGRID, KB, 0, s, k); return cudaGetLastError();
