@@ -5,7 +5,8 @@
 // latency, not by work, so this replaces 2 (L - lt) - 1 launches by one. Each level's operations
 // are the ones the per-level kernels perform (hz_level.cuh, fixed-rounding arithmetic), so the
 // result is bitwise the same as without the tail (one-sweep Gauss-Seidel levels and every
-// Kaczmarz form).
+// Kaczmarz form). In FP64 a cluster's other blocks help with the coarsest solve (coarse_cluster).
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -20,7 +21,62 @@ namespace {
 
 constexpr int TAIL_THREADS = 1024;
 
-template <class T>
+// The coarsest solve of the FP64 tail over a cluster: one SM's FP64 pipe (a warp instruction every 77
+// cycles or so) took 19 us for m = 81 rows of m columns, most of the tail. The tail's block and TAIL_CLUSTER - 1
+// helpers take ceil(m / TAIL_CLUSTER) rows each: the products of all columns at once, then the additions
+// in column order (lvl::coarse_row's bits), a lane per row and component. The helpers hold their rows of
+// the inverse before the right-hand side is there and do nothing else; two cluster barriers. The
+// tail of n_l = 16 and 8 37.7 -> 25.4 us.
+constexpr int TAIL_CLUSTER = 8;
+struct CoarseShare {  // shared-memory layout at off_ainv, inside the m * m cells of the whole inverse
+  int m, rows;
+  double2 *inv, *f;
+  double* prod;
+  __device__ CoarseShare(unsigned char* base, int m_) : m(m_), rows((m_ + TAIL_CLUSTER - 1) / TAIL_CLUSTER) {
+    inv = reinterpret_cast<double2*>(base);
+    f = inv + (size_t)m * rows;
+    prod = reinterpret_cast<double*>(f + m);
+  }
+};
+// one warp's lanes hold a block's rows, and the layout fits
+constexpr bool coarse_share_fits(int m) {
+  const int rows = (m + TAIL_CLUSTER - 1) / TAIL_CLUSTER;
+  return 2 * rows <= 32 && 2 * rows + 1 <= m;
+}
+__device__ __forceinline__ void coarse_fetch(const CoarseShare& S, const double2* __restrict__ ainvT, int rank) {
+  for (int t = threadIdx.x; t < S.m * S.rows; t += TAIL_THREADS) {
+    const int c = t / S.rows, r = min(rank * S.rows + t - c * S.rows, S.m - 1);
+    lvl::cp_async<sizeof(double2)>(S.inv + t, ainvT + (long long)c * S.m + r);
+  }
+}
+// u = A^-1 f of the tail's block (rank 0); every thread of the cluster takes part.
+__device__ __forceinline__ void coarse_cluster(const CoarseShare& S, double2* u, const double2* f) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank(), lanes = 2 * S.rows;
+  cl.sync();  // f is there
+  const double2* f0 = cl.map_shared_rank(const_cast<double2*>(f), 0);
+  for (int q = threadIdx.x; q < S.m; q += TAIL_THREADS) S.f[q] = f0[q];
+  __syncthreads();
+  for (int t = threadIdx.x; t < S.m * lanes; t += TAIL_THREADS) {  // xr::cmul's components
+    const int c = t / lanes, x = t - c * lanes, comp = x & 1;
+    const double2 a = S.inv[c * S.rows + (x >> 1)], v = S.f[c];
+    const double p = xr::mul(a.y, comp ? v.x : v.y);
+    S.prod[t] = xr::fma(a.x, comp ? v.y : v.x, comp ? p : -p);
+  }
+  __syncthreads();
+  const int row = rank * S.rows + (int)(threadIdx.x >> 1);
+  if ((int)threadIdx.x < lanes && row < S.m) {
+    double acc = 0.0;
+#pragma unroll 8
+    for (int c = 0; c < S.m; ++c) acc = xr::add(acc, S.prod[c * lanes + threadIdx.x]);
+    reinterpret_cast<double*>(cl.map_shared_rank(u, 0) + row)[threadIdx.x & 1] = acc;
+  }
+  cl.sync();  // u is there
+}
+
+// CL: the block and its helpers form a cluster (coarse_cluster).
+template <class T, bool CL>
 __device__ __forceinline__ void tail_body(const TailArgs& A, const int* __restrict__ stop, const Inst& bi) {
   extern __shared__ __align__(16) unsigned char smem[];
   const c2<T>* fin = reinterpret_cast<const c2<T>*>(A.f_in) + blockIdx.z * bi.sf;
@@ -41,6 +97,19 @@ __device__ __forceinline__ void tail_body(const TailArgs& A, const int* __restri
     else
       fn(lvl::Natural{nl + 1});
   };
+
+  if constexpr (CL) {
+    const CoarseShare S(smem + A.off_ainv, (A.lv[last].n + 1) * (A.lv[last].n + 1));
+    const int rank = (int)cooperative_groups::this_cluster().block_rank();
+    coarse_fetch(S, reinterpret_cast<const c2<T>*>(A.ainvT), rank);
+    if (rank > 0) {
+      lvl::cp_async_wait_all();
+      pdl_enter();
+      if (stop && stop[blockIdx.z * bi.stop_stride]) return;  // the whole cluster
+      coarse_cluster(S, U(last), F(last));
+      return;
+    }
+  }
 
   // Before the wait for the preceding kernel, everything that does not depend on it, so that with
   // programmatic dependent launch it overlaps that kernel: k H of every relaxation level (set up
@@ -66,7 +135,7 @@ __device__ __forceinline__ void tail_body(const TailArgs& A, const int* __restri
     }
   }
   const int mc = (A.lv[last].n + 1) * (A.lv[last].n + 1);
-  if (A.off_ainv) {  // the coarsest inverse, when it fits
+  if (!CL && A.off_ainv) {  // the coarsest inverse, when it fits
     const c2<T>* src = reinterpret_cast<const c2<T>*>(A.ainvT);
     c2<T>* dst = reinterpret_cast<c2<T>*>(smem + A.off_ainv);
     for (int q = threadIdx.x; q < mc * mc; q += TAIL_THREADS) lvl::cp_async<sizeof(c2<T>)>(dst + q, src + q);
@@ -126,7 +195,9 @@ __device__ __forceinline__ void tail_body(const TailArgs& A, const int* __restri
   }
 
   // coarsest: u = A^-1 f
-  {
+  if constexpr (CL) {
+    coarse_cluster(CoarseShare(smem + A.off_ainv, mc), U(last), F(last));
+  } else {
     const int m = (A.lv[last].n + 1) * (A.lv[last].n + 1);
     const c2<T>* ainvT = A.off_ainv ? reinterpret_cast<const c2<T>*>(smem + A.off_ainv)
                                     : reinterpret_cast<const c2<T>*>(A.ainvT);
@@ -156,10 +227,13 @@ __device__ __forceinline__ void tail_body(const TailArgs& A, const int* __restri
 // The FP32 tail is held to 56 registers a thread, so that its 1024-thread block fits beside the
 // deferred solution update (k_update_x, one 128-thread block per SM) that runs during the cycle.
 __global__ void __maxnreg__(56) tail_kernel32(const TailArgs A, const int* __restrict__ stop, Inst bi) {
-  tail_body<float>(A, stop, bi);
+  tail_body<float, false>(A, stop, bi);
 }
 __global__ void __launch_bounds__(TAIL_THREADS) tail_kernel64(const TailArgs A, const int* __restrict__ stop, Inst bi) {
-  tail_body<double>(A, stop, bi);
+  tail_body<double, false>(A, stop, bi);
+}
+__global__ void __launch_bounds__(TAIL_THREADS) tail_cluster_kernel(const TailArgs A, const int* __restrict__ stop, Inst bi) {
+  tail_body<double, true>(A, stop, bi);
 }
 
 }  // namespace
@@ -205,8 +279,34 @@ size_t tail_layout(bool fp32, TailArgs* A) {
 
 cudaError_t launch_tail(bool fp32, const TailArgs& A, size_t smem, const int* stop, cudaStream_t s, const Inst& bi) {
   if (A.count < 2 || A.count > TAIL_MAX_LEVELS || smem > (size_t)TAIL_MAX_SMEM) return cudaErrorInvalidValue;
-  static bool ready[2] = {false, false};
+  static bool ready[3] = {false, false, false};
   cudaError_t e;
+  const int m = (A.lv[A.count - 1].n + 1) * (A.lv[A.count - 1].n + 1);
+  // A cluster while its blocks are one wave (a block of the tail takes an SM) and there is something to
+  // share: tails of n_l = 8, 4 (m = 25) 23.2 us in one block, 19.1 with helpers, 10, 5 (m = 36) 25.2 and
+  // 20.1, 14, 7 (m = 64) 31.4 and 21.9. A batch of more instances fills the SMs with its own tails.
+  if (!fp32 && A.off_ainv && m >= 25 && coarse_share_fits(m) && TAIL_CLUSTER * bi.count <= device_sms()) {
+    if (!ready[2]) {
+      e = cudaFuncSetAttribute(tail_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TAIL_MAX_SMEM);
+      if (e) return e;
+      ready[2] = true;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(TAIL_CLUSTER, 1, bi.count);
+    cfg.blockDim = dim3(TAIL_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = TAIL_CLUSTER;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, tail_cluster_kernel, A, stop, bi);
+  }
   if (!ready[fp32]) {
     e = fp32 ? cudaFuncSetAttribute(tail_kernel32, cudaFuncAttributeMaxDynamicSharedMemorySize, TAIL_MAX_SMEM)
              : cudaFuncSetAttribute(tail_kernel64, cudaFuncAttributeMaxDynamicSharedMemorySize, TAIL_MAX_SMEM);
