@@ -58,7 +58,9 @@ def kernel_bytes_per_node(kernel: str, fp32: bool) -> float:
         "gs_first": c / 2 + r / 2 + c,
         "gs_colour": (c + c + r + c) / 2,
         "kacz_colour": (5 * c * 2 + c + r) / 5,
-        "kacz_sweep": c + c + r + c,               # u in, f, k h; u out
+        # FP32: a whole pass a launch, the mean of pre (f, k h; u, coarse f) and post (u, coarse e, f, k h; u);
+        # FP64: one sweep a launch (u in, f, k h; u out)
+        "kacz_sweep": (5 * c + c / 2 + 2 * r) / 2 if fp32 else c + c + r + c,
         "restrict_residual": c + c + r + c / 4,
         "prolong_add": 2 * c + c / 4,
         "export": 2 * c,
@@ -72,10 +74,12 @@ def kernel_bytes_per_node(kernel: str, fp32: bool) -> float:
     return table.get(kernel, 0.0)
 
 
-# FP64 work per node of the Krylov kernels: (flops with an FMA counted 2, FP64-pipe instructions).
-# The operator on an interior node: 3 complex adds (6), d = (kh)^2 - 4 (1 FMA), v = nb + d y (2 FMA).
-KRYLOV_FP64 = {"k_update_p": (16, 8), "k_apply_rv": (20, 13), "k_update_s": (12, 6), "k_apply_ts": (24, 15),
-               "k_update_r": (20, 10), "k_update_x": (8, 4)}
+# FP64 work per node of the Krylov kernels: (flops with an FMA counted 2, FP64-pipe instructions in the
+# FP32 form, in the FP64 form). The operator on an interior node: 3 complex adds (6, on the FP32 and integer
+# pipes in the FP32 form, four of them on the integer pipe in the FP64 form from n = 512 on), v = nb + d y
+# (2 FMA; d = (kh)^2 - 4 is stored).
+KRYLOV_FP64 = {"k_update_p": (16, 8, 8), "k_apply_rv": (18, 6, 8), "k_update_s": (12, 6, 6),
+               "k_apply_ts": (22, 8, 10), "k_update_r": (20, 10, 10), "k_update_x": (8, 4, 4)}
 
 
 def load_peaks():
@@ -266,7 +270,7 @@ def roofline(per, fp32: bool, hbm_peak: float, peak_kind: str, n: int, fp64_peak
     nodes = ((n >> level) + 1) ** 2
     gbs = kernel_bytes_per_node(name, fp32) * nodes / (avg_ms * 1e-3) / 1e9
     if name.startswith("k_") and fp64_peak:
-        flops, instr = KRYLOV_FP64[name]
+        flops, instr = KRYLOV_FP64[name][0], KRYLOV_FP64[name][1 if fp32 else 2]
         secs = avg_ms * 1e-3
         achieved = 2 * instr * nodes / secs / 1e12
         peak = fp64_peak["tflops"]

@@ -91,14 +91,16 @@ typedef struct {
                        tiles); 0 = shared-memory tiles; 1..8 = register streaming with 2^v rows
                        per warp. Every form gives the same bits. */
   int coarse_tail;  /* 1 (default): the smallest levels, from the first whose whole V-cycle below it
-                       fits one block's shared memory down to the coarsest, run as one launch (same
+                       fits one block's shared memory (FP32: with at most 256 unknowns on the coarsest
+                       level; FP64: from n_l = 16 down) to the coarsest, run as one launch (same
                        operations, same results as the per-level kernels for one-sweep Gauss-Seidel
-                       and FP32 Kaczmarz levels); 0: one or more launches per level */
+                       and Kaczmarz levels); 0: one or more launches per level */
   int kacz_form;    /* how Kaczmarz levels below the finest run (hz_kacz_form): -1 (default) = one
                        block if the level fits its shared memory, else tiles (even sweep counts), else a
-                       thread-block cluster, else colour launches in the FP32 form; a cluster, else
-                       tiles up to n_l = 512, else colour launches in the FP64 form. A form that does not apply to a level
-                       falls back to that default. */
+                       thread-block cluster, else colour launches in the FP32 form; in the FP64 form a
+                       cluster up to n_l = 144 (in a batch: as far as the level fits), else tiles up to
+                       n_l = 768 (in a batch: 512), else colour launches. A form that does not apply
+                       to a level falls back to that default. */
   int gs_smoother;  /* smoother of the levels the rules of Sec. 5 give Gauss-Seidel: HZ_SMOOTH_GS
                        (default, red-black), HZ_SMOOTH_JACOBI (damped) or HZ_SMOOTH_SOR (red-black,
                        over-relaxed) -- the alternatives the remark of Sec. 4 names. Jacobi and SOR
