@@ -11,7 +11,8 @@ namespace hz {
 namespace gnode {
 
 // FP64 neighbour sums on the integer pipe (xr::nb4_mix): n_l = 1024, 80 colour launches 2.07, 1.94,
-// 1.92 ms with 0, 4, 6 of the six additions there, the restricted residual 117, 102, 98 us.
+// 1.92 ms with 0, 4, 6 of the six additions there, the restricted residual 117, 102, 98 us (with a
+// thread per coarse node).
 constexpr int MIX_GNODE = 6;
 
 // Row action on row (i, j) of A u = f~ (Sec. 4-5, Kaczmarz): delta = (f~_p - a_p u) / |a_p|^2,
