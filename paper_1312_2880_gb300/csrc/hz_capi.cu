@@ -25,6 +25,7 @@ constexpr int HIST_CAP = 32768;       // device history entries (two per iterati
 constexpr int MAX_COARSE_UNKNOWNS = 1089;
 constexpr int PARTIAL_SLOTS = 4;
 constexpr int MAX_G = 16384;
+constexpr int VEC_SLOTS = 9;           // Krylov vectors with a slot of their own (t and tr: make_plan)
 
 // Scale bins in c = k_ref H: geometric midpoints between the paper's scales 0.3125, 0.625, 1.25
 // and 2.5 (Sec. 4-5), and the guard band 1 < kH < 2 sqrt 2 for L relaxation.
@@ -61,13 +62,11 @@ struct Plan {
   size_t total = 0;
   // offsets
   std::vector<size_t> off_kh, off_u, off_f, off_u2, off_inv;
-  size_t off_kh64 = 0, off_d = 0, off_vec = 0, vec_bytes = 0, off_ainv = 0, off_work = 0, off_state = 0, off_partials = 0,
-         off_hist = 0, off_status = 0, off_sync = 0, sync_bytes = 0;
-  int nvec = 11;
+  size_t off_kh64 = 0, off_d = 0, off_vec = 0, vec_bytes = 0, off_t = 0, off_ainv = 0, off_work = 0, off_state = 0,
+         off_partials = 0, off_hist = 0, off_status = 0, off_sync = 0, sync_bytes = 0;
   int m_coarse = 0;
   int batch = 1;
   std::vector<long long> ls;  // elements between instances of a level's arrays
-  size_t rhat_bytes = 0;
 };
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -121,9 +120,9 @@ bool make_plan(int n, const hz_hierarchy_opts& o, Plan* P, std::string* err) {
       P->off_inv[l] = off;
       off = align256(off + cells * 8);
     }
-    P->off_u[l] = off;
-    off = align256(off + cells * ce * B);
     if (l > 0) {
+      P->off_u[l] = off;
+      off = align256(off + cells * ce * B);
       P->off_f[l] = off;
       off = align256(off + cells * ce * B);
       P->off_u2[l] = off;  // out-of-place result of the fused post-smoothing pass
@@ -139,14 +138,18 @@ bool make_plan(int n, const hz_hierarchy_opts& o, Plan* P, std::string* err) {
   P->off_d = off;
   off = align256(off + N * 8);
   P->vec_bytes = align256(N * 16 * B);  // one slot: B consecutive vectors
-  P->rhat_bytes = P->vec_bytes;          // one shadow residual per instance (restarts renew it)
   P->off_vec = off;
-  off += P->vec_bytes * (P->nvec - 1) + P->rhat_bytes;
+  off += P->vec_bytes * VEC_SLOTS;
+  // Krylov vector t, which a V-cycle never overlaps (it lives from the operator pass that forms it to the
+  // update of r): the finest level's correction u has its place.
+  P->off_t = P->off_u[0] = off;
+  off += std::max(P->vec_bytes, align256((size_t)P->ls[0] * ce * B));
+  // The scratch of the coarsest inverse is set-up's alone: the vectors' place.
   P->m_coarse = (nc + 1) * (nc + 1);
+  P->off_work = P->off_vec;
+  off = std::max(off, align256(P->off_work + (size_t)P->m_coarse * P->m_coarse * 2 * 16));
   P->off_ainv = off;
   off = align256(off + (size_t)P->m_coarse * P->m_coarse * ce);
-  P->off_work = off;
-  off = align256(off + (size_t)P->m_coarse * P->m_coarse * 2 * 16);
   P->off_state = off;
   off = align256(off + sizeof(KState) * B);
   P->off_partials = off;
@@ -1387,11 +1390,11 @@ hz_status hz_setup_hierarchy(hz_problem* P, const hz_hierarchy_opts* opts, void*
   }
   // Krylov vectors and scratch.
   KrylovVecs& k = P->kv;
-  unsigned char* vb = A + pl.off_vec;
-  k.rhat = (double2*)vb;
-  vb += pl.rhat_bytes;
-  double2** slots[] = {&k.r, &k.p, &k.v, &k.s, &k.t, &k.y, &k.z, &k.tr, &P->b_int, &P->x_int};
-  for (int q = 0; q < pl.nvec - 1; ++q) *slots[q] = (double2*)(vb + q * pl.vec_bytes);
+  double2** slots[] = {&k.rhat, &k.r, &k.p, &k.v, &k.s, &k.y, &k.z, &P->b_int, &P->x_int};
+  static_assert(sizeof(slots) / sizeof(slots[0]) == VEC_SLOTS, "a slot each");
+  for (int q = 0; q < VEC_SLOTS; ++q) *slots[q] = (double2*)(A + pl.off_vec + q * pl.vec_bytes);
+  k.t = (double2*)(A + pl.off_t);
+  k.tr = k.s;  // formed when the iteration has stopped: s is rewritten before its next use
   k.x = nullptr;
   k.b = nullptr;
   const long long Nn = (long long)(n + 1) * (n + 1);
@@ -1995,8 +1998,8 @@ static size_t ray_layout(int n, int m, RayBlocks* B, double2** ph, unsigned char
   B->y = (double2*)take(vec);
   B->e = (double2*)take(vec);
   B->dz = (double2*)take(vec);
-  B->fcol = (double2*)take(sizeof(double2) * 2 * Bs);
-  B->perm = (int*)take(sizeof(int) * 2 * Bs);
+  B->fcol = B->e;         // 2 Bs: the factorisation's scratch, before any solve (Nr >= 2)
+  B->perm = (int*)B->dz;  // 2 Bs
   B->status = (int*)take(sizeof(int));
   *ph = (double2*)take(sizeof(double2) * 8 * (size_t)(n + 1) * (n + 1));
   return off;
