@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include "hz_common.cuh"
+#include "hz_host.h"
 #include "hz_internal.h"
 
 namespace hz {
@@ -401,12 +402,11 @@ template <class T, class F2, class S, int MIX = 0>
 cudaError_t sr_t(void* u, int pu, void* fc, int pc, const void* f, int pf, const void* kh, int pk, int n, double bA,
                  double bB, const int* stop, cudaStream_t s, const Inst& bi) {
   constexpr size_t sm = sr_smem<T, S>();
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(smooth_restrict_kernel<T, F2, S, MIX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e) return e;
-    attr = true;
-  }
+  static OncePerDevice opt_in;
+  const cudaError_t e = opt_in([] {
+    return cudaFuncSetAttribute(smooth_restrict_kernel<T, F2, S, MIX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  });
+  if (e) return e;
   constexpr int CW = S::W / 2, CH = S::H / 2;
   int nc = n / 2;
   dim3 grid((nc + CW) / CW, (nc + CH) / CH, bi.count);
@@ -419,13 +419,11 @@ template <class T, class F2, class O2, class S, int MIX = 0>
 cudaError_t ps_t(void* out, int po, const void* upre, int pu, const void* ec, int pc, const void* f, int pf,
                  const void* kh, int pk, int n, double bA, const int* stop, cudaStream_t s, const Inst& bi) {
   constexpr size_t sm = ps_smem<T, S>();
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e =
-        cudaFuncSetAttribute(prolong_smooth_kernel<T, F2, O2, S, MIX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e) return e;
-    attr = true;
-  }
+  static OncePerDevice opt_in;
+  const cudaError_t e = opt_in([] {
+    return cudaFuncSetAttribute(prolong_smooth_kernel<T, F2, O2, S, MIX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  });
+  if (e) return e;
   constexpr int W = S::W, HH = S::H;
   dim3 grid((n + W) / W, (n + HH) / HH, bi.count);
   pdl_launch(prolong_smooth_kernel<T, F2, O2, S, MIX>, grid, dim3(TXN, S::FT / TXN), sm, s, (O2*)out, po, (const c2<T>*)upre, pu,

@@ -292,7 +292,6 @@ struct KrylovVecs {
 // The vectors and state of instance b (host side, for launches that touch a single instance).
 KrylovVecs instance_of(const KrylovVecs& k, int b);
 
-int device_sms();  // SMs of the current device
 cudaError_t launch_k_init(const KrylovVecs& k, double tol, int maxit, int hist_cap, cudaStream_t s);
 cudaError_t launch_k_update_p(const KrylovVecs& k, cudaStream_t s);
 cudaError_t launch_k_apply_rv(const KrylovVecs& k, cudaStream_t s);

@@ -24,6 +24,7 @@
 #include <utility>
 
 #include "hz_common.cuh"
+#include "hz_host.h"
 #include "hz_internal.h"
 #include "hz_level.cuh"
 
@@ -352,14 +353,14 @@ size_t level_smem(int n) {
 
 template <class T>
 cudaError_t set_level_attr() {
-  static bool done = false;
-  if (done) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(kacz_level_pre_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       KACZ_LEVEL_MAX_SMEM);
-  if (e) return e;
-  e = cudaFuncSetAttribute(kacz_level_post_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, KACZ_LEVEL_MAX_SMEM);
-  if (!e) done = true;
-  return e;
+  static OncePerDevice opt_in;
+  return opt_in([] {
+    cudaError_t e = cudaFuncSetAttribute(kacz_level_pre_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         KACZ_LEVEL_MAX_SMEM);
+    if (!e)
+      e = cudaFuncSetAttribute(kacz_level_post_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, KACZ_LEVEL_MAX_SMEM);
+    return e;
+  });
 }
 
 }  // namespace
@@ -562,15 +563,13 @@ size_t cluster_smem(int n, int rows) {
 
 template <class T>
 cudaError_t cluster_attr() {
-  static bool done = false;
-  if (done) return cudaSuccess;
+  // the caller holds the lock of cluster_shape
   cudaError_t e = cudaFuncSetAttribute(kacz_cluster_pre_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        KACZ_LEVEL_MAX_SMEM);
   if (!e) e = cudaFuncSetAttribute(kacz_cluster_post_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    KACZ_LEVEL_MAX_SMEM);
   if (!e) e = cudaFuncSetAttribute(kacz_cluster_pre_kernel<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (!e) e = cudaFuncSetAttribute(kacz_cluster_post_kernel<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (!e) done = true;
   return e;
 }
 
@@ -599,13 +598,12 @@ cudaError_t launch_cluster_kernel(void (*kernel)(Args...), int c, size_t smem, c
 template <class G, bool POST>
 cudaError_t tile_launch_t(double2* uout, int po, const double2* uin, int pu, const double2* f, int pf, const double* kh,
                         int pk, int n, double bA, const int* stop, cudaStream_t s, const Inst& bi) {
-  static bool ready = false;
-  if (!ready) {
-    cudaError_t e = cudaFuncSetAttribute(kacz_sweep_tile64_kernel<G, POST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)tile_smem<G>());
-    if (e) return e;
-    ready = true;
-  }
+  static OncePerDevice opt_in;
+  const cudaError_t e = opt_in([] {
+    return cudaFuncSetAttribute(kacz_sweep_tile64_kernel<G, POST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)tile_smem<G>());
+  });
+  if (e) return e;
   const int t = (n + G::KT) / G::KT;
   pdl_launch(kacz_sweep_tile64_kernel<G, POST>, dim3(t, t, bi.count), G::TBK, tile_smem<G>(), s, uout, po, uin, pu, f, pf,
              kh, pk, n, bA, stop, bi);
@@ -648,7 +646,7 @@ namespace {
 
 // Cluster shape of a level: the most blocks (16, 8, 4 or 2; 16 is beyond the portable cluster
 // size) whose bands fit KACZ_LEVEL_MAX_SMEM and that the device can co-schedule, found once per
-// (precision, n). c = 0: no cluster form for this level.
+// (precision, device, n). c = 0: no cluster form for this level.
 struct ClusterShape {
   int c = 0, rows = 0;
   size_t smem = 0;
@@ -656,9 +654,11 @@ struct ClusterShape {
 template <class T>
 ClusterShape cluster_shape(int n) {
   static std::mutex mu;
-  static std::map<int, ClusterShape> cache;
+  static std::map<std::pair<int, int>, ClusterShape> cache;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return ClusterShape();
   std::lock_guard<std::mutex> lock(mu);
-  auto it = cache.find(n);
+  auto it = cache.find({dev, n});
   if (it != cache.end()) return it->second;
   ClusterShape best;
   if (!cluster_attr<T>()) {
@@ -684,7 +684,7 @@ ClusterShape cluster_shape(int n) {
     }
     cudaGetLastError();  // an unsupported shape leaves no sticky error
   }
-  cache[n] = best;
+  cache[{dev, n}] = best;
   return best;
 }
 

@@ -225,7 +225,8 @@ __global__ void __launch_bounds__(CT) cluster64_post_kernel(double2* __restrict_
 }
 
 // Cluster shape of a level: the most blocks (16, 8, 4 or 2; 16 is beyond the portable cluster size)
-// whose bands fit CLUSTER_MAX_SMEM, have two rows and one thread (or pair) per block of five nodes, and that the device can co-schedule, found once per n. c = 0: no cluster form.
+// whose bands fit CLUSTER_MAX_SMEM, have two rows and one thread (or pair) per block of five nodes,
+// and that the device can co-schedule, found once per device and n. c = 0: no cluster form.
 struct Shape {
   int c = 0, rows = 0, split = 1, threads = 256;
   size_t smem = 0;
@@ -239,9 +240,7 @@ auto with_kernels(const Shape& S, F&& fn) {
   return fn(cluster64_pre_kernel<1, 1024>, cluster64_post_kernel<1, 1024>);
 }
 
-cudaError_t cluster_attrs() {
-  static bool done = false;
-  if (done) return cudaSuccess;
+cudaError_t cluster_attrs() {  // the caller holds the lock of cluster_shape
   cudaError_t e = cudaSuccess;
   auto set = [&](auto kernel) {
     if (!e) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, CLUSTER_MAX_SMEM);
@@ -257,7 +256,6 @@ cudaError_t cluster_attrs() {
       return 0;
     });
   }
-  if (!e) done = true;
   return e;
 }
 
@@ -280,9 +278,11 @@ cudaLaunchConfig_t config(const Shape& S, int batch, cudaLaunchAttribute (&attr)
 
 Shape cluster_shape(int n) {
   static std::mutex mu;
-  static std::map<int, Shape> cache;
+  static std::map<std::pair<int, int>, Shape> cache;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return Shape();
   std::lock_guard<std::mutex> lock(mu);
-  auto it = cache.find(n);
+  auto it = cache.find({dev, n});
   if (it != cache.end()) return it->second;
   Shape best;
   if (!cluster_attrs()) {
@@ -309,7 +309,7 @@ Shape cluster_shape(int n) {
     }
     cudaGetLastError();  // an unsupported shape leaves no sticky error
   }
-  cache[n] = best;
+  cache[{dev, n}] = best;
   return best;
 }
 

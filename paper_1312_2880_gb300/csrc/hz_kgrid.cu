@@ -30,6 +30,7 @@
 
 #include "hz_common.cuh"
 #include "hz_gnode.cuh"
+#include "hz_host.h"
 #include "hz_internal.h"
 
 namespace hz {
@@ -162,21 +163,22 @@ __global__ void __launch_bounds__(GT) kacz_grid_post_kernel(c2<T>* __restrict__ 
 }
 
 // Blocks of a level's cooperative launches: one band of at least three rows each, no more than
-// both kernels of the precision can keep resident at once, nor than KGRID_MAX_BLOCKS. The pre and
+// both kernels of the precision can keep resident at once, nor than KGRID_MAX_BLOCKS (found once per device). The pre and
 // post launches of a level use the same count: they share the level's counters.
 template <class KPre, class KPost>
-int grid_blocks(KPre pre, KPost post, int n, int* cap_cache) {
-  if (*cap_cache == 0) {
-    int dev = 0, sms = 0, a = 0, b = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) ||
+int grid_blocks(KPre pre, KPost post, int n, IntPerDevice& cap_of) {
+  const int cap = cap_of([&](int dev) {
+    int sms = 0, a = 0, b = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, pre, GT, 0) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, post, GT, 0) != cudaSuccess || a < 1 || b < 1)
       return -1;
-    const int cap = sms * (a < b ? a : b);
-    *cap_cache = cap < KGRID_MAX_BLOCKS ? cap : KGRID_MAX_BLOCKS;
-  }
+    const int c = sms * (a < b ? a : b);
+    return c < KGRID_MAX_BLOCKS ? c : KGRID_MAX_BLOCKS;
+  });
+  if (cap < 1) return -1;
   const int bands = (n + 1) / 3 > 0 ? (n + 1) / 3 : 1;
-  return bands < *cap_cache ? bands : *cap_cache;
+  return bands < cap ? bands : cap;
 }
 
 template <class K, class... Args>
@@ -201,13 +203,12 @@ __global__ void coop_probe_kernel(int* out) {
 }  // namespace
 
 bool kacz_grid_available() {
-  static std::once_flag once;
-  static bool ok = false;
-  std::call_once(once, [] {
-    int dev = 0, coop = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) ||
-        !coop)
-      return;
+  static std::mutex mu;
+  static IntPerDevice state;  // 1: no, 2: yes
+  std::lock_guard<std::mutex> lock(mu);
+  return state([](int dev) {
+    int coop = 0;
+    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) || !coop) return 1;
     // a cooperative launch captured into a graph, instantiated and run once
     cudaStream_t s = nullptr;
     int* d = nullptr;
@@ -229,15 +230,14 @@ bool kacz_grid_available() {
     if (d) cudaFree(d);
     if (s) cudaStreamDestroy(s);
     cudaGetLastError();  // a refused capture leaves no error behind
-    ok = good;
-  });
-  return ok;
+    return good ? 2 : 1;
+  }) == 2;
 }
 
 int kgrid_blocks(bool fp32, int n) {
-  static int cap32 = 0, cap64 = 0;
-  return fp32 ? grid_blocks(kacz_grid_pre_kernel<float, float2>, kacz_grid_post_kernel<float, float2>, n, &cap32)
-              : grid_blocks(kacz_grid_pre_kernel<double, double2>, kacz_grid_post_kernel<double, double2>, n, &cap64);
+  static IntPerDevice cap32, cap64;
+  return fp32 ? grid_blocks(kacz_grid_pre_kernel<float, float2>, kacz_grid_post_kernel<float, float2>, n, cap32)
+              : grid_blocks(kacz_grid_pre_kernel<double, double2>, kacz_grid_post_kernel<double, double2>, n, cap64);
 }
 
 cudaError_t launch_kacz_grid_pre(bool fp32, void* u, int pu, void* fc, int pc, const void* f, int pf, const void* kh,

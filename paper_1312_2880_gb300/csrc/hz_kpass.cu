@@ -20,6 +20,7 @@
 #include <cuda_runtime.h>
 
 #include "hz_common.cuh"
+#include "hz_host.h"
 #include "hz_internal.h"
 #include "hz_level.cuh"
 
@@ -273,13 +274,12 @@ __global__ void __maxnreg__(56) kacz_pass_kernel(const KaczPassArgs a, Inst bi) 
 template <int S, int COLS, bool POST, bool CAP, bool ZERO>
 cudaError_t launch_one(const KaczPassArgs& a, cudaStream_t s, const Inst& bi) {
   using G = PassGeo<S, COLS, POST, CAP>;
-  static bool ready = false;
-  if (!ready) {
-    cudaError_t e = cudaFuncSetAttribute(kacz_pass_kernel<G, POST, CAP, ZERO>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
-    if (e) return e;
-    ready = true;
-  }
+  static OncePerDevice opt_in;
+  const cudaError_t e = opt_in([] {
+    return cudaFuncSetAttribute(kacz_pass_kernel<G, POST, CAP, ZERO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)G::SMEM);
+  });
+  if (e) return e;
   const int t = (a.n + G::KT) / G::KT;
   pdl_launch(kacz_pass_kernel<G, POST, CAP, ZERO>, dim3(t, t, bi.count), PT, G::SMEM, s, a, bi);
   return cudaGetLastError();

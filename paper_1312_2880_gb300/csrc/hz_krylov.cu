@@ -12,6 +12,7 @@
 #include <math.h>
 
 #include "hz_common.cuh"
+#include "hz_host.h"
 #include "hz_internal.h"
 
 namespace hz {
@@ -779,15 +780,6 @@ __global__ void apply_fp64_kernel(double2* v, const double2* u, const double* kh
 }
 
 }  // namespace
-
-int device_sms() {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) || sms < 1) sms = 1;
-  }
-  return sms;
-}
 
 #define KGRID dim3(k.G, 1, k.batch)
 #define KLAUNCH(name) pdl_launch(name, KGRID, KB, 0, s, k); return cudaGetLastError();

@@ -25,6 +25,7 @@
 #include <stdint.h>
 
 #include "hz_common.cuh"
+#include "hz_host.h"
 #include "hz_internal.h"
 
 namespace hz {
@@ -542,13 +543,11 @@ bool aligned16(const void* p, long long pitch, long long stride) {
   return ((uintptr_t)p & 15) == 0 && !(pitch & 1) && !(stride & 1);
 }
 
-// Dynamic shared memory above the default 48 KB (the FP64 rings), set once per kernel.
+// Dynamic shared memory above the default 48 KB (the FP64 rings).
 template <class K>
-cudaError_t allow_smem(K kernel, size_t bytes, bool& done) {
-  if (done || bytes <= 48 * 1024) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (!e) done = true;
-  return e;
+cudaError_t allow_smem(K kernel, size_t bytes, OncePerDevice& opt_in) {
+  if (bytes <= 48 * 1024) return cudaSuccess;
+  return opt_in([&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); });
 }
 
 template <class Real>
@@ -558,7 +557,7 @@ cudaError_t sr_stream(void* u, int pu, void* fc, int pc, const void* f, int pf, 
   const int strips = (n + 1 + SR_W - 1) / SR_W, segs = (n + 1 + seg_rows - 1) / seg_rows;
   dim3 grid((strips + WPB - 1) / WPB, segs, bi.count);
   constexpr size_t sm = (size_t)WPB * SR_R * sr_slot<Real>();
-  static bool ready[2] = {false, false};
+  static OncePerDevice ready[2];
   cudaError_t e;
   if (aligned16(f, pf, bi.sf)) {
     if ((e = allow_smem(smooth_restrict_stream_kernel<Real, true>, sm, ready[1]))) return e;
@@ -579,7 +578,7 @@ cudaError_t ps_stream(void* out, int po, const void* upre, int pu, const void* e
   const int strips = (n + 1 + PS_W - 1) / PS_W, segs = (n + 1 + seg_rows - 1) / seg_rows;
   dim3 grid((strips + WPB - 1) / WPB, segs, bi.count);
   constexpr size_t sm = (size_t)WPB * PS_R * ps_slot<Real>();
-  static bool ready[2] = {false, false};
+  static OncePerDevice ready[2];
   cudaError_t e;
   if (aligned16(f, pf, bi.sf) && aligned16(out, po, bi.so)) {
     if ((e = allow_smem(prolong_smooth_stream_kernel<Real, true>, sm, ready[1]))) return e;

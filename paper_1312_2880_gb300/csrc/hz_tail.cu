@@ -12,6 +12,7 @@
 #include <algorithm>
 
 #include "hz_common.cuh"
+#include "hz_host.h"
 #include "hz_internal.h"
 #include "hz_level.cuh"
 
@@ -279,18 +280,17 @@ size_t tail_layout(bool fp32, TailArgs* A) {
 
 cudaError_t launch_tail(bool fp32, const TailArgs& A, size_t smem, const int* stop, cudaStream_t s, const Inst& bi) {
   if (A.count < 2 || A.count > TAIL_MAX_LEVELS || smem > (size_t)TAIL_MAX_SMEM) return cudaErrorInvalidValue;
-  static bool ready[3] = {false, false, false};
+  static OncePerDevice ready[3];
+  auto opt_in = [](auto kernel) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TAIL_MAX_SMEM);
+  };
   cudaError_t e;
   const int m = (A.lv[A.count - 1].n + 1) * (A.lv[A.count - 1].n + 1);
   // A cluster while its blocks are one wave (a block of the tail takes an SM) and there is something to
   // share: tails of n_l = 8, 4 (m = 25) 23.2 us in one block, 19.1 with helpers, 10, 5 (m = 36) 25.2 and
   // 20.1, 14, 7 (m = 64) 31.4 and 21.9. A batch of more instances fills the SMs with its own tails.
   if (!fp32 && A.off_ainv && m >= 25 && coarse_share_fits(m) && TAIL_CLUSTER * bi.count <= device_sms()) {
-    if (!ready[2]) {
-      e = cudaFuncSetAttribute(tail_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TAIL_MAX_SMEM);
-      if (e) return e;
-      ready[2] = true;
-    }
+    if ((e = ready[2]([&] { return opt_in(tail_cluster_kernel); }))) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(TAIL_CLUSTER, 1, bi.count);
     cfg.blockDim = dim3(TAIL_THREADS);
@@ -307,12 +307,7 @@ cudaError_t launch_tail(bool fp32, const TailArgs& A, size_t smem, const int* st
     cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, tail_cluster_kernel, A, stop, bi);
   }
-  if (!ready[fp32]) {
-    e = fp32 ? cudaFuncSetAttribute(tail_kernel32, cudaFuncAttributeMaxDynamicSharedMemorySize, TAIL_MAX_SMEM)
-             : cudaFuncSetAttribute(tail_kernel64, cudaFuncAttributeMaxDynamicSharedMemorySize, TAIL_MAX_SMEM);
-    if (e) return e;
-    ready[fp32] = true;
-  }
+  if ((e = ready[fp32]([&] { return fp32 ? opt_in(tail_kernel32) : opt_in(tail_kernel64); }))) return e;
   dim3 grid(1, 1, bi.count);
   if (fp32)
     pdl_launch(tail_kernel32, grid, TAIL_THREADS, smem, s, A, stop, bi);
