@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "hz_internal.h"
+#include "hz_rules.h"
 
 using namespace hz;
 
@@ -1140,10 +1141,10 @@ void plan_tail(hz_problem* P) {
 // Every fused Gauss-Seidel level runs each candidate variant of its two passes
 // (shared-memory tiles, or register streaming with 2 .. 256 rows per warp) on its own arrays,
 // with all right-hand sides of the batch: one untimed launch, then the best of three timings of
-// five back-to-back launches with CUDA events on the library stream. The fastest is kept, and cached per
-// (n_l, batch, pass, finest level or not, precision) for later problems of the same shape.
+// five back-to-back launches with CUDA events on the library stream. The fastest is kept, and cached
+// (rules::tune_key) for later problems of the same shape.
 std::mutex g_tune_mutex;
-std::map<std::tuple<int, int, int, int, int>, int> g_tune_cache;
+std::map<rules::TuneKey, int> g_tune_cache;
 
 // Candidates for a level of n_l intervals: streaming needs n_l >= 4; segments longer than the
 // level add nothing over the one that covers it.
@@ -1214,7 +1215,7 @@ cudaError_t autotune(hz_problem* P) {
     }
     for (int up = 0; up < 2; ++up) {
       int& var = up ? L.var_up : L.var_down;
-      const auto key = std::make_tuple(L.n, B, up, l == 0 ? 1 : 0, P->plan.fp32 ? 1 : 0);
+      const auto key = rules::tune_key(L.n, B, up != 0, l == 0, P->plan.fp32, op_beta(P, L.relax_op), op_beta(P, L.resid_op));
       {
         std::lock_guard<std::mutex> lock(g_tune_mutex);
         auto it = g_tune_cache.find(key);

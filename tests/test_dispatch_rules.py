@@ -1,0 +1,31 @@
+"""The rules that choose how a level or a launch runs (csrc/hz_rules.h), on the CPU."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_1312_2880_gb300", "csrc")
+SMS = 152
+
+
+@pytest.fixture(scope="module")
+def rules(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("rules") / "rules.so")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I" + CSRC, os.path.join(HERE, "rules_probe.cpp"),
+                    "-o", so], check=True)
+    return ctypes.CDLL(so)
+
+
+def test_a_tuned_fp64_pass_is_not_reused_for_another_operator_kind(rules):
+    d = ctypes.c_double
+    kinds = [(0.0, 0.0), (0.5, 0.0), (0.5, 0.5)]  # L / L, M / L, M / M
+    for q, a in enumerate(kinds):
+        for r, b in enumerate(kinds):
+            key = lambda up, fp32: rules.same_tuning(2048, 1, up, 0, fp32, d(a[0]), d(a[1]), d(b[0]), d(b[1]))
+            assert key(0, 0) == (q == r)  # the pass down relaxes and forms the residual
+            assert key(1, 0) == ((a[0] == 0) == (b[0] == 0))  # the pass up only relaxes
+            assert key(0, 1) == key(1, 1) == 1  # FP32: one code for every operator
+    assert rules.same_tuning(2048, 1, 0, 0, 0, d(0.5), d(0.5), d(0.3), d(0.3))
+    assert not rules.same_shape(2048, 1024, 1, 1) and not rules.same_shape(2048, 2048, 1, 2)
