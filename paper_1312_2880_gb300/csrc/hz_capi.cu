@@ -430,7 +430,7 @@ void plan_kaczmarz(hz_problem* P) {
     if (L.smoother != HZ_SMOOTH_KACZMARZ) continue;
     const int want = P->opts.kacz_form;
     L.kform = (want >= 0 && kform_ok(P, l, want)) ? want : default_kform(P, l);
-    L.pass_cfg = pass_config(L.n, L.nu, P->plan.batch, P->num_sms);
+    L.pass_cfg = rules::pass_config(L.n, L.nu, P->plan.batch, P->num_sms);
   }
 }
 

@@ -185,8 +185,8 @@ cudaError_t launch_coarse_setup(bool fp32, void* ainvT, double2* work, const voi
                                 int* status, cudaStream_t s);
 
 // A whole pre- or post-relaxation pass (nu sweeps, nu even) of an FP32 Kaczmarz level below the finest,
-// with its transfer, in launches of independent tiles (hz_kpass.cu) of the geometry that pass_config
-// picks. Pre: zero guess into u, restricted residual into fc. Post: sweeps of u + P ec, ending in u
+// with its transfer, in launches of independent tiles (hz_kpass.cu) of the geometry that
+// rules::pass_config picks. Pre: zero guess into u, restricted residual into fc. Post: sweeps of u + P ec, ending in u
 // (pass_in_place) or in u2.
 struct KaczPassArgs {
   const float2* uin = nullptr;  // set per launch
@@ -202,7 +202,6 @@ struct KaczPassArgs {
   float bA = 0, bB = 0;
   const int* stop = nullptr;
 };
-int pass_config(int n, int nu, int batch, int sms);
 bool pass_in_place(int cfg, int nu);
 cudaError_t launch_kacz_pass(bool post, int cfg, int nu, const KaczPassArgs& a, float2* u, float2* u2, cudaStream_t s,
                              const Inst& bi);

@@ -306,8 +306,8 @@ cudaError_t run_pass(bool post, int nu, KaczPassArgs a, float2* u, float2* u2, c
   return cudaSuccess;
 }
 
-// Geometries: 0, 65 x 81 regions for four sweeps; 1, 65 x 73 regions and 2, 90 x 98 regions for two.
-constexpr int CFGS = 3;
+// Geometries (rules::pass_config): 0, 65 x 81 regions for four sweeps; 1, 65 x 73 regions and 2, 90 x 98
+// regions for two.
 constexpr int cfg_sweeps(int cfg) { return cfg == 0 ? 4 : 2; }
 
 }  // namespace
@@ -324,28 +324,6 @@ cudaError_t launch_kacz_pass(bool post, int cfg, int nu, const KaczPassArgs& arg
     case 2: return run_pass<2, 18>(post, nu, a, u, u2, s, bi);
   }
   return cudaErrorInvalidValue;
-}
-
-// The geometry with the least expected time of a level's four launches or launch pairs in an iteration:
-// a block fills an SM, so a launch takes a wave of blocks' time per 152 blocks. Measured per
-// iteration (us, geometries 0, 1, 2): n_l = 128 93, 101, 143; n_l = 192 119, 103, 155; n_l = 256 178,
-// 105, 156; n_l = 512 565, 171, 156; n_l = 1024 2114, 416, 292, i.e. about 58 + 35, 32 + 72 and
-// 20 + 136 per wave; 16 right-hand sides on n_l = 144 and 288 (whole iteration) 1243, 566, 583 and
-// 4165, 1503, 1320.
-int pass_config(int n, int nu, int batch, int sms) {
-  const int kt[CFGS] = {13, 37, 62};
-  const double fixed[CFGS] = {58, 32, 20}, wave[CFGS] = {35, 72, 136};
-  int best = 1;
-  double cost = 0;
-  for (int q = nu % 4 == 0 ? 0 : 1; q < CFGS; ++q) {
-    const long long t = (n + kt[q]) / kt[q], blocks = t * t * batch;
-    const double c = fixed[q] + wave[q] * (double)((blocks + sms - 1) / sms);
-    if (cost == 0 || c < cost) {
-      best = q;
-      cost = c;
-    }
-  }
-  return best;
 }
 
 }  // namespace hz

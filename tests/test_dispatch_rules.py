@@ -29,3 +29,11 @@ def test_a_tuned_fp64_pass_is_not_reused_for_another_operator_kind(rules):
             assert key(0, 1) == key(1, 1) == 1  # FP32: one code for every operator
     assert rules.same_tuning(2048, 1, 0, 0, 0, d(0.5), d(0.5), d(0.3), d(0.3))
     assert not rules.same_shape(2048, 1024, 1, 1) and not rules.same_shape(2048, 2048, 1, 2)
+
+
+def test_large_batches_of_passes_take_the_largest_tiles(rules):
+    """From four waves of the 62-node tiles on: there the halo decides (n_l = 128 with 64 and 152 right-hand sides)."""
+    for n, batch in ((128, 64), (128, 152), (136, 64), (144, 152), (224, 64)):
+        assert rules.pass_cfg(n, 4, batch, SMS) == 2, (n, batch)
+    for n, nu, batch, want in ((128, 4, 1, 0), (128, 2, 1, 1), (192, 4, 1, 1), (256, 4, 1, 1), (128, 4, 16, 2), (96, 4, 8, 1)):
+        assert rules.pass_cfg(n, nu, batch, SMS) == want, (n, nu, batch)
