@@ -52,7 +52,7 @@ struct Level {
   void* u2 = nullptr; // result of the fused post-smoothing pass (levels >= 1)
   int var_down = 0, var_up = 0;  // fused-pass variants (picked by the tile autotuner)
   int kform = 0;                 // hz_kacz_form of a Kaczmarz level (set up by plan_kaczmarz)
-  int pass_cfg = 0;              // tile geometry of its whole passes (pass_config)
+  int pass_cfg = 0;              // how its FP32 tiles run (rules::pass_config)
   double omega = 1.0;            // relaxation factor of a Jacobi or SOR level
 };
 
@@ -434,8 +434,9 @@ void plan_kaczmarz(hz_problem* P) {
   }
 }
 
-// Tiled FP64 sweeps on level l, one per launch, ping-pong between u and u2 ending in u: `first_in` is
-// the input of the first sweep (null = zero guess). FP32 levels run whole passes (run_kacz_pass).
+// Tiled sweeps on level l, one (FP64) or two (FP32) per launch, ping-pong between u and u2 ending in u:
+// `first_in` is the input of the first launch (null = zero guess). Most FP32 levels run whole passes
+// instead (run_kacz_pass).
 cudaError_t kacz_tile_sweeps(hz_problem* P, int l, Src f, const void* first_in, bool post, const int* stop,
                              const Inst& bi) {
   const Level& L = P->lv[l];
@@ -443,13 +444,18 @@ cudaError_t kacz_tile_sweeps(hz_problem* P, int l, Src f, const void* first_in, 
   const void* kh = kh_of(P, l, &pk);
   const void* in = first_in;
   cudaError_t e;
-  for (int k = 0; k < L.nu; ++k) {
-    void* out = ((L.nu - 1 - k) % 2 == 0) ? L.u : L.u2;
-    if ((e = mark(P, launch_kacz_sweep_tile64((double2*)out, L.pitch, (const double2*)in, L.pitch, (const double2*)f.f,
-                                              f.pf, (const double*)kh, pk, L.n, op_beta(P, L.relax_op), post,
-                                              P->num_sms, stop, P->stream, bi),
-                  HZ_K_KACZ_SWEEP, l)))
-      return e;
+  const bool fp32 = P->plan.fp32;
+  const int launches = fp32 ? L.nu / 2 : L.nu;
+  const double bA = op_beta(P, L.relax_op);
+  for (int k = 0; k < launches; ++k) {
+    void* out = ((launches - 1 - k) % 2 == 0) ? L.u : L.u2;
+    if (fp32)
+      e = launch_kacz_sweep_tile32(rules::tile_edge(L.pass_cfg), (float2*)out, L.pitch, (const float2*)in, L.pitch,
+                                   (const float2*)f.f, f.pf, (const float*)kh, pk, L.n, bA, post, stop, P->stream, bi);
+    else
+      e = launch_kacz_sweep_tile64((double2*)out, L.pitch, (const double2*)in, L.pitch, (const double2*)f.f, f.pf,
+                                   (const double*)kh, pk, L.n, bA, post, P->num_sms, stop, P->stream, bi);
+    if ((e = mark(P, e, HZ_K_KACZ_SWEEP, l))) return e;
     in = out;
   }
   return cudaSuccess;
@@ -486,7 +492,7 @@ cudaError_t jacobi_sweeps(hz_problem* P, int l, Src f, bool from_zero, int sweep
 // A tiled Kaczmarz level whose passes run whole (hz_kpass.cu).
 bool kacz_pass(const hz_problem* P, int l) {
   return l > 0 && l < P->plan.levels - 1 && P->plan.fp32 && P->lv[l].smoother == HZ_SMOOTH_KACZMARZ &&
-         P->lv[l].kform == HZ_KACZ_TILE;
+         P->lv[l].kform == HZ_KACZ_TILE && rules::tile_edge(P->lv[l].pass_cfg) == 0;
 }
 
 // Where level l's result after post-relaxation lives (what level l-1 interpolates).

@@ -139,6 +139,10 @@ cudaError_t launch_kacz_grid_post(bool fp32, void* u, int pu, const void* ec, in
 cudaError_t launch_kacz_sweep_tile64(double2* uout, int po, const double2* uin, int pu, const double2* f, int pf,
                                      const double* kh, int pk, int n, double bA, bool post, int sms, const int* stop,
                                      cudaStream_t s, const Inst& bi = Inst());
+// Two FP32 Kaczmarz sweeps over halo tiles of 32 or 64 nodes (edge).
+cudaError_t launch_kacz_sweep_tile32(int edge, float2* uout, int po, const float2* uin, int pu, const float2* f, int pf,
+                                     const float* kh, int pk, int n, double bA, bool post, const int* stop,
+                                     cudaStream_t s, const Inst& bi = Inst());
 // Coarse tail (hz_tail.cu): levels lt .. L-1 of the V-cycle in one block's shared memory.
 constexpr int TAIL_MAX_LEVELS = 12;
 constexpr int TAIL_MAX_SMEM = 200 * 1024;

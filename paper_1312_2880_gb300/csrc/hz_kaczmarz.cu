@@ -9,10 +9,11 @@
 //   diagonal and 1/|a_p|^2 computed once per launch (operations in hz_level.cuh). Pre mode: zero guess, nu sweeps (colours
 //   0..4), then the residual with the (B) operator and full weighting onto the coarse level. Post
 //   mode: u_pre + P e_c, then nu sweeps (colours 4..0).
-// kacz_sweep_tile64: one full FP64 sweep (all five colours) per launch over tiles with a halo that holds
-//   the dependency cone of the sweep (6 columns each side, 6 and 10 rows), so the tile interior holds
-//   exactly the sequential sweep's values; each phase acts only on the part of the region that can
-//   still reach the tile. Out of place. (FP32 levels run whole passes in tiles: hz_kpass.cu.)
+// kacz_sweep_tile64, kacz_sweep_tile32: one FP64 sweep (all five colours) or two FP32 sweeps per launch over
+//   tiles with a halo that holds their dependency cone (6 columns each side, 6 and 10 rows per sweep),
+//   so the tile interior holds exactly the sequential sweeps' values; each phase acts only on the part
+//   of the region that can still reach the tile. Out of place. (Most FP32 levels run whole passes with
+//   their transfers in tiles instead: hz_kpass.cu, rules::pass_config.)
 // kacz_cluster_*: the kacz_level_* operations with an FP32 level split into row bands over a
 //   thread-block cluster of up to 16 blocks (distributed shared memory, one cluster barrier per
 //   colour), for levels too large for one block with an odd number of sweeps (FP64: hz_kcluster.cu).
@@ -33,7 +34,7 @@ namespace hz {
 namespace {
 
 constexpr int LB = 1024;  // threads of the whole-level kernel
-// Tiles of the tiled forms (FP64 here, FP32 in hz_kpass.cu): KT x KT outputs per block after S sweeps per launch. The halo is the
+// Tiles of the tiled forms: KT x KT outputs per block after S sweeps per launch. The halo is the
 // dependency cone of S five-colour sweeps (found by propagating dependencies through the colour
 // phases on an unbounded grid, every residue of the colour pattern): after one sweep in the order
 // 0..4 an output depends on starting values at most 6 columns to either side, 6 rows below and 10
@@ -45,8 +46,8 @@ struct TileGeo {
   static constexpr int HN = 6 * S_, HF = 10 * S_;  // halo rows on the near and the far side
   static constexpr int RX = KT_ + 2 * HX, RY = KT_ + HN + HF, REG = RX * RY;
 };
-template <class G>
-constexpr size_t tile_smem() { return (size_t)G::REG * (2 * sizeof(double2) + 2 * sizeof(double)); }
+template <class T, class G>  // u, f~, k H and in FP64 the stored 1 / |a_p|^2
+constexpr size_t tile_smem() { return (size_t)G::REG * (2 * sizeof(c2<T>) + (sizeof(T) == 8 ? 2 : 1) * sizeof(T)); }
 
 // Actions of phase ph (of P = 5S; R = P - 1 - ph phases follow it) that can still reach the
 // tile's outputs. Propagating dependencies back from the outputs through the colour phases on an
@@ -88,8 +89,9 @@ __device__ __forceinline__ int mod5(int x) { return ((x % 5) + 5) % 5; }
 
 // Phase PH of a tile: each thread takes up to two slots, reads both supports before updating
 // either (same-colour supports are disjoint), then writes both back. The row constants come from
-// k H and the stored 1 / |a_p|^2 (the values of lvl::row_consts) and the arithmetic is lvl::act_update, so a tiled sweep gives the same bits as the whole-level
-// and cluster forms.
+// k H as in the whole-level forms (lvl::row_consts; strictly inside the square, no boundary term), in
+// FP64 with its value of 1 / |a_p|^2 read, and the arithmetic is lvl::act_update, so a tiled sweep
+// gives the same bits as the whole-level and cluster forms.
 template <class T, class G, bool POST, bool INNER, int PH>
 __device__ __forceinline__ void tile_phase(c2<T>* su, const c2<T>* sf, const T* sk, const T* si,
                                            const unsigned char* c0row, int gx, int gy, int n, T beta) {
@@ -140,14 +142,20 @@ __device__ __forceinline__ void tile_phase(c2<T>* su, const c2<T>* sf, const T* 
       A.un = su[A.on];
       A.f = sf[A.op];
       kh[s] = sk[A.op];
-      inv[s] = si[A.op];
+      if constexpr (sizeof(T) == 8) inv[s] = si[A.op];
     }
   }
 #pragma unroll
   for (int s = 0; s < NS; ++s) {
     TileAct<T>& A = a[s];
     if (A.ok) {
-      const c2<T> d = xr::diag<T>(kh[s], INNER ? 0 : lvl::sides_at(A.i, A.j, n), beta);
+      c2<T> d;
+      if constexpr (sizeof(T) == 4 && !INNER) {
+        lvl::row_consts<T>(kh[s], A.i, A.j, n, beta, &d, &inv[s]);
+      } else {
+        d = xr::diag<T>(kh[s], INNER ? 0 : lvl::sides_at(A.i, A.j, n), beta);
+        if constexpr (sizeof(T) == 4) inv[s] = xr::rcp(xr::add(xr::cabs2<T>(d), (T)4));
+      }
       lvl::act_update<T>(A.up, A.uw, A.ue, A.us, A.un, A.f, d, inv[s], A.mx, A.my);
     }
   }
@@ -275,14 +283,10 @@ __global__ void __launch_bounds__(LB) kacz_level_post_kernel(c2<T>* __restrict__
   lvl::for_nodes_blocked(n, [&](int, int i, int j, int p) { u[(long long)j * pu + i] = S.su[p]; });
 }
 
-template <class G, bool POST>
-__global__ void __launch_bounds__(G::TBK) kacz_sweep_tile64_kernel(double2* __restrict__ uout, int po,
-                                                                         const double2* __restrict__ uin, int pu,
-                                                                         const double2* __restrict__ f, int pf,
-                                                                         const double* __restrict__ kh, int pk, int n,
-                                                                         double bA, const int* __restrict__ stop,
-                                                                         Inst bi) {
-  using T = double;
+template <class T, class G, bool POST>
+__device__ __forceinline__ void tile_sweeps(c2<T>* __restrict__ uout, int po, const c2<T>* __restrict__ uin, int pu,
+                                            const c2<T>* __restrict__ f, int pf, const T* __restrict__ kh, int pk, int n,
+                                            T bA, const int* __restrict__ stop, const Inst& bi) {
   using PR = PhaseRect<G, POST>;
   static_assert(PR::fits(), "phase rectangles must keep their supports inside the tile region");
   constexpr int TBK = G::TBK, RX = G::RX, RY = G::RY, REG = G::REG, KT = G::KT;
@@ -295,7 +299,7 @@ __global__ void __launch_bounds__(G::TBK) kacz_sweep_tile64_kernel(double2* __re
   c2<T>* su = reinterpret_cast<c2<T>*>(smem);
   c2<T>* sf = su + REG;
   T* sk = reinterpret_cast<T*>(sf + REG);
-  T* si = sk + REG;  // the stored 1 / |a_p|^2
+  T* si = sk + (sizeof(T) == 8 ? REG : 0);  // FP64: the stored 1 / |a_p|^2
   __shared__ unsigned char c0row[RY];  // column residue of colour 0 in each region row
   const int x0 = blockIdx.x * KT, y0 = blockIdx.y * KT;
   // sweeps in the order 0..4 (pre) need the near halo below the tile, 4..0 (post) above it
@@ -319,7 +323,7 @@ __global__ void __launch_bounds__(G::TBK) kacz_sweep_tile64_kernel(double2* __re
         su[q] = mk<T>(0, 0);
       lvl::cp_async<sizeof(c2<T>)>(sf + q, f + jf + i);
       lvl::cp_async<sizeof(T)>(sk + q, kh + jk + i);
-      lvl::cp_async<sizeof(T)>(si + q, bi.inv + (long long)j * bi.pi + i);
+      if constexpr (sizeof(T) == 8) lvl::cp_async<sizeof(T)>(si + q, bi.inv + (long long)j * bi.pi + i);
     }
   }
   for (int r = threadIdx.x; r < RY; r += TBK) c0row[r] = (unsigned char)mod5(-2 * (gy + r) - gx);
@@ -344,6 +348,24 @@ __global__ void __launch_bounds__(G::TBK) kacz_sweep_tile64_kernel(double2* __re
       orow[i] = su[r * RX + c];
     }
   }
+}
+template <class G, bool POST>
+__global__ void __launch_bounds__(G::TBK) kacz_sweep_tile64_kernel(double2* __restrict__ uout, int po,
+                                                                   const double2* __restrict__ uin, int pu,
+                                                                   const double2* __restrict__ f, int pf,
+                                                                   const double* __restrict__ kh, int pk, int n,
+                                                                   double bA, const int* __restrict__ stop, Inst bi) {
+  tile_sweeps<double, G, POST>(uout, po, uin, pu, f, pf, kh, pk, n, bA, stop, bi);
+}
+// 56 registers, so that a 1024-thread block leaves room for the deferred solution update (k_update_x, one
+// 128-thread block per SM) beside it.
+template <class G, bool POST>
+__global__ void __maxnreg__(56) kacz_sweep_tile32_kernel(float2* __restrict__ uout, int po,
+                                                         const float2* __restrict__ uin, int pu,
+                                                         const float2* __restrict__ f, int pf,
+                                                         const float* __restrict__ kh, int pk, int n, float bA,
+                                                         const int* __restrict__ stop, Inst bi) {
+  tile_sweeps<float, G, POST>(uout, po, uin, pu, f, pf, kh, pk, n, bA, stop, bi);
 }
 
 template <class T>
@@ -601,15 +623,29 @@ cudaError_t tile_launch_t(double2* uout, int po, const double2* uin, int pu, con
   static OncePerDevice opt_in;
   const cudaError_t e = opt_in([] {
     return cudaFuncSetAttribute(kacz_sweep_tile64_kernel<G, POST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)tile_smem<G>());
+                                (int)tile_smem<double, G>());
   });
   if (e) return e;
   const int t = (n + G::KT) / G::KT;
-  pdl_launch(kacz_sweep_tile64_kernel<G, POST>, dim3(t, t, bi.count), G::TBK, tile_smem<G>(), s, uout, po, uin, pu, f, pf,
+  pdl_launch(kacz_sweep_tile64_kernel<G, POST>, dim3(t, t, bi.count), G::TBK, tile_smem<double, G>(), s, uout, po, uin, pu, f, pf,
              kh, pk, n, bA, stop, bi);
   return cudaGetLastError();
 }
 
+template <class G, bool POST>
+cudaError_t tile32_launch_t(float2* uout, int po, const float2* uin, int pu, const float2* f, int pf, const float* kh,
+                            int pk, int n, float bA, const int* stop, cudaStream_t s, const Inst& bi) {
+  static OncePerDevice opt_in;
+  const cudaError_t e = opt_in([] {
+    return cudaFuncSetAttribute(kacz_sweep_tile32_kernel<G, POST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)tile_smem<float, G>());
+  });
+  if (e) return e;
+  const int t = (n + G::KT) / G::KT;
+  pdl_launch(kacz_sweep_tile32_kernel<G, POST>, dim3(t, t, bi.count), G::TBK, tile_smem<float, G>(), s, uout, po, uin, pu,
+             f, pf, kh, pk, n, bA, stop, bi);
+  return cudaGetLastError();
+}
 template <class G, class... A>
 cudaError_t tile_launch(bool post, A... args) {
   return post ? tile_launch_t<G, true>(args...) : tile_launch_t<G, false>(args...);
@@ -640,6 +676,17 @@ cudaError_t launch_kacz_sweep_tile64(double2* uout, int po, const double2* uin, 
     case 44: return tile_launch<TileGeo<44, 1, 320>>(post, uout, po, uin, pu, f, pf, kh, pk, n, bA, stop, s, bi);
     default: return tile_launch<TileGeo<28, 1, 352>>(post, uout, po, uin, pu, f, pf, kh, pk, n, bA, stop, s, bi);
   }
+}
+
+cudaError_t launch_kacz_sweep_tile32(int edge, float2* uout, int po, const float2* uin, int pu, const float2* f, int pf,
+                                     const float* kh, int pk, int n, double bA, bool post, const int* stop,
+                                     cudaStream_t s, const Inst& bi) {
+  auto go = [&](auto geo) {
+    using G = decltype(geo);
+    return post ? tile32_launch_t<G, true>(uout, po, uin, pu, f, pf, kh, pk, n, (float)bA, stop, s, bi)
+                : tile32_launch_t<G, false>(uout, po, uin, pu, f, pf, kh, pk, n, (float)bA, stop, s, bi);
+  };
+  return edge == 32 ? go(TileGeo<32, 2, 512>()) : go(TileGeo<64, 2, 1024>());
 }
 
 namespace {

@@ -17,8 +17,9 @@ inline TuneKey tune_key(int n, int batch, bool up, bool finest, bool fp32, doubl
   return TuneKey(n, batch, up, finest, fp32, relax_l, resid_l);
 }
 
-// Geometry of the whole passes of an FP32 Kaczmarz level (hz_kpass.cu): tiles of 13 nodes for four sweeps a
-// launch, of 37 or of 62 for two. The one with the least expected time of a level's four launches or launch
+// How the tiles of an FP32 Kaczmarz level run: 0 .. 2, whole passes with their transfers (hz_kpass.cu) in
+// tiles of 13 nodes for four sweeps a launch, of 37 or of 62 for two; 3 and 4, two-sweep launches over tiles
+// of 32 or 64 nodes between separate transfers (hz_kaczmarz.cu). Of the first three, the one with the least expected time of a level's four launches or launch
 // pairs in an iteration: a block fills an SM, so a launch takes a wave of blocks' time per `sms` blocks.
 // Measured per iteration (us, geometries 0, 1, 2): n_l = 128 93, 101, 143; n_l = 192 119, 103, 155;
 // n_l = 256 178, 105, 156; n_l = 512 565, 171, 156; n_l = 1024 2114, 416, 292, i.e. about 58 + 35, 32 + 72
@@ -26,13 +27,27 @@ inline TuneKey tune_key(int n, int batch, bool up, bool finest, bool fp32, doubl
 // 4165, 1503, 1320. From four waves of the largest tiles on, the halo decides and not the waves, many of
 // whose blocks lie mostly outside the square: 64 and 152 right-hand sides on n_l = 128 (six iterations)
 // 9.08 and 19.65 ms with 37-node tiles, which the expected times prefer, 7.89 and 16.72 ms with 62.
+//
+// The two-sweep launches act only on what can still reach a tile, a fifth fewer row actions than whole passes
+// of the same size, and pay two launches and the transfers' traffic for it. V-cycles whose only Kaczmarz
+// level is n_l, in us, whole passes (37 or 62), 32 and 64: n_l = 416 131, 149, 152; 448 153, 149, 154; 512
+// 165, 159, 166; 576 178, 194, 181; 704 210, 238, 208; 768 256, 248, 251; 896 291, 307, 280; 1024 324, 362,
+// 309; 1536 604, 692, 578; 2048 993, 1139, 929. So 64 from where the 62-node tiles take a second wave, and
+// 32 where they leave more than two fifths of the SMs idle and the 37-node tiles already take a second
+// wave. Batches keep whole passes below that size: 16 right-hand sides on n_l = 256 and 512 (six iterations)
+// 6.55, 7.53, 6.98 and 21.0, 24.1, 21.6 ms.
 constexpr int PASS_EDGE[3] = {13, 37, 62};
+inline int tile_edge(int cfg) { return cfg == 3 ? 32 : cfg == 4 ? 64 : 0; }
 inline long long pass_blocks(int cfg, int n, int batch) {
   const long long t = (n + PASS_EDGE[cfg]) / PASS_EDGE[cfg];
   return t * t * batch;
 }
 inline int pass_config(int n, int nu, int batch, int sms) {
   const double fixed[3] = {58, 32, 20}, wave[3] = {35, 72, 136};
+  if (nu % 4 == 0) {  // the two-sweep launches end in the array they start from
+    if (pass_blocks(2, n, 1) > sms) return 4;
+    if (batch == 1 && pass_blocks(1, n, 1) > sms && 5 * pass_blocks(2, n, 1) < 3ll * sms) return 3;
+  }
   if (pass_blocks(2, n, batch) > 3ll * sms) return 2;
   int best = 1;
   double cost = 0;

@@ -37,3 +37,15 @@ def test_large_batches_of_passes_take_the_largest_tiles(rules):
         assert rules.pass_cfg(n, 4, batch, SMS) == 2, (n, batch)
     for n, nu, batch, want in ((128, 4, 1, 0), (128, 2, 1, 1), (192, 4, 1, 1), (256, 4, 1, 1), (128, 4, 16, 2), (96, 4, 8, 1)):
         assert rules.pass_cfg(n, nu, batch, SMS) == want, (n, nu, batch)
+
+
+def test_two_sweep_tiles_where_whole_passes_lose(rules):
+    for n in (448, 512, 557):  # the 37-node tiles take a second wave, the 62-node ones idle two fifths of the SMs
+        assert rules.pass_cfg(n, 4, 1, SMS) == 3 and rules.pass_cfg(n, 8, 1, SMS) == 3, n
+        assert rules.pass_cfg(n, 4, 8, SMS) == 2, n
+    for n in (416, 443, 576, 704, 743):
+        assert rules.pass_cfg(n, 4, 1, SMS) in (1, 2), n
+    for n in (744, 1024, 2048, 16384):
+        assert rules.pass_cfg(n, 4, 1, SMS) == rules.pass_cfg(n, 4, 2, SMS) == 4, n
+    for n in (448, 512, 1024, 2048):  # an odd number of two-sweep launches would not end in its own array
+        assert rules.pass_cfg(n, 2, 1, SMS) in (1, 2) and rules.pass_cfg(n, 6, 1, SMS) in (1, 2), n
