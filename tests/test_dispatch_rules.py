@@ -49,3 +49,10 @@ def test_two_sweep_tiles_where_whole_passes_lose(rules):
         assert rules.pass_cfg(n, 4, 1, SMS) == rules.pass_cfg(n, 4, 2, SMS) == 4, n
     for n in (448, 512, 1024, 2048):  # an odd number of two-sweep launches would not end in its own array
         assert rules.pass_cfg(n, 2, 1, SMS) in (1, 2) and rules.pass_cfg(n, 6, 1, SMS) in (1, 2), n
+
+
+def test_non_blocking_solves_take_no_four_sweep_tiles(rules):
+    for n in range(16, 200, 2):
+        own, shared = rules.pass_cfg(n, 4, 1, SMS), rules.pass_cfg_shared(n, 4, 1, SMS)
+        assert shared != 0 and (own == 0 or shared == own), n
+    assert rules.pass_cfg(128, 4, 1, SMS) == 0 and rules.pass_cfg_shared(128, 4, 1, SMS) == 1
