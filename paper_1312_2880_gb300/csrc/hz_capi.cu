@@ -1145,6 +1145,7 @@ void plan_tail(hz_problem* P) {
     A.pf = P->lv[lt].pitch;
     A.u_out = final_u(P, lt);
     A.po = P->lv[lt].pitch;
+    A.clusters = fp32 ? 0 : tail_max_clusters(A, smem);
     P->tail = A;
     P->tail_smem = smem;
     P->tail_start = lt;

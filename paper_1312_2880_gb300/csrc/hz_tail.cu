@@ -278,36 +278,63 @@ size_t tail_layout(bool fp32, TailArgs* A) {
   return off;
 }
 
+namespace {
+
+template <class K>
+cudaError_t tail_opt_in(K kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TAIL_MAX_SMEM);
+}
+cudaError_t cluster_opt_in() {
+  static OncePerDevice ready;
+  return ready([] { return tail_opt_in(tail_cluster_kernel); });
+}
+cudaLaunchConfig_t cluster_config(int count, size_t smem, cudaLaunchAttribute (&attr)[2], cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(TAIL_CLUSTER, 1, count);
+  cfg.blockDim = dim3(TAIL_THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = TAIL_CLUSTER;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cfg;
+}
+
+}  // namespace
+
+int tail_max_clusters(const TailArgs& A, size_t smem) {
+  const int m = (A.lv[A.count - 1].n + 1) * (A.lv[A.count - 1].n + 1);
+  if (!A.off_ainv || m < 25 || !coarse_share_fits(m) || cluster_opt_in() != cudaSuccess) return 0;
+  cudaLaunchAttribute attr[2];
+  cudaLaunchConfig_t cfg = cluster_config(1, smem, attr, nullptr);
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, tail_cluster_kernel, &cfg) != cudaSuccess) n = 0;
+  cudaGetLastError();  // a refused shape leaves no sticky error
+  return n;
+}
+
 cudaError_t launch_tail(bool fp32, const TailArgs& A, size_t smem, const int* stop, cudaStream_t s, const Inst& bi) {
   if (A.count < 2 || A.count > TAIL_MAX_LEVELS || smem > (size_t)TAIL_MAX_SMEM) return cudaErrorInvalidValue;
-  static OncePerDevice ready[3];
-  auto opt_in = [](auto kernel) {
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TAIL_MAX_SMEM);
-  };
+  static OncePerDevice ready[2];
   cudaError_t e;
-  const int m = (A.lv[A.count - 1].n + 1) * (A.lv[A.count - 1].n + 1);
-  // A cluster while its blocks are one wave (a block of the tail takes an SM) and there is something to
-  // share: tails of n_l = 8, 4 (m = 25) 23.2 us in one block, 19.1 with helpers, 10, 5 (m = 36) 25.2 and
-  // 20.1, 14, 7 (m = 64) 31.4 and 21.9. A batch of more instances fills the SMs with its own tails.
-  if (!fp32 && A.off_ainv && m >= 25 && coarse_share_fits(m) && TAIL_CLUSTER * bi.count <= device_sms()) {
-    if ((e = ready[2]([&] { return opt_in(tail_cluster_kernel); }))) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(TAIL_CLUSTER, 1, bi.count);
-    cfg.blockDim = dim3(TAIL_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
+  // A cluster per instance while the device holds them all at once (a block of the tail takes an SM, and a
+  // cluster's eight lie in one GPC: 15 on 152 SMs) and there is something to share: tails of n_l = 8, 4 (m = 25)
+  // 23.2 us in one block, 19.1 with helpers, 10, 5 (m = 36) 25.2 and 20.1, 14, 7 (m = 64) 31.4 and 21.9. A
+  // second wave of clusters loses: whole solves (n = 32, six iterations) with and without them 1.69 and 1.72 ms
+  // for 15 right-hand sides, 2.20 and 1.79 ms for 16.
+  if (!fp32 && bi.count <= A.clusters) {
+    if ((e = cluster_opt_in())) return e;
     cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = TAIL_CLUSTER;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
+    const cudaLaunchConfig_t cfg = cluster_config(bi.count, smem, attr, s);
     return cudaLaunchKernelEx(&cfg, tail_cluster_kernel, A, stop, bi);
   }
-  if ((e = ready[fp32]([&] { return fp32 ? opt_in(tail_kernel32) : opt_in(tail_kernel64); }))) return e;
+  if ((e = ready[fp32]([&] { return fp32 ? tail_opt_in(tail_kernel32) : tail_opt_in(tail_kernel64); }))) return e;
   dim3 grid(1, 1, bi.count);
   if (fp32)
     pdl_launch(tail_kernel32, grid, TAIL_THREADS, smem, s, A, stop, bi);
