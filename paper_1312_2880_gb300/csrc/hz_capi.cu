@@ -1102,20 +1102,26 @@ bool opts_ok(const hz_hierarchy_opts& o) {
 
 // ------------------------------------------------------------------ coarse tail
 // The largest tail that fits TAIL_MAX_SMEM: levels lt .. L-1 (lt >= 1), each a one-sweep
-// Gauss-Seidel level or a Kaczmarz level, the last the coarsest. Only where one block is the faster
-// way: its FP64 pipe makes every level above 16 intervals slower than launches over several SMs (FP64
-// iteration at n = 64 193 us with levels 32 .. 8 in the tail, 158 without one; n = 512 1104 and 1015;
-// n = 240 848 and 812), and so is a coarsest solve of many unknowns (FP32 iteration at n = 864, 784
-// unknowns: 488 us with the tail, 363 with coarse_solve_kernel over 49 blocks; at 256 unknowns 212 both ways).
-constexpr int TAIL_MAX_N64 = 16, TAIL_MAX_COARSE32 = 256, TAIL_MAX_COARSE64 = 100;
+// Gauss-Seidel level or a Kaczmarz level, the last the coarsest. Only where one block is the faster way
+// (rules::tail_max_n64, tail_max_coarse), measured against the default forms: a level that the options give
+// another form (colour or cooperative launches, one block, streaming passes) is in the tail wherever it fits and
+// one block's coarsest solve (m = 256 in FP64 114 us) costs less than that level's launches (a pass of 20
+// colours 200 us).
+bool spread_form(const hz_problem* P, int l) {
+  if (fused(P, l)) return P->opts.pass_variant <= 0;
+  return P->lv[l].kform == HZ_KACZ_CLUSTER || P->lv[l].kform == HZ_KACZ_TILE;
+}
 void plan_tail(hz_problem* P) {
   P->tail_start = -1;
   const int L = P->plan.levels;
   if (!P->opts.coarse_tail || L < 3) return;
   const bool fp32 = P->plan.fp32;
-  if (P->plan.m_coarse > (fp32 ? TAIL_MAX_COARSE32 : TAIL_MAX_COARSE64)) return;
+  const int max_n = fp32 ? 1 << 30 : rules::tail_max_n64(P->plan.batch, P->num_sms);
+  const int max_m = rules::tail_max_coarse(fp32, P->plan.batch, P->num_sms);
   for (int lt = 1; lt <= L - 2; ++lt) {
-    if (L - lt > TAIL_MAX_LEVELS || (!fp32 && P->lv[lt].n > TAIL_MAX_N64)) continue;
+    if (L - lt > TAIL_MAX_LEVELS) continue;
+    const bool spread = spread_form(P, lt);
+    if (spread ? P->lv[lt].n > max_n || P->plan.m_coarse > max_m : P->plan.m_coarse > std::max(max_m, 256)) continue;
     bool ok = true;
     TailArgs A{};
     A.count = L - lt;
