@@ -14,6 +14,7 @@
 #include "hz_common.cuh"
 #include "hz_host.h"
 #include "hz_internal.h"
+#include "hz_rules.h"
 
 namespace hz {
 
@@ -210,11 +211,10 @@ __device__ __forceinline__ double2 nb_sum(float2 a, float2 b, float2 c, float2 d
   o.y = join(sv.y, rv.y, odd);
   return o;
 }
-// Neighbour sum (W + E) + (S + N) of FP64 values, MIX of its six additions on the integer pipe. On grids
-// that fill the GPU four are the best split (operator alone at n = 1984: 91, 78, 64, 82 us with 0, 2, 4,
-// 6); a grid of a few nodes per thread is bound by latency and takes none.
+// Neighbour sum (W + E) + (S + N) of FP64 values, MIX of its six additions on the integer pipe. In launches
+// that fill the GPU (rules::operator_fills_gpu) four are the best split (operator alone at n = 1984: 91, 78,
+// 64, 82 us with 0, 2, 4, 6).
 constexpr int MIX_LARGE = 4;
-constexpr int MIX_MIN_N = 512;
 template <int MIX>
 __device__ __forceinline__ double2 nb_sum64(double2 w, double2 e, double2 s, double2 n) {
   return xr::nb4_mix<MIX>(w, e, s, n);
@@ -802,7 +802,7 @@ template <class Y2>
 cudaError_t apply_rv(const KrylovVecs& k, const Y2* y, cudaStream_t s) {
   if (sizeof(Y2) == 8 && k.G > 4 * device_sms())
     pdl_launch(k_apply_rv_kernel<float2, 2, 0>, dim3((k.G + 1) / 2, 1, k.batch), KB, 0, s, k, (const float2*)y);
-  else if (sizeof(Y2) == 16 && k.n >= MIX_MIN_N)
+  else if (sizeof(Y2) == 16 && rules::operator_fills_gpu(k.N, k.batch))
     pdl_launch(k_apply_rv_kernel<double2, 1, MIX_LARGE>, KGRID, KB, 0, s, k, (const double2*)y);
   else
     pdl_launch(k_apply_rv_kernel<Y2, 1, 0>, KGRID, KB, 0, s, k, y);
@@ -812,7 +812,7 @@ template <class Y2>
 cudaError_t apply_ts(const KrylovVecs& k, const Y2* z, cudaStream_t s) {
   if (sizeof(Y2) == 8 && k.G > 4 * device_sms())
     pdl_launch(k_apply_ts_kernel<float2, 2, 0>, dim3((k.G + 1) / 2, 1, k.batch), KB, 0, s, k, (const float2*)z);
-  else if (sizeof(Y2) == 16 && k.n >= MIX_MIN_N)
+  else if (sizeof(Y2) == 16 && rules::operator_fills_gpu(k.N, k.batch))
     pdl_launch(k_apply_ts_kernel<double2, 1, MIX_LARGE>, KGRID, KB, 0, s, k, (const double2*)z);
   else
     pdl_launch(k_apply_ts_kernel<Y2, 1, 0>, KGRID, KB, 0, s, k, z);
@@ -838,7 +838,7 @@ cudaError_t launch_k_update_x(const KrylovVecs& k, bool omega_half, cudaStream_t
   return cudaGetLastError();
 }
 cudaError_t launch_k_true_residual(const KrylovVecs& k, cudaStream_t s) {
-  if (k.n >= MIX_MIN_N) pdl_launch(k_true_residual_kernel<MIX_LARGE>, KGRID, KB, 0, s, k);
+  if (rules::operator_fills_gpu(k.N, k.batch)) pdl_launch(k_true_residual_kernel<MIX_LARGE>, KGRID, KB, 0, s, k);
   else pdl_launch(k_true_residual_kernel<0>, KGRID, KB, 0, s, k);
   return cudaGetLastError();
 }
@@ -859,7 +859,7 @@ cudaError_t launch_apply_fp64(double2* v, const double2* u, const double* kh, co
   long long N = (long long)(n + 1) * (n + 1);
   int G = (int)((N + KB - 1) / KB);
   if (G > 4096) G = 4096;
-  if (n >= MIX_MIN_N) pdl_launch(apply_fp64_kernel<MIX_LARGE>, G, KB, 0, s, v, u, kh, d, n, beta, out_scale);
+  if (rules::operator_fills_gpu(N, 1)) pdl_launch(apply_fp64_kernel<MIX_LARGE>, G, KB, 0, s, v, u, kh, d, n, beta, out_scale);
   else pdl_launch(apply_fp64_kernel<0>, G, KB, 0, s, v, u, kh, d, n, beta, out_scale);
   return cudaGetLastError();
 }

@@ -80,5 +80,12 @@ inline int tail_max_n64(int batch, int sms) { return 4 * batch <= sms ? 16 : 3 *
 // and 7.8, 12.9, 46.0).
 inline int tail_max_coarse(bool fp32, int batch, int sms) { return fp32 ? 256 : 3 * batch > sms ? 1 << 30 : 100; }
 
+// Operator kernels of the FP64 form (hz_krylov.cu): part of the neighbour sums goes to the integer pipe where
+// the launch, all right-hand sides together, fills the GPU: from the nodes of one n = 512 grid on. Smaller
+// launches are bound by latency. Measured without and with it (v = A y, t = A z in us): n = 128, 16, 64
+// and 152 right-hand sides 23.6, 61.0, 128 -> 21.9, 54.3, 116 and 25.1, 63.2, 138 -> 23.5, 56.3, 126;
+// n = 400 17.4 -> 17.5 and 16.9 -> 17.0; n = 2000 alone 91 -> 64.
+inline bool operator_fills_gpu(long long nodes, int batch) { return nodes * batch >= 513ll * 513ll; }
+
 }  // namespace rules
 }  // namespace hz

@@ -56,3 +56,8 @@ def test_non_blocking_solves_take_no_four_sweep_tiles(rules):
         own, shared = rules.pass_cfg(n, 4, 1, SMS), rules.pass_cfg_shared(n, 4, 1, SMS)
         assert shared != 0 and (own == 0 or shared == own), n
     assert rules.pass_cfg(128, 4, 1, SMS) == 0 and rules.pass_cfg_shared(128, 4, 1, SMS) == 1
+
+
+def test_the_operator_rule_counts_all_right_hand_sides(rules):
+    for n, batch, want in ((512, 1, 1), (511, 1, 0), (128, 1, 0), (128, 15, 0), (128, 16, 1), (64, 64, 1), (16384, 1, 1)):
+        assert rules.fills_gpu(ctypes.c_longlong((n + 1) ** 2), batch) == want, (n, batch)
