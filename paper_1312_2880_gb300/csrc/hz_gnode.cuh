@@ -14,11 +14,15 @@ namespace gnode {
 // 1.92 ms with 0, 4, 6 of the six additions there, the restricted residual 117, 102, 98 us (with a
 // thread per coarse node).
 constexpr int MIX_GNODE = 6;
+// The grid-synchronised form (hz_kgrid.cu) has few warps per SM and pays for the longer chain on small levels:
+// per iteration n_l = 64 and 128 392 and 439 us with no addition there, 420 and 472 with six; V-cycles of
+// n = 1024 and 2048 (n_l = 512 and more) 1224 and 2686 us with none, 1117 and 2351 with six.
+constexpr int MIX_GRID_MIN_N = 512;
 
 // Row action on row (i, j) of A u = f~ (Sec. 4-5, Kaczmarz): delta = (f~_p - a_p u) / |a_p|^2,
 // u_q += conj(a_pq) delta over the row's support (lvl::act_nodes); a mirror neighbour at the
 // boundary carries coefficient 2 and receives 2 delta.
-template <class T, class F2>
+template <class T, class F2, int MIX = MIX_GNODE>
 __device__ __forceinline__ void kacz_row(c2<T>* __restrict__ u, int pu, const F2* __restrict__ f, int pf,
                                          const T* __restrict__ kh, int pk, int n, int i, int j, T beta,
                                          const double* __restrict__ stored = nullptr, int pi = 0) {
@@ -32,7 +36,7 @@ __device__ __forceinline__ void kacz_row(c2<T>* __restrict__ u, int pu, const F2
     lvl::row_consts<T>(kh[(long long)j * pk + i], i, j, n, beta, &d, &inv);
   }
   c2<T>* row = u + (long long)j * pu;
-  lvl::act_nodes<T, MIX_GNODE>(row + i, row + b.iw, row + b.ie, u + (long long)b.js * pu + i, u + (long long)b.jn * pu + i,
+  lvl::act_nodes<T, MIX>(row + i, row + b.iw, row + b.ie, u + (long long)b.js * pu + i, u + (long long)b.jn * pu + i,
                     ldc<T>(f, (long long)j * pf + i), d, inv);
 }
 

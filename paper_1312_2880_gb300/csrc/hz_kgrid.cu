@@ -88,16 +88,24 @@ __device__ bool band_step(BandSync bs, unsigned int base, unsigned int done, int
 }
 
 // One colour phase on the band's rows.
-template <class T, class F2>
-__device__ __forceinline__ void colour_phase(const Band& bd, c2<T>* u, int pu, const F2* f, int pf, const T* kh, int pk,
-                                             int n, int colour, T beta) {
+template <class T, class F2, int MIX>
+__device__ __forceinline__ void colour_rows(const Band& bd, c2<T>* u, int pu, const F2* f, int pf, const T* kh, int pk,
+                                            int n, int colour, T beta) {
   const int w5 = (n + 5) / 5;
   const int slots = (bd.j1 - bd.j0) * w5;
   for (int s = threadIdx.x; s < slots; s += GT) {
     const int r = s / w5, m = s - r * w5, j = bd.j0 + r;
     const int i = ((colour - 2 * j) % 5 + 5) % 5 + 5 * m;
-    if (i <= n) gnode::kacz_row<T, F2>(u, pu, f, pf, kh, pk, n, i, j, beta);
+    if (i <= n) gnode::kacz_row<T, F2, MIX>(u, pu, f, pf, kh, pk, n, i, j, beta);
   }
+}
+template <class T, class F2>
+__device__ __forceinline__ void colour_phase(const Band& bd, c2<T>* u, int pu, const F2* f, int pf, const T* kh, int pk,
+                                             int n, int colour, T beta) {
+  if (sizeof(T) == 8 && n >= gnode::MIX_GRID_MIN_N)
+    colour_rows<T, F2, gnode::MIX_GNODE>(bd, u, pu, f, pf, kh, pk, n, colour, beta);
+  else
+    colour_rows<T, F2, 0>(bd, u, pu, f, pf, kh, pk, n, colour, beta);
 }
 
 template <class T, class F2>
