@@ -317,6 +317,17 @@ __device__ __forceinline__ void prolong_smooth_body(O2* __restrict__ out, int po
   }
 }
 
+// The same for FP32 tiles at the boundary. Out of line: in line, the compiler's schedule of the FP32 interior path,
+// which nearly all tiles of a large grid take, was worse by a tenth (prolong_smooth at n = 2048 146 -> 163 us, V-cycles
+// of n = 2048 and 4096 in the tile form 311 -> 319 and 907 -> 941 us; out of line 305 and 895).
+template <class T, class F2, class O2, class S, int MIX>
+__device__ __noinline__ void prolong_smooth_edge(O2* __restrict__ out, int po, const c2<T>* __restrict__ upre, int pu,
+                                                 const c2<T>* __restrict__ ec, int pc, const F2* __restrict__ f, int pf,
+                                                 const T* __restrict__ kh, int pk, int n, T bA, const Inst& bi, c2<T>* su,
+                                                 c2<T>* sf, T* sk, int gx, int gy) {
+  prolong_smooth_body<T, F2, O2, S, MIX, xr::DIAG_ANY>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, bi, su, sf, sk, gx, gy);
+}
+
 template <class T, class F2, class S, int MIX>
 __global__ void __launch_bounds__(S::FT) smooth_restrict_kernel(c2<T>* __restrict__ u, int pu, c2<T>* __restrict__ fc,
                                                               int pc, const F2* __restrict__ f, int pf,
@@ -386,7 +397,10 @@ __global__ void __launch_bounds__(S::FT) prolong_smooth_kernel(O2* __restrict__ 
       return;
     }
   }
-  prolong_smooth_body<T, F2, O2, S, MIX, xr::DIAG_ANY>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, bi, su, sf, sk, gx, gy);
+  if constexpr (sizeof(T) == 4)
+    prolong_smooth_edge<T, F2, O2, S, MIX>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, bi, su, sf, sk, gx, gy);
+  else
+    prolong_smooth_body<T, F2, O2, S, MIX, xr::DIAG_ANY>(out, po, upre, pu, ec, pc, f, pf, kh, pk, n, bA, bi, su, sf, sk, gx, gy);
 }
 
 template <class T, class S>
