@@ -58,9 +58,7 @@ def kernel_bytes_per_node(kernel: str, fp32: bool) -> float:
         "gs_first": c / 2 + r / 2 + c,
         "gs_colour": (c + c + r + c) / 2,
         "kacz_colour": (5 * c * 2 + c + r) / 5,
-        # FP32: a whole pass a launch, the mean of pre (f, k h; u, coarse f) and post (u, coarse e, f, k h; u);
-        # FP64: one sweep a launch (u in, f, k h; u out)
-        "kacz_sweep": (5 * c + c / 2 + 2 * r) / 2 if fp32 else c + c + r + c,
+        "kacz_sweep": c + c + r + c,               # u in, f, k h; u out (FP32: kacz_launch_bytes)
         "restrict_residual": c + c + r + c / 4,
         "prolong_add": 2 * c + c / 4,
         "export": 2 * c,
@@ -72,6 +70,22 @@ def kernel_bytes_per_node(kernel: str, fp32: bool) -> float:
         "k_update_x": y + 32,                      # y or z; x in and out (one half of the update)
     }
     return table.get(kernel, 0.0)
+
+
+def kacz_launch_bytes(per, level: int, iterations: int = 2) -> float:
+    """FP32 tiles of a Kaczmarz level: mean bytes per node of one launch. A profiled iteration has two V-cycles of
+    two passes; the first launch of the pass down reads no u (zero guess). Where the level has no transfer launch of
+    its own, the last one down writes the coarse f and the first one up reads the coarse e."""
+    c, r = 8, 4
+    per_pass = len(per[("kacz_sweep", level)]) / (4 * iterations)
+    whole = ("restrict_residual", level) not in per
+    return (2 * per_pass * (3 * c + r) - c + (c / 2 if whole else 0)) / (2 * per_pass)
+
+
+def launch_bytes_per_node(per, kernel: str, level: int, fp32: bool) -> float:
+    if fp32 and kernel == "kacz_sweep":
+        return kacz_launch_bytes(per, level)
+    return kernel_bytes_per_node(kernel, fp32)
 
 
 # FP64 work per node of the Krylov kernels: (flops with an FMA counted 2, FP64-pipe instructions in the
@@ -268,7 +282,7 @@ def roofline(per, fp32: bool, hbm_peak: float, peak_kind: str, n: int, fp64_peak
     (name, level), times = max(per.items(), key=lambda kv: sum(kv[1]))
     avg_ms = sum(times) / len(times)
     nodes = ((n >> level) + 1) ** 2
-    gbs = kernel_bytes_per_node(name, fp32) * nodes / (avg_ms * 1e-3) / 1e9
+    gbs = launch_bytes_per_node(per, name, level, fp32) * nodes / (avg_ms * 1e-3) / 1e9
     if name.startswith("k_") and fp64_peak:
         flops, instr = KRYLOV_FP64[name][0], KRYLOV_FP64[name][1 if fp32 else 2]
         secs = avg_ms * 1e-3
@@ -285,7 +299,7 @@ def roofline(per, fp32: bool, hbm_peak: float, peak_kind: str, n: int, fp64_peak
     else:
         roof = {"kernel": name, "level": level, "bound": "hbm", "achieved": round(gbs, 1), "peak": hbm_peak,
                 "unit": "GB/s", "frac": round(gbs / hbm_peak, 4), "peak_source": peak_kind,
-                "bytes_per_node": kernel_bytes_per_node(name, fp32), "nodes": nodes}
+                "bytes_per_node": launch_bytes_per_node(per, name, level, fp32), "nodes": nodes}
     roof.update({"traffic": None, "avg_launch_ms": round(avg_ms, 5), "launches": len(times),
                  "share": round(sum(times) / total, 4)})
     return roof
@@ -302,7 +316,7 @@ def sweep_rates(per, fp32: bool, hbm_peak: float, n: int):
         if nl < 2048 and not name.startswith("kacz"):
             continue
         avg = sum(times) / len(times)
-        gbs = kernel_bytes_per_node(name, fp32) * (nl + 1) ** 2 / (avg * 1e-3) / 1e9
+        gbs = launch_bytes_per_node(per, name, level, fp32) * (nl + 1) ** 2 / (avg * 1e-3) / 1e9
         out[f"{name}@L{level}"] = {"n_l": nl, "gbs": round(gbs, 1), "frac": round(gbs / hbm_peak, 4),
                                    "ms": round(avg, 4), "launches_per_iteration": len(times) // 2}
     return out
