@@ -47,7 +47,7 @@ __device__ __forceinline__ void kacz_row(c2<T>* __restrict__ u, int pu, const F2
 // grid-synchronised form other blocks wrote u earlier in the same launch, and a const __restrict__
 // pointer lets the compiler read it through the non-coherent read-only path, which may return
 // lines cached before those writes.
-template <class T, class F2>
+template <class T, class F2, int MIX = MIX_GNODE>
 __device__ __forceinline__ c2<T> restrict_node(const c2<T>* u, int pu, const F2* __restrict__ f, int pf,
                                                const T* __restrict__ kh, int pk, int n, T beta, int I, int J) {
   c2<T> rows[3];
@@ -61,7 +61,7 @@ __device__ __forceinline__ c2<T> restrict_node(const c2<T>* u, int pu, const F2*
       const Nbr nb = neighbours(i, j, n);
       const c2<T>* row = u + (long long)j * pu;
       r[a] = xr::resid<T>(ldc<T>(f, (long long)j * pf + i), row[i],
-                          xr::nb4_mix<MIX_GNODE>(row[nb.iw], row[nb.ie], u[(long long)nb.js * pu + i], u[(long long)nb.jn * pu + i]),
+                          xr::nb4_mix<MIX>(row[nb.iw], row[nb.ie], u[(long long)nb.js * pu + i], u[(long long)nb.jn * pu + i]),
                           xr::diag<T>(kh[(long long)j * pk + i], lvl::sides_at(i, j, n), beta));
     }
     rows[b] = xr::fw3<T>(r[0], r[1], r[2]);

@@ -137,7 +137,9 @@ __global__ void __launch_bounds__(GT) kacz_grid_pre_kernel(c2<T>* __restrict__ u
   const int nc = n / 2, wc = nc + 1, J0 = (bd.j0 + 1) / 2, J1 = (bd.j1 + 1) / 2;
   for (int q = threadIdx.x; q < (J1 - J0) * wc; q += GT) {
     const int r = q / wc, I = q - r * wc, J = J0 + r;
-    fc[(long long)J * pc + I] = gnode::restrict_node<T, F2>(u, pu, f, pf, kh, pk, n, bB, I, J);
+    fc[(long long)J * pc + I] = sizeof(T) == 8 && n >= gnode::MIX_GRID_MIN_N
+                                    ? gnode::restrict_node<T, F2>(u, pu, f, pf, kh, pk, n, bB, I, J)
+                                    : gnode::restrict_node<T, F2, 0>(u, pu, f, pf, kh, pk, n, bB, I, J);
   }
 }
 
