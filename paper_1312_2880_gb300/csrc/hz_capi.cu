@@ -53,7 +53,6 @@ struct Level {
   int var_down = 0, var_up = 0;  // fused-pass variants (picked by the tile autotuner)
   int kform = 0;                 // hz_kacz_form of a Kaczmarz level (set up by plan_kaczmarz)
   int pass_cfg = 0;              // how its FP32 tiles run (rules::pass_config)
-  int pass_cfg_shared = 0;       // the same in non-blocking solves
   double omega = 1.0;            // relaxation factor of a Jacobi or SOR level
 };
 
@@ -432,7 +431,6 @@ void plan_kaczmarz(hz_problem* P) {
     const int want = P->opts.kacz_form;
     L.kform = (want >= 0 && kform_ok(P, l, want)) ? want : default_kform(P, l);
     L.pass_cfg = rules::pass_config(L.n, L.nu, P->plan.batch, P->num_sms);
-    L.pass_cfg_shared = rules::pass_config(L.n, L.nu, P->plan.batch, P->num_sms, true);
   }
 }
 
@@ -791,19 +789,12 @@ hz_status build_graph(hz_problem* P) {
   return HZ_OK;
 }
 
-// One Bi-CGSTAB iteration as a plain graph, replayed from the host (polled mode). Levels above the tail take
-// their form for non-blocking solves while it is captured (where a level's result lies depends on it).
+// One Bi-CGSTAB iteration as a plain graph, replayed from the host (polled mode).
 hz_status build_iter_graph(hz_problem* P) {
   if (P->graph_iter) return HZ_OK;
   cudaGraph_t g = nullptr;
-  const int above = P->tail_start > 0 ? P->tail_start : P->plan.levels - 1;
-  auto swap_forms = [&] {
-    for (int l = 0; l < above; ++l) std::swap(P->lv[l].pass_cfg, P->lv[l].pass_cfg_shared);
-  };
   CK(cudaStreamBeginCapture(P->stream, cudaStreamCaptureModeThreadLocal));
-  swap_forms();
   cudaError_t e = enqueue_iteration(P);
-  swap_forms();
   cudaError_t e2 = cudaStreamEndCapture(P->stream, &g);
   if (e) return cuda_fail(P, e, "capture of one Bi-CGSTAB iteration");
   if (e2) return cuda_fail(P, e2, "cudaStreamEndCapture");

@@ -42,11 +42,7 @@ inline long long pass_blocks(int cfg, int n, int batch) {
   const long long t = (n + PASS_EDGE[cfg]) / PASS_EDGE[cfg];
   return t * t * batch;
 }
-// shared: of a non-blocking solve, which others run beside. It takes no four-sweep tiles: at n_l = 128 they are
-// 100 blocks with five times the level's row actions, and hold the SMs from the other solves (ten iterations of
-// 8 and 16 concurrent n = 256 problems 10.1 and 20.6 ms, 8.6 and 17.8 ms without them; 10.1 and 20.1 ms with
-// the clusters before there were whole passes; one alone 2.57 and 2.64 ms, 2.91 then).
-inline int pass_config(int n, int nu, int batch, int sms, bool shared = false) {
+inline int pass_config(int n, int nu, int batch, int sms) {
   const double fixed[3] = {58, 32, 20}, wave[3] = {35, 72, 136};
   if (nu % 4 == 0) {  // the two-sweep launches end in the array they start from
     if (pass_blocks(2, n, 1) > sms) return 4;
@@ -55,7 +51,7 @@ inline int pass_config(int n, int nu, int batch, int sms, bool shared = false) {
   if (pass_blocks(2, n, batch) > 3ll * sms) return 2;
   int best = 1;
   double cost = 0;
-  for (int q = nu % 4 == 0 && !shared ? 0 : 1; q < 3; ++q) {
+  for (int q = nu % 4 == 0 ? 0 : 1; q < 3; ++q) {
     const double c = fixed[q] + wave[q] * (double)((pass_blocks(q, n, batch) + sms - 1) / sms);
     if (cost == 0 || c < cost) {
       best = q;

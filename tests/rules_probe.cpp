@@ -10,5 +10,4 @@ extern "C" int same_shape(int n, int n2, int batch, int batch2) {
   return tune_key(n, batch, false, false, true, 0, 0) == tune_key(n2, batch2, false, false, true, 0, 0);
 }
 extern "C" int pass_cfg(int n, int nu, int batch, int sms) { return pass_config(n, nu, batch, sms); }
-extern "C" int pass_cfg_shared(int n, int nu, int batch, int sms) { return pass_config(n, nu, batch, sms, true); }
 extern "C" int fills_gpu(long long nodes, int batch) { return operator_fills_gpu(nodes, batch); }

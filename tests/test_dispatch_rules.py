@@ -51,13 +51,6 @@ def test_two_sweep_tiles_where_whole_passes_lose(rules):
         assert rules.pass_cfg(n, 2, 1, SMS) in (1, 2) and rules.pass_cfg(n, 6, 1, SMS) in (1, 2), n
 
 
-def test_non_blocking_solves_take_no_four_sweep_tiles(rules):
-    for n in range(16, 200, 2):
-        own, shared = rules.pass_cfg(n, 4, 1, SMS), rules.pass_cfg_shared(n, 4, 1, SMS)
-        assert shared != 0 and (own == 0 or shared == own), n
-    assert rules.pass_cfg(128, 4, 1, SMS) == 0 and rules.pass_cfg_shared(128, 4, 1, SMS) == 1
-
-
 def test_the_operator_rule_counts_all_right_hand_sides(rules):
     for n, batch, want in ((512, 1, 1), (511, 1, 0), (128, 1, 0), (128, 15, 0), (128, 16, 1), (64, 64, 1), (16384, 1, 1)):
         assert rules.fills_gpu(ctypes.c_longlong((n + 1) ** 2), batch) == want, (n, batch)
