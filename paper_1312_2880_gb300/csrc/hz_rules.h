@@ -33,8 +33,8 @@ inline TuneKey tune_key(int n, int batch, bool up, bool finest, bool fp32, doubl
 // level is n_l, in us, whole passes (37 or 62), 32 and 64: n_l = 416 131, 149, 152; 448 153, 149, 154; 512
 // 165, 159, 166; 576 178, 194, 181; 704 210, 238, 208; 768 256, 248, 251; 896 291, 307, 280; 1024 324, 362,
 // 309; 1536 604, 692, 578; 2048 993, 1139, 929. So 64 from where the 62-node tiles take a second wave, and
-// 32 where they leave more than two fifths of the SMs idle and the 37-node tiles already take a second
-// wave. Batches keep whole passes below that size: 16 right-hand sides on n_l = 256 and 512 (six iterations)
+// 32 where the 37-node tiles take one and at most two of the 32-node tiles come on an SM (n_l = 544, more
+// than two, 177 and 186). Batches keep whole passes below that size: 16 right-hand sides on n_l = 256 and 512 (six iterations)
 // 6.55, 7.53, 6.98 and 21.0, 24.1, 21.6 ms.
 constexpr int PASS_EDGE[3] = {13, 37, 62};
 inline int tile_edge(int cfg) { return cfg == 3 ? 32 : cfg == 4 ? 64 : 0; }
@@ -46,7 +46,8 @@ inline int pass_config(int n, int nu, int batch, int sms) {
   const double fixed[3] = {58, 32, 20}, wave[3] = {35, 72, 136};
   if (nu % 4 == 0) {  // the two-sweep launches end in the array they start from
     if (pass_blocks(2, n, 1) > sms) return 4;
-    if (batch == 1 && pass_blocks(1, n, 1) > sms && 5 * pass_blocks(2, n, 1) < 3ll * sms) return 3;
+    const long long t = (n + 32) / 32;
+    if (batch == 1 && pass_blocks(1, n, 1) > sms && t * t <= 2ll * sms) return 3;
   }
   if (pass_blocks(2, n, batch) > 3ll * sms) return 2;
   int best = 1;

@@ -40,10 +40,10 @@ def test_large_batches_of_passes_take_the_largest_tiles(rules):
 
 
 def test_two_sweep_tiles_where_whole_passes_lose(rules):
-    for n in (448, 512, 557):  # the 37-node tiles take a second wave, the 62-node ones idle two fifths of the SMs
+    for n in (448, 512, 543):  # the 37-node tiles take a second wave, two 32-node tiles come on an SM
         assert rules.pass_cfg(n, 4, 1, SMS) == 3 and rules.pass_cfg(n, 8, 1, SMS) == 3, n
         assert rules.pass_cfg(n, 4, 8, SMS) == 2, n
-    for n in (416, 443, 576, 704, 743):
+    for n in (416, 443, 544, 576, 704, 743):
         assert rules.pass_cfg(n, 4, 1, SMS) in (1, 2), n
     for n in (744, 1024, 2048, 16384):
         assert rules.pass_cfg(n, 4, 1, SMS) == rules.pass_cfg(n, 4, 2, SMS) == 4, n

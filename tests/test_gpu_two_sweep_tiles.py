@@ -8,9 +8,9 @@ pytestmark = pytest.mark.gpu
 from paper_1312_2880_gb300 import hz, inputs as I  # noqa: E402
 
 
-# n_l = n / 2: 448 and 544 (tiles of 32, a remainder of one node), 768 and 832 (tiles of 64, one node) and 800
+# n_l = n / 2: 448 and 512 (tiles of 32, a remainder of one node), 768 and 832 (tiles of 64, one node) and 800
 # (half a tile); two or four launches a pass, right-hand sides side by side.
-@pytest.mark.parametrize("n,batch,nu", [(896, 1, 4), (896, 1, 8), (1088, 1, 4), (1536, 1, 4), (1600, 1, 8), (1664, 2, 4)])
+@pytest.mark.parametrize("n,batch,nu", [(896, 1, 4), (896, 1, 8), (1024, 1, 4), (1536, 1, 4), (1600, 1, 8), (1664, 2, 4)])
 def test_tiles_give_the_bits_of_colour_launches(n, batch, nu):
     kf = I.wedge_k(n, 0.625 * n, 11)
     rng = np.random.default_rng(n)
