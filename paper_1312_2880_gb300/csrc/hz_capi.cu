@@ -201,6 +201,7 @@ struct hz_problem {
   int tail_start = -1;  // first level run by the one-block coarse tail (-1: none)
   TailArgs tail{};
   size_t tail_smem = 0;
+  int tail_clusters = 0;  // FP64: tails with helper blocks that the device holds at once
   std::string err;
   // Solve in flight (see solve_begin/solve_advance/solve_end).
   struct Run {
@@ -701,7 +702,7 @@ cudaError_t run_vcycle(hz_problem* P, const void* f0, void* z, const int* stop, 
   }
   if (lt > 0) {
     const Inst bi = inst_for(P, lt, all);
-    if ((e = mark(P, launch_tail(P->plan.fp32, P->tail, P->tail_smem, stop, P->stream, bi), HZ_K_TAIL, lt))) return e;
+    if ((e = mark(P, launch_tail(P->plan.fp32, P->tail, P->tail_smem, P->tail_clusters, stop, P->stream, bi), HZ_K_TAIL, lt))) return e;
   } else if ((e = coarse(P, stop, all))) {
     return e;
   }
@@ -1142,7 +1143,7 @@ void plan_tail(hz_problem* P) {
     A.pf = P->lv[lt].pitch;
     A.u_out = final_u(P, lt);
     A.po = P->lv[lt].pitch;
-    A.clusters = fp32 ? 0 : tail_max_clusters(A, smem);
+    P->tail_clusters = fp32 ? 0 : tail_max_clusters(A, smem);
     P->tail = A;
     P->tail_smem = smem;
     P->tail_start = lt;

@@ -159,7 +159,6 @@ struct TailLevel {
 };
 struct TailArgs {
   int count;  // levels in the tail, the last the coarsest
-  int clusters;  // FP64: tails with helper blocks that the device holds at once (tail_max_clusters)
   TailLevel lv[TAIL_MAX_LEVELS];
   unsigned off_r;    // residual scratch
   unsigned off_ainv; // coarsest inverse staged in shared memory when it fits (0: read from global)
@@ -173,7 +172,8 @@ struct TailArgs {
 size_t tail_layout(bool fp32, TailArgs* A);
 // FP64 tails that can run at once with their coarsest solve shared by a cluster (0: that form does not apply).
 int tail_max_clusters(const TailArgs& A, size_t smem);
-cudaError_t launch_tail(bool fp32, const TailArgs& A, size_t smem, const int* stop, cudaStream_t s,
+// clusters: tail_max_clusters in FP64.
+cudaError_t launch_tail(bool fp32, const TailArgs& A, size_t smem, int clusters, const int* stop, cudaStream_t s,
                         const Inst& bi = Inst());
 // dst (precision of fp32, pitch pd) = src (double2, pitch ps) * scale, on an (n+1)^2 grid.
 cudaError_t launch_import(bool fp32, void* dst, int pd, const double2* src, int ps, int n, double scale,

@@ -319,7 +319,8 @@ int tail_max_clusters(const TailArgs& A, size_t smem) {
   return n;
 }
 
-cudaError_t launch_tail(bool fp32, const TailArgs& A, size_t smem, const int* stop, cudaStream_t s, const Inst& bi) {
+cudaError_t launch_tail(bool fp32, const TailArgs& A, size_t smem, int clusters, const int* stop, cudaStream_t s,
+                        const Inst& bi) {
   if (A.count < 2 || A.count > TAIL_MAX_LEVELS || smem > (size_t)TAIL_MAX_SMEM) return cudaErrorInvalidValue;
   static OncePerDevice ready[2];
   cudaError_t e;
@@ -328,7 +329,7 @@ cudaError_t launch_tail(bool fp32, const TailArgs& A, size_t smem, const int* st
   // 23.2 us in one block, 19.1 with helpers, 10, 5 (m = 36) 25.2 and 20.1, 14, 7 (m = 64) 31.4 and 21.9. A
   // second wave of clusters loses: whole solves (n = 32, six iterations) with and without them 1.69 and 1.72 ms
   // for 15 right-hand sides, 2.20 and 1.79 ms for 16.
-  if (!fp32 && bi.count <= A.clusters) {
+  if (!fp32 && bi.count <= clusters) {
     if ((e = cluster_opt_in())) return e;
     cudaLaunchAttribute attr[2];
     const cudaLaunchConfig_t cfg = cluster_config(bi.count, smem, attr, s);
