@@ -67,15 +67,16 @@ inline int pass_config(int n, int nu, int batch, int sms) {
 // one; n = 512 1104 and 1015; n = 240 848 and 812) while a few instances leave the SMs idle. A batch gives
 // every SM a tail of its own and the launches no idle SMs: six iterations with the limit at 16 and at 32 (48),
 // n = 64 with a Kaczmarz level of 32, 24, 48, 64 and 152 right-hand sides 3.2, 4.5, 5.4, 10.1 and 4.0, 4.4, 4.7,
-// 6.8 ms; n = 96 with one of 24, 24, 48, 96 and 152 3.6, 5.3, 8.9, 12.9 and 3.7, 4.9, 7.2, 9.9 (4.2, 5.1, 7.2,
-// 9.5) ms.
-inline int tail_max_n64(int batch, int sms) { return 4 * batch <= sms ? 16 : 3 * batch <= 2 * sms ? 32 : 48; }
+// 6.8 ms; n = 96 with one of 24, 24, 48 and 152 3.6, 5.3, 12.9 and 3.7, 4.9, 9.9 ms; and with the limit at 32 and
+// 48, n = 72 with one of 36, 56, 64 and 100 4.86, 5.72, 7.72 and 5.04, 5.28, 6.22 ms, n = 88 with one of 44, 64, 80
+// and 100 6.63, 7.50, 8.91 and 6.67, 7.18, 7.81 ms.
+inline int tail_max_n64(int batch, int sms) { return 4 * batch <= sms ? 16 : 5 * batch <= 2 * sms ? 32 : 48; }
 // The most unknowns on the coarsest level: beyond, coarse_solve_kernel over several blocks is the faster way (FP32
-// iteration at n = 864, 784 unknowns: 488 us with the tail, 363 without; at 256 212 both ways), in FP64 batches
-// from a third of the SMs on the tail (n = 88, 120 and 240, coarsest 11 and 15: 40 right-hand sides 3.86, 5.22, 14.5
-// ms without and 3.67, 6.02, 15.2 with the tail, 64 5.43, 7.59, 22.0 and 4.62, 7.40, 21.9, 152 10.8, 16.1, 49.0
-// and 7.8, 12.9, 46.0).
-inline int tail_max_coarse(bool fp32, int batch, int sms) { return fp32 ? 256 : 3 * batch > sms ? 1 << 30 : 100; }
+// iteration at n = 864, 784 unknowns: 488 us with the tail, 363 without; at 256 212 both ways), but not beside a
+// tail on every SM: FP64, without and with the tail, n = 88, 120 and 240 (coarsest 11 and 15), 58 right-hand sides
+// 4.90, 6.90, 19.5 and 4.34, 7.06, 19.8 ms, 64 5.41, 7.58, 22.0 and 4.59, 7.39, 21.9, 152 10.8, 16.1, 49.0 and 7.8,
+// 12.9, 46.0; FP32 n = 136 and 368 (17 and 23), 64 2.66, 11.1 and 2.68, 11.0 ms, 152 5.35, 24.1 and 5.07, 23.4.
+inline int tail_max_coarse(bool fp32, int batch, int sms) { return 5 * batch > 2 * sms ? 1 << 30 : fp32 ? 256 : 100; }
 
 // Operator kernels of the FP64 form (hz_krylov.cu): part of the neighbour sums goes to the integer pipe where
 // the launch, all right-hand sides together, fills the GPU: from the nodes of one n = 512 grid on. Smaller
