@@ -402,7 +402,8 @@ bool kform_ok(const hz_problem* P, int l, int form) {
   }
   return false;
 }
-// Default form: FP32 - one block if the level fits, else tiles, else (odd sweep counts) a cluster; FP64
+// Default form: FP32 - one block if the level fits, else (rules::batch_takes_cluster) a cluster, else tiles, else
+// (odd sweep counts) a cluster; FP64
 // - a cluster (the FP64 pipe of one SM bounds the one-block form) up to CLUSTER_BEST64 or, in a batch,
 // as far as it fits (its rows are acted on once, a tile's halo again by its neighbours), else tiles up to
 // TILE_MAX64, else colour launches (the halo's FP64 work outweighs the saved launches on the largest
@@ -416,7 +417,8 @@ int default_kform(const hz_problem* P, int l) {
   constexpr int CLUSTER_BEST64 = 144, TILE_MAX64 = 768, TILE_MAX64_BATCH = 512;
   const bool one = P->plan.batch == 1;
   const int n = P->lv[l].n;
-  const int order32[] = {HZ_KACZ_LEVEL, HZ_KACZ_TILE, HZ_KACZ_CLUSTER};
+  const bool ragged = rules::batch_takes_cluster(n, P->plan.batch, P->num_sms);
+  const int order32[] = {HZ_KACZ_LEVEL, ragged ? HZ_KACZ_CLUSTER : HZ_KACZ_TILE, ragged ? HZ_KACZ_TILE : HZ_KACZ_CLUSTER};
   const int cluster_first[] = {HZ_KACZ_CLUSTER, HZ_KACZ_TILE}, tile_first[] = {HZ_KACZ_TILE, HZ_KACZ_CLUSTER};
   const int* o = P->plan.fp32 ? order32 : one && n > CLUSTER_BEST64 ? tile_first : cluster_first;
   const int cnt = P->plan.fp32 ? 3 : n <= (one ? TILE_MAX64 : TILE_MAX64_BATCH) ? 2 : 0;

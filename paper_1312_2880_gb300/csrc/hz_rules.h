@@ -62,6 +62,16 @@ inline int pass_config(int n, int nu, int batch, int sms) {
   return best;
 }
 
+// FP32 Kaczmarz levels of batches that take clusters before tiles: from two waves of the 62-node tiles on, levels
+// whose third tile each way lies mostly outside the square. Tiles and clusters, six iterations with 24, 64
+// and 152 right-hand sides: n_l = 120 3.51, 7.16, 14.9 and 3.61, 7.41, 15.5 ms; 128 4.21, 7.93, 16.8 and 3.84, 7.97,
+// 16.9; 136 4.70, 9.66, 20.6 and 4.30, 8.84, 18.7; 144 5.03, 10.2, 21.5 and 4.81, 9.72, 20.5; 160 5.47, 11.1, 23.8 and
+// 5.15, 11.1, 23.1; 168 5.69, 12.4, 27.2 and 5.35, 12.3, 26.9; 184 6.10, 13.5, 30.2 and 6.37, 14.2, 31.5. With 16
+// tiles are the faster way (128 3.04 and 3.16).
+inline bool batch_takes_cluster(int n, int batch, int sms) {
+  return batch > 1 && n >= 2 * PASS_EDGE[2] && n <= 2 * PASS_EDGE[2] + PASS_EDGE[1] && pass_blocks(2, n, batch) > sms;
+}
+
 // Coarse tail (hz_tail.cu): the levels that one block runs. In FP64 its pipe makes every level above 16 intervals
 // slower than launches over several SMs (iteration at n = 64 193 us with levels 32 .. 8 in the tail, 158 without
 // one; n = 512 1104 and 1015; n = 240 848 and 812) while a few instances leave the SMs idle. A batch gives

@@ -11,3 +11,4 @@ extern "C" int same_shape(int n, int n2, int batch, int batch2) {
 }
 extern "C" int pass_cfg(int n, int nu, int batch, int sms) { return pass_config(n, nu, batch, sms); }
 extern "C" int fills_gpu(long long nodes, int batch) { return operator_fills_gpu(nodes, batch); }
+extern "C" int ragged_batch(int n, int batch, int sms) { return batch_takes_cluster(n, batch, sms); }

@@ -54,3 +54,10 @@ def test_two_sweep_tiles_where_whole_passes_lose(rules):
 def test_the_operator_rule_counts_all_right_hand_sides(rules):
     for n, batch, want in ((512, 1, 1), (511, 1, 0), (128, 1, 0), (128, 15, 0), (128, 16, 1), (64, 64, 1), (16384, 1, 1)):
         assert rules.fills_gpu(ctypes.c_longlong((n + 1) ** 2), batch) == want, (n, batch)
+
+
+def test_batches_of_ragged_levels_take_clusters(rules):
+    """n_l = 124 .. 161, three 62-node tiles each way, from 17 right-hand sides (two waves of them) on."""
+    for n, batch, want in ((136, 17, 1), (136, 16, 0), (136, 1, 0), (124, 24, 1), (161, 24, 1), (123, 64, 0), (162, 64, 0),
+                           (256, 64, 0)):
+        assert rules.ragged_batch(n, batch, SMS) == want, (n, batch)
