@@ -5,7 +5,7 @@ random medium k (1 + 0.3 g) with g a seeded Gaussian random field of correlation
 a centre point source of 1/h^2, hybrid (HYB-V) hierarchy of 10 levels, Bi-CGSTAB to relres 1e-6.
 A step is one complete solve (every kernel of the hot path) with the inputs resident in HBM; the
 library rewrites every Krylov vector from the right-hand side, so no state carries over between
-solves. The problem's arrays (3.6 GB) are far larger than L2 (129 MB); L2 is also flushed (a 512 MB
+solves. The problem's arrays (3.2 GB) are far larger than L2 (129 MB); L2 is also flushed (a 512 MB
 write, untimed) before each timed solve.
 
 Beside the headline: the FP64 form of the same solve, the solve through host buffers (``e2e``),
@@ -73,9 +73,10 @@ def kernel_bytes_per_node(kernel: str, fp32: bool) -> float:
 
 
 def kacz_launch_bytes(per, level: int, iterations: int = 2) -> float:
-    """FP32 tiles of a Kaczmarz level: mean bytes per node of one launch. A profiled iteration has two V-cycles of
-    two passes; the first launch of the pass down reads no u (zero guess). Where the level has no transfer launch of
-    its own, the last one down writes the coarse f and the first one up reads the coarse e."""
+    """FP32 tiles of a Kaczmarz level: mean bytes per node of one record of the profile. A profiled iteration has two
+    V-cycles of two passes, in records of one whole pass (however many launches it takes) or of one two-sweep launch;
+    the first record of the pass down reads no u (zero guess). Where the level has no transfer launch of its own, the
+    last record down writes the coarse f and the first one up reads the coarse e."""
     c, r = 8, 4
     per_pass = len(per[("kacz_sweep", level)]) / (4 * iterations)
     whole = ("restrict_residual", level) not in per
@@ -675,7 +676,7 @@ def headline_line(args, wl, results, replica, e2e_ms, roof, per32, per64, hbm_pe
         "data": "synthetic",
         "config": {"workload": wl.name, "n": wl.n, "k": wl.k_ref, "medium": wl.meta.get("medium", ""),
                    "levels": wl.levels, "variant": wl.variant, "tol": wl.tol, "rhs": wl.meta.get("rhs", ""),
-                   "l2": "inputs (3.6 GB of arrays) larger than L2, and L2 flushed before every timed solve (512 MB write)",
+                   "l2": "inputs (3.2 GB of arrays) larger than L2, and L2 flushed before every timed solve (512 MB write)",
                    "parallelism": replica["parallelism"]},
         "iterations": r32["iterations"],
         "relres_true": r32["relres_true"],

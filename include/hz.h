@@ -64,7 +64,8 @@ typedef enum { HZ_SMOOTH_GS = 0, HZ_SMOOTH_KACZMARZ = 1, HZ_SMOOTH_DIRECT = 2, H
 
 /* Kernel forms of a Kaczmarz level (Sec. 4): one launch per colour; the whole level (sweeps,
    residual and full weighting, or correction and sweeps) in one block's shared memory; halo tiles
-   (FP32: one or two launches per pass, transfers included; FP64: one launch per sweep); the whole level in the shared memory of a thread-block cluster of up
+   (FP32: two or four sweeps per launch, on most levels with the pass's transfers in the same launches;
+   FP64: one launch per sweep); the whole level in the shared memory of a thread-block cluster of up
    to 16 blocks (row bands, neighbour rows through distributed shared memory); the whole level in
    global memory by one persistent cooperative launch per pass, with bounded grid-wide barriers
    between the colour phases (single right-hand side only; a barrier wait that runs out ends the
@@ -92,12 +93,14 @@ typedef struct {
                        per warp. Every form gives the same bits. */
   int coarse_tail;  /* 1 (default): the smallest levels, from the first whose whole V-cycle below it
                        fits one block's shared memory (FP32: with at most 256 unknowns on the coarsest
-                       level; FP64: from n_l = 16 down) to the coarsest, run as one launch (same
-                       operations, same results as the per-level kernels for one-sweep Gauss-Seidel
+                       level; FP64: from n_l = 16 down with at most 100; larger ones in batches that
+                       fill a quarter of the SMs or more, and for FP64 levels whose form is not the
+                       default one) to the coarsest, run as one launch (same operations, same results as the per-level kernels for one-sweep Gauss-Seidel
                        and Kaczmarz levels); 0: one or more launches per level */
   int kacz_form;    /* how Kaczmarz levels below the finest run (hz_kacz_form): -1 (default) = one
                        block if the level fits its shared memory, else tiles (even sweep counts), else a
-                       thread-block cluster, else colour launches in the FP32 form; in the FP64 form a
+                       thread-block cluster (n_l = 124 .. 161 in larger batches: before tiles), else
+                       colour launches in the FP32 form; in the FP64 form a
                        cluster up to n_l = 144 (in a batch: as far as the level fits), else tiles up to
                        n_l = 768 (in a batch: 512), else colour launches. A form that does not apply
                        to a level falls back to that default. */
@@ -280,7 +283,7 @@ typedef enum {
   HZ_K_SMOOTH_RESTRICT, /* fused: GS sweep from a zero guess, residual, full weighting */
   HZ_K_PROLONG_SMOOTH, /* fused: bilinear correction and GS post-sweep */
   HZ_K_KACZ_LEVEL,     /* whole Kaczmarz level in one block (pre: sweeps + residual + FW; post: correction + sweeps) */
-  HZ_K_KACZ_SWEEP,     /* Kaczmarz sweeps over halo tiles (FP32: a whole pass) */
+  HZ_K_KACZ_SWEEP,     /* Kaczmarz sweeps over halo tiles (FP32: a whole pass, or two sweeps per launch) */
   HZ_K_TAIL,           /* coarse tail: every level from hz_level_info.in_tail down, in one block */
   HZ_K_KACZ_CLUSTER,   /* whole Kaczmarz level over a thread-block cluster (pre or post, as HZ_K_KACZ_LEVEL) */
   HZ_K_JACOBI,         /* one damped Jacobi sweep, out of place */

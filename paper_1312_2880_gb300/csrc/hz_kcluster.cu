@@ -28,7 +28,6 @@ namespace hz {
 namespace {
 
 namespace cgx = cooperative_groups;
-// Threads per block: 256, or 1024 where a band has more than 256 blocks of five nodes.
 
 // The band of a block: rows r0 .. r1 - 1 (row j at local row j - r0 + 1 of su, the ghosts at 0 and
 // r1 - r0 + 1; at j - r0 of the other arrays). Every band but the last has `rows` >= 2 rows.
@@ -226,7 +225,8 @@ __global__ void __launch_bounds__(CT) cluster64_post_kernel(double2* __restrict_
 
 // Cluster shape of a level: the most blocks (16, 8, 4 or 2; 16 is beyond the portable cluster size)
 // whose bands fit CLUSTER_MAX_SMEM, have two rows and one thread (or pair) per block of five nodes,
-// and that the device can co-schedule, found once per device and n. c = 0: no cluster form.
+// and that the device can co-schedule, found once per device and n. c = 0: no cluster form. threads: 256 a
+// block, or 1024 where a band has more than 256 blocks of five nodes.
 struct Shape {
   int c = 0, rows = 0, split = 1, threads = 256;
   size_t smem = 0;

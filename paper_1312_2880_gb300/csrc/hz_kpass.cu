@@ -1,5 +1,6 @@
 // Whole pre- and post-relaxation passes of an FP32 Kaczmarz level (Sec. 4-5: 4 sweeps of Gauss-Seidel on
-// the normal equations each way), transfers included, in one or two launches of independent tiles.
+// the normal equations each way), transfers included, in launches of independent tiles with four or two
+// sweeps each (nu / 4 or nu / 2 launches a pass).
 //
 // Pre: zero guess, the sweeps (colours 0..4), residual with the (B) operator and full weighting onto the
 // coarse level. Post: u_pre + P e_c, the sweeps (colours 4..0). A tile holds a region with the

@@ -192,9 +192,11 @@ __device__ __forceinline__ double join(float s, float r, unsigned& odd) {
 // Sum of four FP32 complex values in FP64 without the FP64 pipe, which bounds the operator kernels:
 // error-free additions on the FP32 pipe leave a leading part and a remainder, joined in integers
 // (six FP64 additions, 460 cycles of a sub-partition's pipe per node, and eight widenings become
-// about 100 ordinary instructions). The result is the exact sum, which is what adding in FP64 gives
-// unless one of its additions rounds; `odd` is set where the remainder has more than 24 bits or join
-// cannot place it, and the caller then adds in FP64.
+// about 100 ordinary instructions). The result is the exact sum: what adding in FP64 gives, or, where one
+// of those additions would round, the more exact value. `odd` is set where the remainder has more than
+// 24 bits or join cannot place it, and the caller then adds in FP64. A warp with one such node issues both
+// ways, so the time depends on the data: k_apply_ts at n = 4096 0.34 ms in mid-solve, 0.44 ms in the first
+// iterations from a point source (nearly empty fields), 0.48 ms with FP64 additions alone.
 __device__ __forceinline__ double2 nb_sum(float2 a, float2 b, float2 c, float2 d, unsigned& odd) {
   f32x2 s1, r1, s2, r2, s, r3, r, r4, r5;
   two_sum(pack(a), pack(b), s1, r1);

@@ -372,7 +372,9 @@ __global__ void __launch_bounds__(256) ray_gemm_kernel(GemmJobs jobs, int Bs, in
 // cycles each, four warps per row with a tree apiece spent a third of a step's FP64 time there, and
 // 128 threads on 520 columns left one warp twice the work of the others). A solve at n = 512 took
 // 2.23 ms with the one-sided elimination and four warps per row, 1.86 ms now; at n = 256 0.71 and
-// 0.50 ms; the factorisation 1.21 s and 0.77 s.
+// 0.50 ms; the factorisation 1.21 s and 0.77 s. GEMV_PRE covers rows of 544 elements (n = 512 with ray cells of
+// 8 h has 520) at 110 registers a thread; longer rows fetch the rest after the wait and gain less (n = 1024,
+// 1032 elements, 10.7 and 10.4 ms).
 constexpr int GEMV_WARPS = 4, GEMV_PRE = 17;
 struct GemvJob {
   double2* out;
