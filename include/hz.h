@@ -94,8 +94,8 @@ typedef struct {
   int coarse_tail;  /* 1 (default): the smallest levels, from the first whose whole V-cycle below it
                        fits one block's shared memory (FP32: with at most 256 unknowns on the coarsest
                        level; FP64: from n_l = 16 down with at most 100; larger ones in batches that
-                       fill a quarter of the SMs or more, and for FP64 levels whose form is not the
-                       default one) to the coarsest, run as one launch (same operations, same results as the per-level kernels for one-sweep Gauss-Seidel
+                       fill a quarter of the SMs or more, and for FP64 levels whose kacz_form is not
+                       the default one) to the coarsest, run as one launch (same operations, same results as the per-level kernels for one-sweep Gauss-Seidel
                        and Kaczmarz levels); 0: one or more launches per level */
   int kacz_form;    /* how Kaczmarz levels below the finest run (hz_kacz_form): -1 (default) = one
                        block if the level fits its shared memory, else tiles (even sweep counts), else a

@@ -1097,13 +1097,11 @@ bool opts_ok(const hz_hierarchy_opts& o) {
 // ------------------------------------------------------------------ coarse tail
 // The largest tail that fits TAIL_MAX_SMEM: levels lt .. L-1 (lt >= 1), each a one-sweep
 // Gauss-Seidel level or a Kaczmarz level, the last the coarsest. Only where one block is the faster way
-// (rules::tail_max_n64, tail_max_coarse), measured against the default forms: a level that the options give
-// another form (colour or cooperative launches, one block, streaming passes) is in the tail wherever it fits and
-// one block's coarsest solve (m = 256 in FP64 114 us) costs less than that level's launches (a pass of 20
-// colours 200 us).
+// (rules::tail_max_n64, tail_max_coarse), measured against the default forms: a Kaczmarz level that the options
+// give another form (colour or cooperative launches, one block) is in the tail wherever it fits and one block's
+// coarsest solve (m = 256 in FP64 114 us) costs less than that level's launches (a pass of 20 colours 200 us).
 bool spread_form(const hz_problem* P, int l) {
-  if (fused(P, l)) return P->opts.pass_variant <= 0;
-  return P->lv[l].kform == HZ_KACZ_CLUSTER || P->lv[l].kform == HZ_KACZ_TILE;
+  return fused(P, l) || P->lv[l].kform == HZ_KACZ_CLUSTER || P->lv[l].kform == HZ_KACZ_TILE;
 }
 void plan_tail(hz_problem* P) {
   P->tail_start = -1;
